@@ -45,13 +45,19 @@ extern "C" int gks_gp_flux_host(const double* p, const double* ql, const double*
                                 const double* qr, const double* dqr, double dt, double* Fn,
                                 double* Ft) {
   const gks::FluxParams<double> P = params_from(p);
-  double a[3][5], b[3][5];
+  const double n[3] = {1.0, 0.0, 0.0};
+  double a[5][3], b[5][3], acc[10];
   for (int d = 0; d < 3; ++d)
     for (int v = 0; v < 5; ++v) {
-      a[d][v] = dql[5 * d + v];
-      b[d][v] = dqr[5 * d + v];
+      a[v][d] = dql[5 * d + v];
+      b[v][d] = dqr[5 * d + v];
     }
-  return gks::gks_gp_flux(P, ql, a, qr, b, dt, Fn, Ft) ? 0 : 1;
+  if (!gks::gp_flux_global(P, ql, a, qr, b, n, 1.0, dt, acc)) return 1;
+  for (int v = 0; v < 5; ++v) {
+    Fn[v] = acc[v];
+    Ft[v] = acc[5 + v];
+  }
+  return 0;
 }
 
 // Its vector-Jacobian product: cotangents (gFn, gFt) -> (gql, gdql[3][5], gqr, gdqr[3][5]).

@@ -634,16 +634,20 @@ __device__ __forceinline__ void first_order_if_nonphysical(const R* __restrict__
 
 // ------------------------------------------------------------------------------------------
 // Flux: four consecutive threads per face, one per Gauss point. Each evaluates both sides'
-// reconstructions, rotates into the local frame (n1 normal, n2 = n1 x e_k normalised with e_k
-// the axis least aligned with n1, n3 = n1 x n2), computes F^n and dF/dt, rotates back and
-// weights by the quadrature weight; the four are summed with shuffles and written once.
+// reconstructions and gradients, computes F^n and dF/dt in the global frame (gks_flux.cuh) and
+// weights them by the quadrature weight; the four are summed with shuffles and written once.
 // kFull selects the flux form and kTau0 a zero collision time at compile time, so that each
 // instance carries only the arithmetic (and registers) of its own form. The FP32 instances do
-// the two sides' work on packed f32x2 arithmetic (gp_flux_global2: the flux templates
-// instantiated with the pair type P2). Resident blocks per SM, measured: smooth form 6 (0.442 ms
-// per launch on the 64^3-cube mesh; 5 and 7 blocks 0.456 and 0.446; the scalar form at 7
-// blocks 0.477); full form 4 (6.53 ms per launch on the 128^3-cube explosion; 3 and 5 blocks
-// 6.99 and 7.44; the scalar form 7.06).
+// the two sides' work on packed f32x2 arithmetic (gp_flux_global2: side_terms instantiated with
+// the pair type P2). Bound by the FMA pipe (FP64: the FP64 pipe, 1/64 of the FP32 rate), so the
+// form with the fewest operations wins: against the flux in the face frame (values and
+// gradients rotated to the normal and two tangents, one moment derivative per axis), per
+// launch: FP32 smooth 0.418 -> 0.326 ms (64^3-cube mesh, 2.39 M faces), FP32 full 326 -> 231 us
+// (48^3-cube explosion, 1.02 M faces), FP64 smooth 2.53 -> 1.77 ms (32^3 cubes, 299 k faces),
+// FP64 full 2.05 -> 1.31 ms (124 k faces of tetrahedra). Resident blocks per SM, measured on
+// the same meshes: FP32 smooth 6 (0.326 ms; 4, 5, 7 and 8 blocks 0.380, 0.354, 0.333 and
+// 0.356); FP32 full 4 (231 us; 3 and 5 blocks 254 and 254); FP64 unbounded (2 blocks equal; 3
+// and 4 blocks 1 and 3 % slower).
 #ifndef GKS_FLUX_SMOOTH_MIN_BLOCKS
 #define GKS_FLUX_SMOOTH_MIN_BLOCKS 6  // resident 128-thread blocks per SM, FP32 smooth flux
 #endif
@@ -1451,8 +1455,10 @@ void launch_flux(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const 
                  const R* QA, double dt, R* fface, int* flag, cudaStream_t st) {
   const FluxParams<R> fp = flux_params(p);
   const unsigned nb = blocks_for(4 * m.nf, 128);
-  auto kern = fp.full ? (fp.tau_model == 0 ? k_flux<R, true, true> : k_flux<R, true, false>)
-                      : (fp.tau_model == 0 ? k_flux<R, false, true> : k_flux<R, false, false>);
+  // without a collision time the full form is the smooth one (its non-equilibrium terms carry
+  // the weight tau = 0)
+  auto kern = fp.tau_model == 0 ? k_flux<R, false, true>
+                                : (fp.full ? k_flux<R, true, false> : k_flux<R, false, false>);
   kern<<<nb, 128, 0, st>>>(m.nf, m.nc, m.f_owner, m.f_nb, m.f_wall, g.fgp, poly, QA,
                            p.gp_fallback, fp, wall_table<R>(m), (R)dt, fface, flag);
 }

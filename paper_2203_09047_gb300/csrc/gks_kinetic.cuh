@@ -514,190 +514,6 @@ GKS_HD void flux1_integrals(R tau, R d, R c[6]) {
   c[5] = -tau * tau * om;
 }
 
-// Interface-equilibrium terms of both flux forms from the interface state Q0 (primitives w0)
-// and its conserved-variable slopes dW_d along the local axes: the equilibrium time slope
-// rho0 <Ab psi>_0 = -sum_d rho0 <c_d ab_d psi>_0 = -sum_d A_d dW_d, the flux moments
-// E0 = rho0 <u psi>_0, E1 = rho0 <u (ab . c) psi>_0 = sum_d D T_d(W0)[dW_d] (only with a
-// collision-time model; zero otherwise, where tau = 0 multiplies it) and
-// E2 = rho0 <u Ab psi>_0 = A_x dWt, and the collision time from the two sides' pressures.
-template <class R>
-GKS_HD void interface_terms(const FluxParams<R>& P, R pl, R pr, const R q0[5], const Prim<R>& w0,
-                            const R dW[3][5], R dt, R dWt[5], R E0[5], R E1[5], R E2[5],
-                            R& tau) {
-  const R gm1 = P.gamma - R(1);
-  const R ir0 = w0.ir, Ep0 = q0[4] + w0.p;
-  R t[5];
-  euler_jvp(w0, ir0, gm1, Ep0, 0, dW[0], dWt);
-  euler_jvp(w0, ir0, gm1, Ep0, 1, dW[1], t);
-#pragma unroll
-  for (int q = 0; q < 5; ++q) dWt[q] += t[q];
-  euler_jvp(w0, ir0, gm1, Ep0, 2, dW[2], t);
-#pragma unroll
-  for (int q = 0; q < 5; ++q) dWt[q] = -(dWt[q] + t[q]);
-  euler_flux_x(w0, q0[4], E0);
-  euler_jvp(w0, ir0, gm1, Ep0, 0, dWt, E2);
-  const R dp = k_abs(k_div(pl - pr, pl + pr));
-  tau = collision_time(P, w0.p, ir0, dp, dt);
-  if (P.tau_model != 0) {
-    second_moment_jvp(w0, ir0, gm1, P.K, 0, dW[0], E1);
-#pragma unroll
-    for (int d = 1; d < 3; ++d) {
-      second_moment_jvp(w0, ir0, gm1, P.K, d, dW[d], t);
-#pragma unroll
-      for (int q = 0; q < 5; ++q) E1[q] += t[q];
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < 5; ++q) E1[q] = R(0);
-  }
-}
-
-// Smooth flux (Eq. flux-2) from the interface terms: F(delta) = E0 delta - tau delta (E1 + E2)
-// + delta^2/2 E2, so the two-point time fit is exact; with the heat-flux correction the energy
-// components gain pr_fix times the heat flux relative to the interface velocity, from the flux
-// moments F and the conserved moments m of the time-integrated distribution (m^n = Q0,
-// dm/dt = dWt; the tau terms of m vanish by the compatibility condition defining Ab).
-template <class R>
-GKS_HD void smooth_from_terms(const FluxParams<R>& P, const R q0[5], const Prim<R>& w0,
-                              const R dWt[5], const R E0[5], const R E1[5], const R E2[5], R tau,
-                              R Fn[5], R Ft[5]) {
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    Fn[q] = E0[q] - tau * (E1[q] + E2[q]);
-    Ft[q] = E2[q];
-  }
-  if (P.pr_fix != R(0)) {
-    const R u2 = w0.U * w0.U + w0.V * w0.V + w0.W * w0.W;
-    auto heat = [&](const R F[5], const R m[5]) {
-      return F[4] - (w0.U * F[1] + w0.V * F[2] + w0.W * F[3]) + R(0.5) * u2 * F[0] -
-             (w0.U * m[4] - w0.U * (w0.U * m[1] + w0.V * m[2] + w0.W * m[3]) +
-              R(0.5) * w0.U * u2 * m[0]);
-    };
-    const R qn = heat(Fn, q0);
-    const R qt = heat(Ft, dWt);
-    Fn[4] += P.pr_fix * qn;
-    Ft[4] += P.pr_fix * qt;
-  }
-}
-
-// Coefficients of the two-point time fit of the full flux: F^n and dF/dt are sums over the six
-// terms of Eq. flux-1 with weights cn and ct from the time integrals over [0, dt/2] and [0, dt]
-// (tau = 0: the equilibrium flux and its time derivative alone).
-template <class R>
-GKS_HD void full_fit_coeffs(R tau, R dt, R cn[6], R ct[6]) {
-  if (tau > R(0)) {
-    R ch[6], cf[6];
-    flux1_integrals(tau, R(0.5) * dt, ch);
-    flux1_integrals(tau, dt, cf);
-    const R idt = k_div(R(1), dt);
-#pragma unroll
-    for (int q = 0; q < 6; ++q) {
-      cn[q] = (R(4) * ch[q] - cf[q]) * idt;
-      ct[q] = R(4) * (cf[q] - R(2) * ch[q]) * idt * idt;
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < 6; ++q) cn[q] = ct[q] = R(0);
-    cn[0] = R(1);
-    ct[2] = R(1);
-  }
-}
-
-// Gauss-point flux in the local frame (u along the normal). ql/qr: conserved states;
-// dql/dqr[m]: their derivatives along n1, n2, n3 (momentum already in the local frame).
-// Writes Fn = F^n and Ft = dF/dt of the two-point time fit. Returns false for a non-physical
-// state.
-template <class R>
-GKS_HD bool gks_gp_flux(const FluxParams<R>& P, const R ql[5],
-                                            const R dql[3][5], const R qr[5], const R dqr[3][5],
-                                            R dt, R Fn[5], R Ft[5]) {
-  Prim<R> wl, wr, w0;
-  bool ok = to_prim(ql, P.gamma, wl) & to_prim(qr, P.gamma, wr);
-  if (!ok) return false;
-  const R gm1 = P.gamma - R(1);
-  Half<R> hl, hr;
-  half_init(wl, P.K, +1, hl);
-  half_init(wr, P.K, -1, hr);
-  // interface equilibrium Q0 from the two half-space moments
-  R q0[5], t[5];
-  half_moments(wl, hl, q0);
-  half_moments(wr, hr, t);
-#pragma unroll
-  for (int q = 0; q < 5; ++q) q0[q] += t[q];
-  if (!to_prim(q0, P.gamma, w0)) return false;
-  // conserved-variable slopes of the interface equilibrium, dW_d = rho0 <ab_d psi>_0: the
-  // half-space parts rho <a_d psi>_{u>0} + rho <a_d psi>_{u<0} of both sides' slopes
-  const R irl = wl.ir, irr = wr.ir;
-  R dW[3][5];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    half_jvp(wl, gm1, P.K, +1, hl, dql[d], dW[d]);
-    half_jvp(wr, gm1, P.K, -1, hr, dqr[d], t);
-#pragma unroll
-    for (int q = 0; q < 5; ++q) dW[d][q] += t[q];
-  }
-  R dWt[5], E0[5], E1[5], E2[5], tau;
-  interface_terms(P, wl.p, wr.p, q0, w0, dW, dt, dWt, E0, E1, E2, tau);
-  if (!P.full) {
-    smooth_from_terms(P, q0, w0, dWt, E0, E1, E2, tau, Fn, Ft);
-    return true;
-  }
-  // full flux: the non-equilibrium parts of both sides. With the side's slopes a_d (rho <a_d psi>
-  // = dq_d) and time slope A (rho <A psi> = -sum_d A_d(W) dq_d, Euler Jacobians at the side's
-  // state): N0 = F+(W), N1 = sum_d DT+_d[dq_d] = rho <u (a . c) psi>_+, N2 = DF+[rho <A psi>]
-  // = rho <u A psi>_+ (half line u > 0 on the left, u < 0 on the right)
-  R NL[3][5], NR[3][5];
-  {
-    HalfLine<R> ml, mr;
-    half_line(wl, hl, ml);
-    half_line(wr, hr, mr);
-    half_flux(wl, P.K, ml, NL[0]);
-    half_flux(wr, P.K, mr, NR[0]);
-    R dtl[5], dtr[5];
-    const R Epl = ql[4] + wl.p, Epr = qr[4] + wr.p;
-    euler_jvp(wl, irl, gm1, Epl, 0, dql[0], dtl);
-    euler_jvp(wr, irr, gm1, Epr, 0, dqr[0], dtr);
-    half_second_jvp(wl, gm1, P.K, +1, ml, 0, dql[0], NL[1]);
-    half_second_jvp(wr, gm1, P.K, -1, mr, 0, dqr[0], NR[1]);
-#pragma unroll
-    for (int d = 1; d < 3; ++d) {
-      euler_jvp(wl, irl, gm1, Epl, d, dql[d], t);
-#pragma unroll
-      for (int q = 0; q < 5; ++q) dtl[q] += t[q];
-      euler_jvp(wr, irr, gm1, Epr, d, dqr[d], t);
-#pragma unroll
-      for (int q = 0; q < 5; ++q) dtr[q] += t[q];
-      half_second_jvp(wl, gm1, P.K, +1, ml, d, dql[d], t);
-#pragma unroll
-      for (int q = 0; q < 5; ++q) NL[1][q] += t[q];
-      half_second_jvp(wr, gm1, P.K, -1, mr, d, dqr[d], t);
-#pragma unroll
-      for (int q = 0; q < 5; ++q) NR[1][q] += t[q];
-    }
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      dtl[q] = -dtl[q];
-      dtr[q] = -dtr[q];
-    }
-    half_flux_jvp(wl, gm1, P.K, +1, ml, dtl, NL[2]);
-    half_flux_jvp(wr, gm1, P.K, -1, mr, dtr, NR[2]);
-  }
-  R cn[6], ct[6];
-  full_fit_coeffs(tau, dt, cn, ct);
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    const R geq_n = cn[0] * E0[q] + cn[1] * E1[q] + cn[2] * E2[q];
-    const R geq_t = ct[0] * E0[q] + ct[1] * E1[q] + ct[2] * E2[q];
-    const R gl_n = cn[3] * NL[0][q] + cn[4] * NL[1][q] + cn[5] * NL[2][q];
-    const R gl_t = ct[3] * NL[0][q] + ct[4] * NL[1][q] + ct[5] * NL[2][q];
-    const R gr_n = cn[3] * NR[0][q] + cn[4] * NR[1][q] + cn[5] * NR[2][q];
-    const R gr_t = ct[3] * NR[0][q] + ct[4] * NR[1][q] + ct[5] * NR[2][q];
-    Fn[q] = geq_n + gl_n + gr_n;
-    Ft[q] = geq_t + gl_t + gr_t;
-  }
-  return true;
-}
-
 // The ten coefficients of variable v through the accessor; accessors over device memory
 // provide their own (vector-load) version, found by argument-dependent lookup.
 template <class Coef, class R>
@@ -711,89 +527,19 @@ GKS_HD void load_coefs(const Coef& coef, int v, R k[10]) {
 // + c9 dydz. `coef(v, j)` returns coefficient j of variable v.
 template <class R, class Coef>
 GKS_HD void eval_poly(const Coef& coef, const R d[3], R val[5], R grad[5][3]) {
-  const R xx = d[0] * d[0], yy = d[1] * d[1], zz = d[2] * d[2];
-  const R xy = d[0] * d[1], xz = d[0] * d[2], yz = d[1] * d[2];
+  const R tx = R(2) * d[0], ty = R(2) * d[1], tz = R(2) * d[2];
+  const R hx = R(0.5) * d[0], hy = R(0.5) * d[1], hz = R(0.5) * d[2];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     R k[10];
     load_coefs(coef, v, k);
-    val[v] = k[0] + k[1] * d[0] + k[2] * d[1] + k[3] * d[2] + k[4] * xx + k[5] * yy + k[6] * zz +
-             k[7] * xy + k[8] * xz + k[9] * yz;
-    grad[v][0] = k[1] + R(2) * k[4] * d[0] + k[7] * d[1] + k[8] * d[2];
-    grad[v][1] = k[2] + R(2) * k[5] * d[1] + k[7] * d[0] + k[9] * d[2];
-    grad[v][2] = k[3] + R(2) * k[6] * d[2] + k[8] * d[0] + k[9] * d[1];
+    grad[v][0] = k[1] + k[4] * tx + k[7] * d[1] + k[8] * d[2];
+    grad[v][1] = k[2] + k[5] * ty + k[7] * d[0] + k[9] * d[2];
+    grad[v][2] = k[3] + k[6] * tz + k[8] * d[0] + k[9] * d[1];
+    // Q(d) = c0 + d . (grad Q(0) + grad Q(d)) / 2 for a quadratic: 15 instructions a variable
+    // against 21 with the products of the offsets
+    val[v] = k[0] + hx * (k[1] + grad[v][0]) + hy * (k[2] + grad[v][1]) + hz * (k[3] + grad[v][2]);
   }
-}
-
-// The local frame of a Gauss point: n1 the unit normal, n2 = n1 x e_k / |n1 x e_k| with e_k the
-// axis least aligned with n1, n3 = n1 x n2.
-template <class R>
-GKS_HD void face_frame(const R n1[3], R n2[3], R n3[3]) {
-  int kk = 0;
-  if (k_abs(n1[1]) < k_abs(n1[kk])) kk = 1;
-  if (k_abs(n1[2]) < k_abs(n1[kk])) kk = 2;
-  if (kk == 0) { n2[0] = R(0); n2[1] = n1[2]; n2[2] = -n1[1]; }
-  else if (kk == 1) { n2[0] = -n1[2]; n2[1] = R(0); n2[2] = n1[0]; }
-  else { n2[0] = n1[1]; n2[1] = -n1[0]; n2[2] = R(0); }
-  const R il = k_div(R(1), k_sqrt(n2[0] * n2[0] + n2[1] * n2[1] + n2[2] * n2[2]));
-  n2[0] = n2[0] * il; n2[1] = n2[1] * il; n2[2] = n2[2] * il;
-  n3[0] = n1[1] * n2[2] - n1[2] * n2[1];
-  n3[1] = n1[2] * n2[0] - n1[0] * n2[2];
-  n3[2] = n1[0] * n2[1] - n1[1] * n2[0];
-}
-
-// A local-frame flux (F^n, dF/dt) rotated back to the global frame and weighted by the
-// quadrature weight w: acc[0..4] = w F^n, acc[5..9] = w dF/dt.
-template <class R>
-GKS_HD void rotate_flux_out(const R Fn[5], const R Ft[5], const R n1[3], const R n2[3],
-                            const R n3[3], R w, R acc[10]) {
-  acc[0] = w * Fn[0];
-  acc[4] = w * Fn[4];
-  acc[5] = w * Ft[0];
-  acc[9] = w * Ft[4];
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    acc[1 + a] = w * (Fn[1] * n1[a] + Fn[2] * n2[a] + Fn[3] * n3[a]);
-    acc[6 + a] = w * (Ft[1] * n1[a] + Ft[2] * n2[a] + Ft[3] * n3[a]);
-  }
-}
-
-// Whole Gauss-point contribution in the global frame. Left/right values and gradients are
-// rotated into the local frame (n1 the unit normal, n2 = n1 x e_k / |n1 x e_k| with e_k the axis
-// least aligned with n1, n3 = n1 x n2), the local flux is computed, rotated back and multiplied
-// by the quadrature weight w: acc[0..4] = w F^n, acc[5..9] = w dF/dt.
-template <class R>
-GKS_HD bool gp_flux_global(const FluxParams<R>& P, const R vl[5], const R gl[5][3], const R vr[5],
-                           const R gr[5][3], const R n1[3], R w, R dt, R acc[10]) {
-  R n2[3], n3[3];
-  face_frame(n1, n2, n3);
-  const R* nm[3] = {n1, n2, n3};
-  R ql[5], qr[5], dql[3][5], dqr[3][5];
-  ql[0] = vl[0]; ql[4] = vl[4]; qr[0] = vr[0]; qr[4] = vr[4];
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    ql[1 + d] = vl[1] * nm[d][0] + vl[2] * nm[d][1] + vl[3] * nm[d][2];
-    qr[1 + d] = vr[1] * nm[d][0] + vr[2] * nm[d][1] + vr[3] * nm[d][2];
-  }
-#pragma unroll
-  for (int d = 0; d < 3; ++d) {
-    R sl[5], sr[5];
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      sl[v] = gl[v][0] * nm[d][0] + gl[v][1] * nm[d][1] + gl[v][2] * nm[d][2];
-      sr[v] = gr[v][0] * nm[d][0] + gr[v][1] * nm[d][1] + gr[v][2] * nm[d][2];
-    }
-    dql[d][0] = sl[0]; dql[d][4] = sl[4]; dqr[d][0] = sr[0]; dqr[d][4] = sr[4];
-#pragma unroll
-    for (int e = 0; e < 3; ++e) {
-      dql[d][1 + e] = sl[1] * nm[e][0] + sl[2] * nm[e][1] + sl[3] * nm[e][2];
-      dqr[d][1 + e] = sr[1] * nm[e][0] + sr[2] * nm[e][1] + sr[3] * nm[e][2];
-    }
-  }
-  R Fn[5], Ft[5];
-  if (!gks_gp_flux(P, ql, dql, qr, dqr, dt, Fn, Ft)) return false;
-  rotate_flux_out(Fn, Ft, n1, n2, n3, w, acc);
-  return true;
 }
 
 }  // namespace gks

@@ -1,11 +1,10 @@
 // Algorithmic operation count of one face Gauss point of the flux kernel: the same templated
-// device code (polynomial evaluation of both sides, frame rotation, gas-kinetic flux, back
-// rotation, weighting) instantiated on the host with a scalar type that counts its arithmetic.
+// device code (polynomial evaluation of both sides, gas-kinetic flux, weighting) instantiated on the host with a scalar type that counts its arithmetic.
 // Used to state the flops per unit behind the roofline fraction of the flux kernel.
 #include <cmath>
 #include <cstdint>
 
-#include "gks_kinetic.cuh"
+#include "gks_flux.cuh"
 
 namespace gks {
 namespace opc {
