@@ -62,6 +62,28 @@ __device__ __forceinline__ void poly_mean_adj(const double mu[6], const double g
   }
 }
 
+// Sum over the four Gauss points of a face (four consecutive lanes) of one side's polynomial
+// cotangents x[50], written to dst. Each exchange halves what a lane carries (lane bit 0 keeps
+// coefficients 0..24 or 25..49, bit 1 the first 13 or the rest of those), so a lane does 38
+// additions and exchanges instead of 100 of each, and all four write.
+__device__ __forceinline__ void sum_points(const double x[5][10], bool store,
+                                           double* __restrict__ dst) {
+  const int b0 = threadIdx.x & 1, b1 = (threadIdx.x >> 1) & 1;
+  double y[26];
+#pragma unroll
+  for (int i = 0; i < 25; ++i) {
+    const double lo = x[i / 10][i % 10], hi = x[(i + 25) / 10][(i + 25) % 10];
+    y[i] = (b0 ? hi : lo) + __shfl_xor_sync(0xffffffffu, b0 ? lo : hi, 1);
+  }
+  y[25] = 0.0;
+  double* o = dst + 25 * b0 + 13 * b1;
+#pragma unroll
+  for (int i = 0; i < 13; ++i) {
+    const double z = (b1 ? y[13 + i] : y[i]) + __shfl_xor_sync(0xffffffffu, b1 ? y[i] : y[13 + i], 2);
+    if (store && (i < 12 || !b1)) o[i] = z;
+  }
+}
+
 // kFull and kTau0 fix the flux form and a zero collision time at compile time (as in the forward
 // kernel), so that each instance holds only its own form's recomputed forward state. kWalls =
 // false is the instance for meshes without boundary planes (every face has two cells; no
@@ -79,14 +101,19 @@ __global__ void __launch_bounds__(128) k_vjp_flux(
   const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   const int64_t f = gid >> 2;
   const bool active = f < nf;
-  double go[5][10], gn[5][10];
+  double gvl[5] = {0, 0, 0, 0, 0}, gvr[5] = {0, 0, 0, 0, 0};
+  double ggl[5][3], ggr[5][3];
 #pragma unroll
   for (int v = 0; v < 5; ++v)
 #pragma unroll
-    for (int j = 0; j < 10; ++j) go[v][j] = gn[v][j] = 0.0;
+    for (int a = 0; a < 3; ++a) ggl[v][a] = ggr[v][a] = 0.0;
+  double dl[3] = {0, 0, 0}, dr[3] = {0, 0, 0};
+  bool fbl = false, fbr = false;
+  int32_t o = 0, nb = 0;
   if (active) {
     const int64_t stride = 4 * nf;
-    const int32_t o = f_owner[f], nb = f_nb[f];
+    o = f_owner[f];
+    nb = f_nb[f];
     const int wall = f_wall[f];
     // cotangent of the face flux: L_o -= F / |O_o|, L_nb += F / |O_nb|
     double gacc[10];
@@ -106,7 +133,7 @@ __global__ void __launch_bounds__(128) k_vjp_flux(
     } else {
       wall_flux_fix_adj(wall, wall_data(wall_tab, wall), gacc);  // the wall treatment, reversed
     }
-    double dl[3], dr[3], n1[3];
+    double n1[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
       dl[a] = fgp[a * stride + gid];
@@ -116,13 +143,12 @@ __global__ void __launch_bounds__(128) k_vjp_flux(
     const double w = fgp[9 * stride + gid];
     double vl[5], gl[5][3], vr[5], gr[5][3];
     eval_poly(PolyRef64{poly + (int64_t)kPolyStride * o}, dl, vl, gl);
-    const bool fbl = fallback && nonphysical(vl);
-    double mu[6];
+    fbl = fallback && nonphysical(vl);
     if (fbl) {
+      double mu[6];
       central_moments(mom, hcell, nc, o, mu);
       poly_mean(poly + (int64_t)kPolyStride * o, mu, vl, gl);
     }
-    bool fbr = false;
     if (!kWalls || nb >= 0) {
       eval_poly(PolyRef64{poly + (int64_t)kPolyStride * nb}, dr, vr, gr);
       fbr = fallback && nonphysical(vr);
@@ -134,50 +160,36 @@ __global__ void __launch_bounds__(128) k_vjp_flux(
     } else {
       wall_ghost<double, true>(P, wall, wall_data(wall_tab, wall), vl, gl, vr, gr);
     }
-    double gvl[5] = {0, 0, 0, 0, 0}, gvr[5] = {0, 0, 0, 0, 0};
-    double ggl[5][3], ggr[5][3];
-#pragma unroll
-    for (int v = 0; v < 5; ++v)
-#pragma unroll
-      for (int a = 0; a < 3; ++a) ggl[v][a] = ggr[v][a] = 0.0;
     if (gp_flux_global_vjp(P, vl, gl, vr, gr, n1, w, dt, gacc, gvl, ggl, gvr, ggr)) {
       // the wall's ghost is a function of the owner's value and gradient: fold its cotangent back
       if (kWalls && nb < 0)
         wall_ghost_vjp(P, wall, wall_data(wall_tab, wall), vl, gl, gvr, ggr, gvl, ggl);
-      if (fbl)
-        poly_mean_adj(mu, gvl, go);
-      else
-        eval_poly_adj(dl, gvl, ggl, go);
-      if (fbr) {
-        double mun[6];
-        central_moments(mom, hcell, nc, nb, mun);
-        poly_mean_adj(mun, gvr, gn);
-      } else if (!kWalls || nb >= 0) {
-        eval_poly_adj(dr, gvr, ggr, gn);
-      }
     } else {
       atomicOr(flag, kErrNonphysical);
     }
   }
+  // one side after the other, so that 50 cotangents are held at a time; a point that
+  // contributes nothing (inactive lane, non-physical state) has zero gv, gg
+  double* po = gpf + (int64_t)2 * kPolyStride * f;
 #pragma unroll
-  for (int v = 0; v < 5; ++v)
-#pragma unroll
-    for (int j = 0; j < 10; ++j) {
-      go[v][j] += __shfl_xor_sync(0xffffffffu, go[v][j], 1);
-      go[v][j] += __shfl_xor_sync(0xffffffffu, go[v][j], 2);
-      gn[v][j] += __shfl_xor_sync(0xffffffffu, gn[v][j], 1);
-      gn[v][j] += __shfl_xor_sync(0xffffffffu, gn[v][j], 2);
-    }
-  if (active && (gid & 3) == 0) {
-    double* po = gpf + (int64_t)2 * kPolyStride * f;
-    double* pn = po + kPolyStride;
+  for (int side = 0; side < 2; ++side) {
+    double x[5][10];
 #pragma unroll
     for (int v = 0; v < 5; ++v)
 #pragma unroll
-      for (int j = 0; j < 10; ++j) {
-        po[10 * v + j] = go[v][j];
-        pn[10 * v + j] = gn[v][j];
-      }
+      for (int j = 0; j < 10; ++j) x[v][j] = 0.0;
+    const int32_t c = side ? nb : o;
+    if (side ? fbr : fbl) {
+      double mu[6];
+      central_moments(mom, hcell, nc, c, mu);
+      poly_mean_adj(mu, side ? gvr : gvl, x);
+    } else if (!kWalls || c >= 0) {
+      if (side)
+        eval_poly_adj(dr, gvr, ggr, x);
+      else
+        eval_poly_adj(dl, gvl, ggl, x);
+    }
+    sum_points(x, active, po + side * kPolyStride);
   }
 }
 
@@ -488,9 +500,10 @@ void launch_vjp(const DevMesh& m, const Geo64& g64, const GeoR<double>& g, const
   const Kern tab[2][2][2] = {
       {{k_vjp_flux<false, false, false>, k_vjp_flux<false, false, true>},
        {k_vjp_flux<false, true, false>, k_vjp_flux<false, true, true>}},
-      {{k_vjp_flux<true, false, false>, k_vjp_flux<true, false, true>},
-       {k_vjp_flux<true, true, false>, k_vjp_flux<true, true, true>}}};
-  const Kern kern = tab[fp.full ? 1 : 0][fp.tau_model == 0 ? 1 : 0][m.bcs != 0 ? 1 : 0];
+      {{k_vjp_flux<true, false, false>, k_vjp_flux<true, false, true>}, {nullptr, nullptr}}};
+  // without a collision time the full form is the smooth one, as in the forward
+  const Kern kern = fp.tau_model == 0 ? tab[0][1][m.bcs != 0 ? 1 : 0]
+                                      : tab[fp.full ? 1 : 0][0][m.bcs != 0 ? 1 : 0];
   // the flux adjoint keeps kilobytes of spilled state per thread in its stack frame (4-6 KB for
   // the full flux): raise the context's per-thread stack limit to cover it before the launch
   cudaFuncAttributes at;

@@ -66,19 +66,23 @@ extern "C" int gks_gp_flux_vjp_host(const double* p, const double* ql, const dou
                                     const double* gFn, const double* gFt, double* gql,
                                     double* gdql, double* gqr, double* gdqr) {
   const gks::FluxParams<double> P = params_from(p);
-  double a[3][5], b[3][5], ga[3][5], gb[3][5];
-  for (int d = 0; d < 3; ++d)
-    for (int v = 0; v < 5; ++v) {
-      a[d][v] = dql[5 * d + v];
-      b[d][v] = dqr[5 * d + v];
-      ga[d][v] = gb[d][v] = 0.0;
+  const double n[3] = {1.0, 0.0, 0.0};
+  double a[5][3], b[5][3], ga[5][3], gb[5][3], gacc[10];
+  for (int v = 0; v < 5; ++v) {
+    gql[v] = gqr[v] = 0.0;
+    gacc[v] = gFn[v];
+    gacc[5 + v] = gFt[v];
+    for (int d = 0; d < 3; ++d) {
+      a[v][d] = dql[5 * d + v];
+      b[v][d] = dqr[5 * d + v];
+      ga[v][d] = gb[v][d] = 0.0;
     }
-  for (int v = 0; v < 5; ++v) gql[v] = gqr[v] = 0.0;
-  if (!gks::gks_gp_flux_vjp_cf(P, ql, a, qr, b, dt, gFn, gFt, gql, ga, gqr, gb)) return 1;
+  }
+  if (!gks::gp_flux_global_vjp(P, ql, a, qr, b, n, 1.0, dt, gacc, gql, ga, gqr, gb)) return 1;
   for (int d = 0; d < 3; ++d)
     for (int v = 0; v < 5; ++v) {
-      gdql[5 * d + v] = ga[d][v];
-      gdqr[5 * d + v] = gb[d][v];
+      gdql[5 * d + v] = ga[v][d];
+      gdqr[5 * d + v] = gb[v][d];
     }
   return 0;
 }

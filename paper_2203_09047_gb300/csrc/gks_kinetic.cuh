@@ -1,6 +1,6 @@
-// Gas-kinetic flux at one Gauss point (Section 3.2), written for the GPU: the half-space and
-// interface-equilibrium moments in closed form, the slope terms as directional derivatives of
-// closed-form moment vectors (no slope solve), and the time-fitted flux F^n, dF/dt.
+// Shared parts of the Gauss-point flux (Section 3.2): scalar functions per type, primitives,
+// flux parameters, collision time, boundary ghosts and the evaluation of the reconstruction. The
+// flux itself is in gks_flux.cuh.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -60,254 +60,6 @@ GKS_HD bool to_prim(const R q[5], R gamma, Prim<R>& w) {
   w.lam = R(0.5) * w.rho * w.ip;
   w.hil = w.p * w.ir;
   return (w.rho > R(0)) && (w.p > R(0));  // false also for NaN
-}
-
-// Moments of an equilibrium in closed form. For a Maxwellian g(W) of the conserved state W,
-// dg = g (a . psi) with rho <a psi> = dW, so rho <c_d (a psi) psi> is the derivative of the
-// Euler flux along axis d applied to dW. euler_flux_x: rho <u psi> = F_x(W).
-// euler_jvp: A_d(W) dW = dF_d/dW dW, with dU = (dm - U drho)/rho and
-// dp = (gamma - 1) (dE - U . dm + |U|^2 drho / 2).
-template <class R>
-GKS_HD void euler_flux_x(const Prim<R>& w, R E, R F[5]) {
-  const R m = w.rho * w.U;
-  F[0] = m;
-  F[1] = m * w.U + w.p;
-  F[2] = m * w.V;
-  F[3] = m * w.W;
-  F[4] = w.U * (E + w.p);
-}
-template <class R>
-GKS_HD void euler_jvp(const Prim<R>& w, R ir, R gm1, R Ep, int d, const R dq[5], R out[5]) {
-  const R U[3] = {w.U, w.V, w.W};
-  const R du[3] = {(dq[1] - U[0] * dq[0]) * ir, (dq[2] - U[1] * dq[0]) * ir,
-                   (dq[3] - U[2] * dq[0]) * ir};
-  const R u2 = U[0] * U[0] + U[1] * U[1] + U[2] * U[2];
-  const R dp = gm1 * (dq[4] - (U[0] * dq[1] + U[1] * dq[2] + U[2] * dq[3]) + R(0.5) * u2 * dq[0]);
-  const R md = w.rho * U[d], dmd = dq[1 + d];
-  out[0] = dmd;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) out[1 + a] = dmd * U[a] + md * du[a];
-  out[1 + d] += dp;
-  out[4] = du[d] * Ep + U[d] * (dq[4] + dp);  // Ep = E + p
-}
-
-// Second-moment flux of an equilibrium along axis d, T_d(W) = rho <u c_d psi>, with theta = p/rho:
-//   T_d[0]     = rho (U_0 U_d + theta delta_0d)
-//   T_d[1 + a] = rho (U_0 U_d U_a + theta (U_0 delta_da + U_d delta_0a + U_a delta_0d))
-//   T_d[4]     = rho/2 (U_0 U_d (|U|^2 + (K + 7) theta) + delta_0d theta (|U|^2 + (K + 5) theta))
-// (u = c_0 the normal velocity). second_moment_jvp returns its derivative along the conserved
-// increment dq, which equals rho <u c_d (a psi) psi> for the slope a with rho <a psi> = dq.
-template <class R>
-GKS_HD void second_moment_jvp(const Prim<R>& w, R ir, R gm1, R K, int d, const R dq[5], R out[5]) {
-  const R U[3] = {w.U, w.V, w.W};
-  const R dU[3] = {(dq[1] - U[0] * dq[0]) * ir, (dq[2] - U[1] * dq[0]) * ir,
-                   (dq[3] - U[2] * dq[0]) * ir};
-  const R q = U[0] * U[0] + U[1] * U[1] + U[2] * U[2];
-  const R dp = gm1 * (dq[4] - (U[0] * dq[1] + U[1] * dq[2] + U[2] * dq[3]) + R(0.5) * q * dq[0]);
-  const R th = w.p * ir;
-  const R dth = (dp - th * dq[0]) * ir;
-  const R dq2 = R(2) * (U[0] * dU[0] + U[1] * dU[1] + U[2] * dU[2]);
-  const R Ud = U[d], dUd = dU[d];
-  const R uu = U[0] * Ud, duu = dU[0] * Ud + U[0] * dUd;  // U_0 U_d and its derivative
-  const R n = d == 0 ? R(1) : R(0);
-  // per unit density: t and its derivative dt; out = drho t + rho dt
-  R t[5], dt[5];
-  t[0] = uu + th * n;
-  dt[0] = duu + dth * n;
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    const R da = a == d ? R(1) : R(0), za = a == 0 ? R(1) : R(0);
-    const R g = U[0] * da + Ud * za + U[a] * n, dg = dU[0] * da + dUd * za + dU[a] * n;
-    t[1 + a] = uu * U[a] + th * g;
-    dt[1 + a] = duu * U[a] + uu * dU[a] + dth * g + th * dg;
-  }
-  const R c7 = K + R(7), c5 = K + R(5);
-  t[4] = R(0.5) * (uu * (q + c7 * th) + n * th * (q + c5 * th));
-  dt[4] = R(0.5) * (duu * (q + c7 * th) + uu * (dq2 + c7 * dth) +
-                    n * (dth * (q + c5 * th) + th * (dq2 + c5 * dth)));
-#pragma unroll
-  for (int k = 0; k < 5; ++k) out[k] = dq[0] * t[k] + w.rho * dt[k];
-}
-
-// Half-line equilibrium of one side (u > 0 for s = +1, u < 0 for s = -1; s is an int, or a
-// packed pair of signs when R carries both sides) in closed form:
-// A = <1>, A1 = <u>, A2 = <u^2> over the half line, B = exp(-lam U^2) / (2 sqrt(pi lam)) and
-// S = <v^2 + w^2 + xi^2>, so that rho <psi> = rho (A, A1, V A, W A, (A2 + S A) / 2).
-template <class R>
-struct Half {
-  R A, A1, A2, B, S;
-};
-template <class R, class Sg>
-GKS_HD void half_init(const Prim<R>& w, R K, Sg s, Half<R>& h) {
-  const R sl = k_sqrt(w.lam);
-  h.A = R(0.5) * k_erfc(-R(s) * sl * w.U);
-  h.B = k_div(R(0.28209479177387814) * k_exp(-w.lam * w.U * w.U), sl);  // 1/(2 sqrt(pi))
-  h.A1 = w.U * h.A + R(s) * h.B;
-  h.A2 = w.U * h.A1 + w.hil * h.A;
-  h.S = w.V * w.V + w.W * w.W + (K + R(2)) * w.hil;
-}
-template <class R>
-GKS_HD void half_moments(const Prim<R>& w, const Half<R>& h, R Q[5]) {
-  Q[0] = w.rho * h.A;
-  Q[1] = w.rho * h.A1;
-  Q[2] = w.rho * w.V * h.A;
-  Q[3] = w.rho * w.W * h.A;
-  Q[4] = R(0.5) * w.rho * (h.A2 + h.S * h.A);
-}
-// Derivative of rho <psi> (half line) along the conserved increment dq, through the primitive
-// increments dU = (dm - U drho)/rho, dp = (gamma - 1)(dE - U . dm + |U|^2 drho / 2),
-// dlam/lam = drho/rho - dp/p, with dA = s B (2 lam dU + U dlam),
-// dB = -B (2 lam U dU + (U^2 + 1/(2 lam)) dlam). Equals rho <a psi> (half line) for the slope a
-// of the Maxwellian with rho <a psi> = dq over the full line. No division: the reciprocals come
-// with the primitives.
-template <class R, class Sg>
-GKS_HD void half_jvp(const Prim<R>& w, R gm1, R K, Sg s, const Half<R>& h, const R dq[5],
-                     R dQ[5]) {
-  const R ir = w.ir, hil = w.hil;
-  const R dU = (dq[1] - w.U * dq[0]) * ir, dV = (dq[2] - w.V * dq[0]) * ir,
-          dW = (dq[3] - w.W * dq[0]) * ir;
-  const R u2 = w.U * w.U + w.V * w.V + w.W * w.W;
-  const R dp = gm1 * (dq[4] - (w.U * dq[1] + w.V * dq[2] + w.W * dq[3]) + R(0.5) * u2 * dq[0]);
-  const R dll = dq[0] * ir - dp * w.ip;  // dlam / lam
-  const R dlam = w.lam * dll;
-  const R dA = R(s) * h.B * (R(2) * w.lam * dU + w.U * dlam);
-  const R dB = -h.B * (R(2) * w.lam * w.U * dU + (w.U * w.U + hil) * dlam);
-  const R dA1 = dU * h.A + w.U * dA + R(s) * dB;
-  const R dA2 = dU * h.A1 + w.U * dA1 + hil * (dA - h.A * dll);
-  const R dS = R(2) * (w.V * dV + w.W * dW) - (K + R(2)) * hil * dll;
-  dQ[0] = dq[0] * h.A + w.rho * dA;
-  dQ[1] = dq[0] * h.A1 + w.rho * dA1;
-  dQ[2] = dq[0] * w.V * h.A + w.rho * (dV * h.A + w.V * dA);
-  dQ[3] = dq[0] * w.W * h.A + w.rho * (dW * h.A + w.W * dA);
-  dQ[4] = R(0.5) * (dq[0] * (h.A2 + h.S * h.A) + w.rho * (dA2 + dS * h.A + h.S * dA));
-}
-
-// Half-line flux terms of the full flux in closed form. With the half-line moments
-// A_n = <u^n> (n = 0..4, A_{n+2} = U A_{n+1} + (n + 1) A_n / (2 lam)), the full-line moments of
-// v, w and xi^2 = K / (2 lam):
-//   F+(W)    = rho <u psi>     = rho (A1, A2, V A1, W A1, (A3 + S A1) / 2),
-//   T+_0(W)  = rho <u u psi>   = rho (A2, A3, V A2, W A2, (A4 + S A2) / 2),
-//   T+_1(W)  = rho <u v psi>   = rho (V A1, V A2, <v^2> A1, V W A1, (V A3 + Y_v A1) / 2),
-//   T+_2(W)  = rho <u w psi>   = rho (W A1, W A2, V W A1, <w^2> A1, (W A3 + Y_w A1) / 2),
-// S = V^2 + W^2 + (K + 2)/(2 lam), Y_v = V (V^2 + W^2 + (K + 4)/(2 lam)), Y_w likewise. Their
-// derivatives along a conserved increment dW are the half-line slope terms of Eq. flux-1:
-// rho <u (a psi) psi>_+ = DF+[dW] and rho <u c_d (a psi) psi>_+ = DT+_d[dW] for the slope a with
-// rho <a psi> = dW.
-template <class R>
-struct HalfLine {
-  R A[5], B;
-};
-template <class R>
-GKS_HD void half_line(const Prim<R>& w, const Half<R>& h, HalfLine<R>& m) {
-  m.A[0] = h.A;
-  m.A[1] = h.A1;
-  m.A[2] = h.A2;
-  m.A[3] = w.U * m.A[2] + R(2) * w.hil * m.A[1];
-  m.A[4] = w.U * m.A[3] + R(3) * w.hil * m.A[2];
-  m.B = h.B;
-}
-// Primitive increments along dq and the half-line moment increments dA[0..4].
-template <class R>
-struct DPrim {
-  R drho, dU, dV, dW, dlam, dhil;
-};
-template <class R>
-GKS_HD void dprim(const Prim<R>& w, R gm1, const R dq[5], DPrim<R>& d) {
-  const R ir = w.ir;
-  d.drho = dq[0];
-  d.dU = (dq[1] - w.U * dq[0]) * ir;
-  d.dV = (dq[2] - w.V * dq[0]) * ir;
-  d.dW = (dq[3] - w.W * dq[0]) * ir;
-  const R u2 = w.U * w.U + w.V * w.V + w.W * w.W;
-  const R dp = gm1 * (dq[4] - (w.U * dq[1] + w.V * dq[2] + w.W * dq[3]) + R(0.5) * u2 * dq[0]);
-  const R dll = dq[0] * ir - dp * w.ip;  // dlam / lam
-  d.dlam = w.lam * dll;
-  d.dhil = -w.hil * dll;
-}
-template <class R, class Sg>
-GKS_HD void dhalf_line(const Prim<R>& w, Sg s, const HalfLine<R>& m, const DPrim<R>& d,
-                       R dA[5]) {
-  const R U = w.U, hil = w.hil;
-  dA[0] = R(s) * m.B * (R(2) * w.lam * d.dU + U * d.dlam);
-  const R dB = -m.B * (R(2) * w.lam * U * d.dU + (U * U + hil) * d.dlam);
-  dA[1] = d.dU * m.A[0] + U * dA[0] + R(s) * dB;
-  dA[2] = d.dU * m.A[1] + U * dA[1] + d.dhil * m.A[0] + hil * dA[0];
-  dA[3] = d.dU * m.A[2] + U * dA[2] + R(2) * (d.dhil * m.A[1] + hil * dA[1]);
-  dA[4] = d.dU * m.A[3] + U * dA[3] + R(3) * (d.dhil * m.A[2] + hil * dA[2]);
-}
-template <class R>
-GKS_HD void half_flux(const Prim<R>& w, R K, const HalfLine<R>& m, R F[5]) {
-  const R S = w.V * w.V + w.W * w.W + (K + R(2)) * w.hil;
-  F[0] = w.rho * m.A[1];
-  F[1] = w.rho * m.A[2];
-  F[2] = w.rho * w.V * m.A[1];
-  F[3] = w.rho * w.W * m.A[1];
-  F[4] = R(0.5) * w.rho * (m.A[3] + S * m.A[1]);
-}
-// DF+[dq]
-template <class R, class Sg>
-GKS_HD void half_flux_jvp(const Prim<R>& w, R gm1, R K, Sg s, const HalfLine<R>& m,
-                          const R dq[5], R out[5]) {
-  DPrim<R> d;
-  dprim(w, gm1, dq, d);
-  R dA[5];
-  dhalf_line(w, s, m, d, dA);
-  const R S = w.V * w.V + w.W * w.W + (K + R(2)) * w.hil;
-  const R dS = R(2) * (w.V * d.dV + w.W * d.dW) + (K + R(2)) * d.dhil;
-  out[0] = d.drho * m.A[1] + w.rho * dA[1];
-  out[1] = d.drho * m.A[2] + w.rho * dA[2];
-  out[2] = d.drho * w.V * m.A[1] + w.rho * (d.dV * m.A[1] + w.V * dA[1]);
-  out[3] = d.drho * w.W * m.A[1] + w.rho * (d.dW * m.A[1] + w.W * dA[1]);
-  out[4] = R(0.5) * (d.drho * (m.A[3] + S * m.A[1]) +
-                     w.rho * (dA[3] + dS * m.A[1] + S * dA[1]));
-}
-// DT+_k[dq] for the velocity component k (0 normal, 1, 2 tangential)
-template <class R, class Sg>
-GKS_HD void half_second_jvp(const Prim<R>& w, R gm1, R K, Sg s, const HalfLine<R>& m, int k,
-                            const R dq[5], R out[5]) {
-  DPrim<R> d;
-  dprim(w, gm1, dq, d);
-  R dA[5];
-  dhalf_line(w, s, m, d, dA);
-  const R V = w.V, W = w.W, hil = w.hil;
-  R t[5], dt[5];
-  if (k == 0) {
-    const R S = V * V + W * W + (K + R(2)) * hil;
-    const R dS = R(2) * (V * d.dV + W * d.dW) + (K + R(2)) * d.dhil;
-    t[0] = m.A[2];
-    dt[0] = dA[2];
-    t[1] = m.A[3];
-    dt[1] = dA[3];
-    t[2] = V * m.A[2];
-    dt[2] = d.dV * m.A[2] + V * dA[2];
-    t[3] = W * m.A[2];
-    dt[3] = d.dW * m.A[2] + W * dA[2];
-    t[4] = R(0.5) * (m.A[4] + S * m.A[2]);
-    dt[4] = R(0.5) * (dA[4] + dS * m.A[2] + S * dA[2]);
-  } else {
-    // c = the tangential component k, o = the other one
-    const R c = k == 1 ? V : W, o = k == 1 ? W : V;
-    const R dc = k == 1 ? d.dV : d.dW, dO = k == 1 ? d.dW : d.dV;
-    const R c2 = c * c + hil, dc2 = R(2) * c * dc + d.dhil;  // <c^2>
-    const R q = V * V + W * W + (K + R(4)) * hil;
-    const R dqq = R(2) * (V * d.dV + W * d.dW) + (K + R(4)) * d.dhil;
-    const R Y = c * q, dY = dc * q + c * dqq;
-    t[0] = c * m.A[1];
-    dt[0] = dc * m.A[1] + c * dA[1];
-    t[1] = c * m.A[2];
-    dt[1] = dc * m.A[2] + c * dA[2];
-    // momentum components along this tangential axis and the other one
-    const R tc = c2 * m.A[1], dtc = dc2 * m.A[1] + c2 * dA[1];
-    const R to = c * o * m.A[1], dto = (dc * o + c * dO) * m.A[1] + c * o * dA[1];
-    t[2] = k == 1 ? tc : to;
-    dt[2] = k == 1 ? dtc : dto;
-    t[3] = k == 1 ? to : tc;
-    dt[3] = k == 1 ? dto : dtc;
-    t[4] = R(0.5) * (c * m.A[3] + Y * m.A[1]);
-    dt[4] = R(0.5) * (dc * m.A[3] + c * dA[3] + dY * m.A[1] + Y * dA[1]);
-  }
-#pragma unroll
-  for (int q2 = 0; q2 < 5; ++q2) out[q2] = d.drho * t[q2] + w.rho * dt[q2];
 }
 
 template <class R>
@@ -499,19 +251,6 @@ GKS_HD void wall_flux_fix(int code, const WallData<R>& wd, R acc[10]) {
     acc[4] = wd.uw[0] * acc[1] + wd.uw[1] * acc[2] + wd.uw[2] * acc[3];
     acc[9] = wd.uw[0] * acc[6] + wd.uw[1] * acc[7] + wd.uw[2] * acc[8];
   }
-}
-
-// Time integrals over [0, d] of the six coefficients of Eq. flux-1.
-template <class R>
-GKS_HD void flux1_integrals(R tau, R d, R c[6]) {
-  const R e = k_exp(k_div(-d, tau));
-  const R om = R(1) - e;
-  c[0] = d - tau * om;
-  c[1] = R(2) * tau * tau * om - tau * d * (R(1) + e);
-  c[2] = R(0.5) * d * d - tau * d + tau * tau * om;
-  c[3] = tau * om;
-  c[4] = tau * d * e - R(2) * tau * tau * om;
-  c[5] = -tau * tau * om;
 }
 
 // The ten coefficients of variable v through the accessor; accessors over device memory

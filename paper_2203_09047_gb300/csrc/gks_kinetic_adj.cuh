@@ -1,11 +1,11 @@
-// Reverse-mode (vector-Jacobian) companion of gks_kinetic.cuh: the boundary treatment, the frame
-// rotation and the polynomial evaluation around the Gauss-point flux, reversed by hand in the
-// reverse order of the forward code; the flux itself is reversed in gks_kinetic_rev.cuh.
+// Reverse-mode (vector-Jacobian) companion of gks_kinetic.cuh: the boundary treatment and the
+// polynomial evaluation around the Gauss-point flux, reversed by hand in the reverse order of
+// the forward code; the flux itself is reversed in gks_flux_rev.cuh.
 // Forward intermediates are recomputed (no tape).
 #pragma once
 
 #include "gks_kinetic.cuh"
-#include "gks_kinetic_rev.cuh"
+#include "gks_flux_rev.cuh"
 
 namespace gks {
 
@@ -171,80 +171,6 @@ GKS_HD void wall_ghost_vjp(const FluxParams<R>& P, int code, const WallData<R>& 
 #pragma unroll
     for (int a = 0; a < 3; ++a) gv[1 + a] += R(2) * ir * (Dm[a] - U[a] * D0);
   }
-}
-
-// Vector-Jacobian product of gp_flux_global: gacc[10] -> cotangents of vl, gl, vr, gr
-// (accumulated).
-template <class R>
-GKS_HD bool gp_flux_global_vjp(const FluxParams<R>& P, const R vl[5], const R gl[5][3],
-                               const R vr[5], const R gr[5][3], const R n1[3], R w, R dt,
-                               const R gacc[10], R gvl[5], R ggl[5][3], R gvr[5], R ggr[5][3]) {
-  int kk = 0;
-  if (k_abs(n1[1]) < k_abs(n1[kk])) kk = 1;
-  if (k_abs(n1[2]) < k_abs(n1[kk])) kk = 2;
-  R n2[3];
-  if (kk == 0) { n2[0] = R(0); n2[1] = n1[2]; n2[2] = -n1[1]; }
-  else if (kk == 1) { n2[0] = -n1[2]; n2[1] = R(0); n2[2] = n1[0]; }
-  else { n2[0] = n1[1]; n2[1] = -n1[0]; n2[2] = R(0); }
-  const R il = R(1) / k_sqrt(n2[0] * n2[0] + n2[1] * n2[1] + n2[2] * n2[2]);
-  n2[0] = n2[0] * il; n2[1] = n2[1] * il; n2[2] = n2[2] * il;
-  const R n3[3] = {n1[1] * n2[2] - n1[2] * n2[1], n1[2] * n2[0] - n1[0] * n2[2],
-                   n1[0] * n2[1] - n1[1] * n2[0]};
-  const R* nm[3] = {n1, n2, n3};
-  R ql[5], qr[5], dql[3][5], dqr[3][5];
-  ql[0] = vl[0]; ql[4] = vl[4]; qr[0] = vr[0]; qr[4] = vr[4];
-  for (int d = 0; d < 3; ++d) {
-    ql[1 + d] = vl[1] * nm[d][0] + vl[2] * nm[d][1] + vl[3] * nm[d][2];
-    qr[1 + d] = vr[1] * nm[d][0] + vr[2] * nm[d][1] + vr[3] * nm[d][2];
-  }
-  for (int d = 0; d < 3; ++d) {
-    R sl[5], sr[5];
-    for (int v = 0; v < 5; ++v) {
-      sl[v] = gl[v][0] * nm[d][0] + gl[v][1] * nm[d][1] + gl[v][2] * nm[d][2];
-      sr[v] = gr[v][0] * nm[d][0] + gr[v][1] * nm[d][1] + gr[v][2] * nm[d][2];
-    }
-    dql[d][0] = sl[0]; dql[d][4] = sl[4]; dqr[d][0] = sr[0]; dqr[d][4] = sr[4];
-    for (int e = 0; e < 3; ++e) {
-      dql[d][1 + e] = sl[1] * nm[e][0] + sl[2] * nm[e][1] + sl[3] * nm[e][2];
-      dqr[d][1 + e] = sr[1] * nm[e][0] + sr[2] * nm[e][1] + sr[3] * nm[e][2];
-    }
-  }
-  // back rotation and weight: acc = w [Fn0, sum_j Fn_j n_j, Fn4, Ft0, sum_j Ft_j n_j, Ft4]
-  R gFn[5], gFt[5];
-  gFn[0] = w * gacc[0];
-  gFn[4] = w * gacc[4];
-  gFt[0] = w * gacc[5];
-  gFt[4] = w * gacc[9];
-  for (int j = 0; j < 3; ++j) {
-    gFn[1 + j] = w * (gacc[1] * nm[j][0] + gacc[2] * nm[j][1] + gacc[3] * nm[j][2]);
-    gFt[1 + j] = w * (gacc[6] * nm[j][0] + gacc[7] * nm[j][1] + gacc[8] * nm[j][2]);
-  }
-  R gql[5] = {R(0), R(0), R(0), R(0), R(0)}, gqr[5] = {R(0), R(0), R(0), R(0), R(0)};
-  R gdql[3][5], gdqr[3][5];
-  for (int d = 0; d < 3; ++d)
-    for (int v = 0; v < 5; ++v) gdql[d][v] = gdqr[d][v] = R(0);
-  if (!gks_gp_flux_vjp_cf(P, ql, dql, qr, dqr, dt, gFn, gFt, gql, gdql, gqr, gdqr)) return false;
-  // rotation into the local frame, reversed
-  gvl[0] += gql[0]; gvl[4] += gql[4]; gvr[0] += gqr[0]; gvr[4] += gqr[4];
-  for (int d = 0; d < 3; ++d)
-    for (int a = 0; a < 3; ++a) {
-      gvl[1 + a] += gql[1 + d] * nm[d][a];
-      gvr[1 + a] += gqr[1 + d] * nm[d][a];
-    }
-  for (int d = 0; d < 3; ++d) {
-    R gsl[5], gsr[5];
-    gsl[0] = gdql[d][0]; gsl[4] = gdql[d][4]; gsr[0] = gdqr[d][0]; gsr[4] = gdqr[d][4];
-    for (int b = 0; b < 3; ++b) {
-      gsl[1 + b] = gdql[d][1] * nm[0][b] + gdql[d][2] * nm[1][b] + gdql[d][3] * nm[2][b];
-      gsr[1 + b] = gdqr[d][1] * nm[0][b] + gdqr[d][2] * nm[1][b] + gdqr[d][3] * nm[2][b];
-    }
-    for (int v = 0; v < 5; ++v)
-      for (int a = 0; a < 3; ++a) {
-        ggl[v][a] += gsl[v] * nm[d][a];
-        ggr[v][a] += gsr[v] * nm[d][a];
-      }
-  }
-  return true;
 }
 
 // Adjoint of eval_poly: cotangents of value and gradient at offset d -> cotangents of the ten
