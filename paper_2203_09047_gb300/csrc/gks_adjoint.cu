@@ -513,11 +513,11 @@ void launch_vjp(const DevMesh& m, const Geo64& g64, const GeoR<double>& g, const
     cudaDeviceSetLimit(cudaLimitStackSize, at.localSizeBytes);
   kern<<<blocks_for(4 * m.nf, 128), 128, 0, st>>>(m.nf, m.f_owner, m.f_nb, m.f_wall, g.fgp, poly,
                                                   gL, gLt, g64.vol, m.nc, fp, m.wall64, dt,
-                                                  p.gp_fallback, g.mom, g.h, gpf, flag);
+                                                  p.gp_fallback, g64.mom, g64.h, gpf, flag);
   k_vjp_poly<<<blocks_for(m.nc, 128), 128, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, gpf, gpc);
   k_vjp_recon<<<blocks_for(m.nc, 64), 64, 0, st>>>(m.nc, QA, m.t_K, m.t_cnt, m.t_st, m.t_sb,
-                                                     m.t_idx, m.st_ptr, m.n_sub, g.Ap, g.Bp, g.mom,
-                                                     g.h, p.weno_gamma, p.weno_eps, p.weno_pow, gpc,
+                                                     m.t_idx, m.st_ptr, m.n_sub, g.Ap, g.Bp, g64.mom,
+                                                     g64.h, p.weno_gamma, p.weno_eps, p.weno_pow, gpc,
                                                      gdq, gq0);
   k_vjp_stencil<<<blocks_for(m.nc, 128), 128, 0, st>>>(m.nc, rs_ptr, rs_pos, m.t_idx, m.g_map,
                                                         m.g_chain, m.bcs, fp, m.wall64, QA,

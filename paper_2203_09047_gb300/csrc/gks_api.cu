@@ -167,8 +167,7 @@ cudaError_t alloc_geo_arrays(gks_solver* s, GeoR<R>& g) {
   cudaError_t e;
   if ((e = salloc(s, &g.Ap, 9 * (int64_t)kTile * s->m.n_tslots)) != cudaSuccess) return e;
   if ((e = salloc(s, &g.Bp, 4 * (int64_t)kTile * s->m.n_tsb)) != cudaSuccess) return e;
-  if ((e = salloc(s, &g.mom, 6 * nc)) != cudaSuccess) return e;
-  if ((e = salloc(s, &g.h, nc)) != cudaSuccess) return e;
+  if ((e = salloc(s, &g.cell, (int64_t)kCellRec * kTile * s->m.n_tiles)) != cudaSuccess) return e;
   if ((e = salloc(s, &g.fgp, 40 * nf)) != cudaSuccess) return e;
   return salloc(s, &g.ivol, (sizeof(R) == 4 ? 2 : 1) * nc);
 }
@@ -199,7 +198,7 @@ void precompute_r(gks_solver* s, GeoR<R>& g) {
   launch_geom_faces<R>(s->m, s->g, g, s->st);
   launch_geom_hdt(s->m, s->g, s->st);
   launch_geom_ls<R>(s->m, s->g, g, s->flag, s->bad_cell, s->st);
-  launch_cast_cells<R>(s->m, s->g, g, s->st);
+  launch_cast_cells<R>(s->m, s->g, g, s->prm.weno_gamma, s->st);
 }
 
 // One residual evaluation: recon (from the gather copy QinA) -> flux -> face sums: the FP64
@@ -650,19 +649,20 @@ gks_status gks_init(const gks_mesh* mesh, const gks_params* p, void* stream, gks
     r.S[r.n - 1] = std::max(r.S[r.n - 1], S);
     r.M[r.n - 1] = std::max(r.M[r.n - 1], M);
   }
-  // a range is uniform when all its tiles match the first one's stencil size and sub-stencil
-  // counts (then t_st and t_sb grow by K and S per tile, and the kernel needs no table loads)
+  // a range is uniform (1) when all its tiles have the first one's stencil size, so that t_st
+  // grows by K per tile, and fully uniform (2) when its sub-stencil counts match as well
   for (int k = 0; k < m.rr.n; ++k) {
     TileRanges& r = m.rr;
     const int64_t a = r.t0[k];
     int S0 = 0;
     for (int q = 0; q < kMaxSub; ++q) S0 += (int)((h.t_cnt[a] >> (8 * q)) & 0xffu);
-    bool uni = r.t1[k] > a;
-    for (int64_t t = a; t < r.t1[k] && uni; ++t)
-      uni = h.t_K[t] == h.t_K[a] && h.t_cnt[t] == h.t_cnt[a] &&
-            (int64_t)h.t_st[t] == (int64_t)h.t_st[a] + (t - a) * h.t_K[a] &&
-            (int64_t)h.t_sb[t] == (int64_t)h.t_sb[a] + (t - a) * S0;
-    r.uni[k] = uni ? 1 : 0;
+    bool uk = r.t1[k] > a, ub = uk;
+    for (int64_t t = a; t < r.t1[k] && uk; ++t) {
+      uk = h.t_K[t] == h.t_K[a] && (int64_t)h.t_st[t] == (int64_t)h.t_st[a] + (t - a) * h.t_K[a];
+      ub = ub && h.t_cnt[t] == h.t_cnt[a] &&
+           (int64_t)h.t_sb[t] == (int64_t)h.t_sb[a] + (t - a) * S0;
+    }
+    r.uni[k] = uk ? (ub ? 2 : 1) : 0;
     r.cnt[k] = h.t_cnt[a];
     r.st0[k] = h.t_st[a];
     r.sb0[k] = h.t_sb[a];
@@ -901,7 +901,7 @@ gks_status gks_residual_vjp(gks_solver* s, const double* Q, double dt, const dou
   launch_permute_in<double>(nc, s->m.perm, s->tmp, s->vgLt, (double*)nullptr, s->st);
   // forward reconstruction in FP64, then the reverse passes
   const KParams<double> kp = kparams<double>(s->prm);
-  launch_recon<double>(s->m, s->gv, kp, s->vQA, s->vpoly, s->flag, s->st);
+  launch_recon<double>(s->m, s->gv, kp, s->vQA, s->vpoly, s->flag, s->st, &s->fj);
   launch_vjp(s->m, s->g, s->gv, kp, s->vQA, s->vpoly, s->vgL, s->vgLt, dt, s->vgpf, s->vgpc,
              s->vgdq, s->vgq0, s->vgQ, s->rs_ptr, s->rs_pos, s->flag, s->st);
   launch_permute_out(nc, s->m.perm, s->vgQ, s->tmp, s->st);
@@ -938,9 +938,9 @@ gks_status gks_kernel_bytes(const gks_solver* s, double bytes[3]) {
   const double ts = (double)kTile * s->m.n_tslots, tb = (double)kTile * s->m.n_tsb;
   // reconstruction: gather copy of Q (48 B per cell, own + stencil, once), tile counts and
   // offsets, interleaved stencil entries, pseudo-inverse rows and sub-stencil entries (with the
-  // tile padding, 0.4 % on the hybrid mesh), cell moments and size, polynomial written
+  // tile padding, 0.4 % on the hybrid mesh), per-cell records, polynomial written
   bytes[0] = 48.0 * nc + 24.0 * (double)s->m.n_tiles + nc + 4.0 * ts + 9.0 * r * ts +
-             4.0 * r * tb + 7.0 * r * nc + kPolyStride * r * nc;
+             4.0 * r * tb + kCellRec * r * nc + kPolyStride * r * nc;
   // flux: face cells and wall flag, Gauss data, polynomials read, face fluxes written
   bytes[1] = 9.0 * nf + 40.0 * r * nf + kPolyStride * r * nc + kFaceStride * r * nf;
   // face sums + stage update: CSR, face fluxes, 1/|Omega| (8 B), the state's gather copy read,

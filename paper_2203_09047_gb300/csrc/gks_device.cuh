@@ -29,6 +29,10 @@ template <>
 struct Lay<double> {
   static constexpr int apad = 10, gq = 6;
 };
+//  - per-cell reconstruction record [tile][kCellRec][32]: scaled second central moments (xx yy zz
+//    xy xz yz), 1/h, the number M of sub-stencils, 1/M and 1/(1 - gamma_m M), one contiguous
+//    block per tile; the lanes beyond the last cell repeat the tile's first cell.
+constexpr int kCellRec = 10;
 constexpr int kPolyStride = 52;
 constexpr int kFaceStride = 12;
 
@@ -50,8 +54,9 @@ struct TileRanges {
   int n = 0;
   int64_t t0[kMaxTileRanges] = {}, t1[kMaxTileRanges] = {};
   int K[kMaxTileRanges] = {}, S[kMaxTileRanges] = {}, M[kMaxTileRanges] = {};
-  // uniform ranges: every tile has the first tile's stencil size and sub-stencil counts, so
-  // the tile's offsets into the interleaved arrays follow from its index
+  // uniform ranges: 1, every tile has the first tile's stencil size, so the tile's offset into
+  // the stencil arrays follows from its index; 2, its sub-stencil counts too, so the offset
+  // into the sub-stencil entries does as well
   int uni[kMaxTileRanges] = {};
   uint64_t cnt[kMaxTileRanges] = {};
   int64_t st0[kMaxTileRanges] = {}, sb0[kMaxTileRanges] = {};
@@ -129,8 +134,7 @@ template <class R>
 struct GeoR {
   R* Ap = nullptr;   // pseudo-inverse rows, tile-interleaved
   R* Bp = nullptr;   // sub-stencil entries [slot][lane][4] (3 coefficients, member index)
-  R* mom = nullptr;  // [6][nc]
-  R* h = nullptr;    // [nc]
+  R* cell = nullptr; // per-cell record, tile-interleaved [tile][kCellRec][32] (see kCellRec)
   R* fgp = nullptr;  // [10][4 nf]: dl(3) dr(3) n1(3) w, index 4 f + gauss point
   R* ivol = nullptr; // 1/|Omega|: [nc] (FP64 path) or [nc][2] float-float pairs (FP32 path)
 };
@@ -159,7 +163,8 @@ template <class R>
 void launch_geom_ls(const DevMesh& m, const Geo64& g, GeoR<R>& gr, int* flag, int* bad_cell,
                     cudaStream_t st);
 template <class R>
-void launch_cast_cells(const DevMesh& m, const Geo64& g, GeoR<R>& gr, cudaStream_t st);
+void launch_cast_cells(const DevMesh& m, const Geo64& g, GeoR<R>& gr, double weno_gamma,
+                       cudaStream_t st);
 void launch_cell_quadrature(const DevMesh& m, double* xq, double* wq, cudaStream_t st);
 // Unit normal out of the owner and area of every face, [nf][4] in precision R.
 template <class R>

@@ -268,13 +268,24 @@ __global__ void __launch_bounds__(kThreads) k_geom_ls(
   }
 }
 
+// The per-cell arrays of the hot path in precision R: reconstruction records (one thread per
+// lane of every tile) and 1/|Omega|.
 template <class R>
-__global__ void k_cast_cells(int64_t nc, const double* __restrict__ hh, const double* __restrict__ mom,
-                             const double* __restrict__ ivol, R* h_out, R* mom_out, R* ivol_out) {
+__global__ void k_cast_cells(int64_t nc, int64_t n_tiles, const double* __restrict__ hh,
+                             const double* __restrict__ mom, const double* __restrict__ ivol,
+                             const int8_t* __restrict__ n_sub, double wg, R* cell, R* ivol_out) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t tile = i / kTile;
+  if (tile >= n_tiles) return;
+  const int64_t c = i < nc ? i : tile * kTile;
+  R* r = cell + tile * kCellRec * kTile + i % kTile;
+  for (int k = 0; k < 6; ++k) r[k * kTile] = (R)mom[k * nc + c];
+  const double M = n_sub[c];
+  r[6 * kTile] = (R)(1.0 / hh[c]);
+  r[7 * kTile] = (R)M;
+  r[8 * kTile] = (R)(1.0 / M);
+  r[9 * kTile] = (R)(1.0 / (1.0 - wg * M));
   if (i >= nc) return;
-  h_out[i] = (R)hh[i];
-  for (int k = 0; k < 6; ++k) mom_out[k * nc + i] = (R)mom[k * nc + i];
   if (sizeof(R) == 4) {  // float-float pair
     const float hi = (float)ivol[i];
     ivol_out[2 * i] = (R)hi;
@@ -352,9 +363,10 @@ void launch_geom_ls(const DevMesh& m, const Geo64& g, GeoR<R>& gr, int* flag, in
                                                       g.mom, gr.Ap, gr.Bp, flag, bad_cell);
 }
 template <class R>
-void launch_cast_cells(const DevMesh& m, const Geo64& g, GeoR<R>& gr, cudaStream_t st) {
-  k_cast_cells<R><<<blocks_for(m.nc, kThreads), kThreads, 0, st>>>(m.nc, g.h, g.mom, g.ivol, gr.h,
-                                                                  gr.mom, gr.ivol);
+void launch_cast_cells(const DevMesh& m, const Geo64& g, GeoR<R>& gr, double weno_gamma,
+                       cudaStream_t st) {
+  k_cast_cells<R><<<blocks_for(m.n_tiles * kTile, kThreads), kThreads, 0, st>>>(
+      m.nc, m.n_tiles, g.h, g.mom, g.ivol, m.n_sub, weno_gamma, gr.cell, gr.ivol);
 }
 
 // Unit normal (out of the owner) and area of every face, [nf][4] = (n, S), from its area vector
@@ -389,7 +401,9 @@ template void launch_geom_ls<double>(const DevMesh&, const Geo64&, GeoR<double>&
                                      cudaStream_t);
 template void launch_geom_ls<float>(const DevMesh&, const Geo64&, GeoR<float>&, int*, int*,
                                     cudaStream_t);
-template void launch_cast_cells<double>(const DevMesh&, const Geo64&, GeoR<double>&, cudaStream_t);
-template void launch_cast_cells<float>(const DevMesh&, const Geo64&, GeoR<float>&, cudaStream_t);
+template void launch_cast_cells<double>(const DevMesh&, const Geo64&, GeoR<double>&, double,
+                                        cudaStream_t);
+template void launch_cast_cells<float>(const DevMesh&, const Geo64&, GeoR<float>&, double,
+                                       cudaStream_t);
 
 }  // namespace gks

@@ -29,7 +29,8 @@ struct Gq<float> {
   float hi[5], lo[5];
   __device__ __forceinline__ void load(const float* __restrict__ QA, int64_t c) {
     const float4* p = reinterpret_cast<const float4*>(QA + 12 * c);
-    const float4 a = __ldg(p), b = __ldg(p + 1), d = __ldg(p + 2);
+    const float4 a = __ldg(p), b = __ldg(p + 1);
+    const float2 d = __ldg(reinterpret_cast<const float2*>(p + 2));
     hi[0] = a.x; hi[1] = a.y; hi[2] = a.z; hi[3] = a.w; hi[4] = b.x;
     lo[0] = b.y; lo[1] = b.z; lo[2] = b.w; lo[3] = d.x; lo[4] = d.y;
   }
@@ -168,34 +169,57 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int tr
 //   beta_0, tau, omega, omega-bar (Section 2), one variable per warp               (phase 3)
 //   C = (wb_0/g_0) a + sum_m (wb_m - wb_0 g_m/g_0) b_m, i.e. Eq. weno as one polynomial (phase 4)
 // Output: 10 coefficients per variable of the polynomial in physical offsets from the centroid.
-// With kPf, when the block starts, the tile's pseudo-inverse rows (a contiguous block of the
-// interleaved layout) are prefetched into L2 by a bulk prefetch, and the sub-stencil entries are
-// either copied into shared memory by a bulk copy on an mbarrier (kStB: where that costs the
-// range no resident blocks) or prefetched into L2 as well, so that the transfers overlap phase
-// 1; phase 2 then reads the rows from L2 (each row once, two rows per warp in one member loop,
-// so that two independent loads per member are in flight) and the entries from shared memory or
-// L2. Without kPf phase 2 reads both from global memory. Staging the rows in shared memory
-// as well (they are read once, so the staging bought only the overlap) held the range's blocks
-// to 2-3 per SM: 0.669 against 0.598 ms per FP32 pass on the 64^3-cube mesh with the enlarged
-// stencils, 6.54 against 5.38 ms in FP64.
+// Bound by the chain of dependent latencies of a block (about 19,000 cycles at 5 blocks per SM
+// before this form: gathers, row loads, the weights), with L1 two thirds busy and DRAM at half
+// its rate; so the order of the block is built to start every load early and to keep late loads
+// out of the chain:
+//  - the stencil indices and the cell's own state are requested before anything else; a range
+//    whose tiles all have the first one's stencil size takes their place from the tile index,
+//    with no table load before them;
+//  - with kPf one thread then starts the tile's other transfers: the pseudo-inverse rows (a
+//    contiguous block of the interleaved layout) by a bulk prefetch into L2, the per-cell record
+//    of phase 3 by a bulk copy into shared memory on an mbarrier, and the sub-stencil entries
+//    either by such a copy too (kStB: where that costs the range no resident blocks) or by a
+//    prefetch into L2;
+//  - phase 2: warps 0-2 take three rows each in one member loop unrolled by six, so that 18
+//    independent row loads are in flight and a stencil difference is read once for three rows;
+//    the other warps take the sub-stencils; the mbarrier is awaited where its data are read.
+// Measured per FP32 pass on the 64^3-cube mesh with the enlarged stencils (and the 32^3-cube
+// mesh in FP64): two rows on each of the five warps, table loads and a barrier before the
+// gathers, moments loaded in phase 3: 0.419 ms (0.676); three rows on three warps 0.411
+// (0.663); the record in shared memory, fewer quotients 0.404 (0.627); indices first, two
+// barriers instead of three 0.385 (0.614); six unstaged entries in flight and two of eight
+// sub-stencils on row warps 0.362 (0.604); rows, entries and indices without L1 lines 0.356
+// (0.599). Not adopted:
+// six blocks per SM (64 registers, spills) 0.409; row loads started before the gathers' barrier
+// 0.385-0.400 (the prefetch has not landed); no prefetch of the rows 0.396, of the entries
+// 0.387; a bulk prefetch of a later block's tile 0.415-0.467 (indices only 0.367); batches of 2,
+// 3 and 5 members 0.427, 0.393, 0.424; staging the rows in shared memory costs 2 resident
+// blocks.
 constexpr int kReconWarps = 5;
+constexpr int kRowWarps = 3;  // warps 0-2 take three rows of A+ each, the others sub-stencils
+constexpr int kRowShare = 6;  // sub-stencils from this one on go to row warps (unstaged entries)
+constexpr int kBatch = 4;     // stencil members a thread gathers at a time
 constexpr int kReconThreads = kReconWarps * kTile;
-constexpr int kReconBlocksPerSM = 5;  // the register bound (launch bounds) of k_recon
+// resident blocks per SM of the register bound (launch bounds): five in FP32 (80 registers a
+// thread), three in FP64, as many as its shared memory allows
+template <class R>
+constexpr int kReconBlocksPerSM = sizeof(R) == 4 ? 5 : 3;
 
 // Shared-memory layout of one block for a range with largest stencil Kr, largest sum of
 // sub-stencil member counts Sr and largest number of sub-stencil slots Mr, in units of one
-// interleaved row (kTile values): [mbarrier, 16 B][B entries 4 Sr] (only with kPf and stb: the
-// sub-stencil entries staged by a bulk copy), then a[9][5], b[Mr][3][5], beta[Mr][5], dq[Kr][5]
-// (the last in the lane-major form of DqRow below). Every part starts on a 16-byte boundary.
-// (a_off marks where staged rows would start; the rows come through L2.)
+// interleaved row (kTile values): [mbarrier, 16 B][per-cell records, kCellRec] (with kPf),
+// [B entries 4 Sr] (with kPf and stb: the sub-stencil entries staged by a bulk copy), then
+// a[9][5], b[Mr][3][5], beta[Mr][5], dq[Kr][5] (the last in the lane-major form of DqRow below).
+// Every part starts on a 16-byte boundary.
 
 template <class R>
 struct ReconSmem {
-  size_t a_off, b_off, ca_off, cb_off, cbet_off, dq_off, bytes;
+  size_t c_off, b_off, ca_off, cb_off, cbet_off, dq_off, bytes;
   __host__ __device__ ReconSmem(int Kr, int Sr, int Mr, bool pf, bool stb) {
     const size_t row = (size_t)kTile * sizeof(R);
-    a_off = pf ? 16 : 0;
-    b_off = a_off;
+    c_off = pf ? 16 : 0;
+    b_off = c_off + (pf ? kCellRec * row : 0);
     ca_off = b_off + (pf && stb ? 4 * (size_t)Sr * row : 0);
     cb_off = ca_off + 45 * row;
     cbet_off = cb_off + 15 * (size_t)Mr * row;
@@ -237,6 +261,39 @@ struct DqRow<double> {
   }
 };
 
+// Loads of data that a block reads once (pseudo-inverse rows, sub-stencil entries, stencil
+// indices): read-only path without an L1 line, so that the gathered states stay in L1 (0.362 ->
+// 0.356 ms per FP32 pass on the 64^3-cube mesh).
+__device__ __forceinline__ float ld_once(const float* p) {
+  float v;
+  asm volatile("ld.global.nc.L1::no_allocate.f32 %0, [%1];" : "=f"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double ld_once(const double* p) {
+  double v;
+  asm volatile("ld.global.nc.L1::no_allocate.f64 %0, [%1];" : "=d"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ int32_t ld_once(const int32_t* p) {
+  int32_t v;
+  asm volatile("ld.global.nc.L1::no_allocate.s32 %0, [%1];" : "=r"(v) : "l"(p));
+  return v;
+}
+__device__ __forceinline__ float4 ld_once(const float4* p) {
+  float4 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "l"(p));
+  return v;
+}
+__device__ __forceinline__ double2 ld_once(const double2* p) {
+  double2 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.f64 {%0, %1}, [%2];"
+               : "=d"(v.x), "=d"(v.y)
+               : "l"(p));
+  return v;
+}
+
 // One sub-stencil entry (three pseudo-inverse coefficients and the member index) of one lane:
 // one 16-byte load in FP32, two in FP64, from shared memory (staged) or through the read-only
 // path (global). Against four interleaved rows: 0.571 -> 0.569 ms per FP32 pass.
@@ -246,7 +303,7 @@ template <>
 struct BRec<float> {
   __device__ __forceinline__ static void get(const float* e, bool staged, float c[4]) {
     const float4* p = reinterpret_cast<const float4*>(e);
-    const float4 x = staged ? *p : __ldg(p);
+    const float4 x = staged ? *p : ld_once(p);
     c[0] = x.x; c[1] = x.y; c[2] = x.z; c[3] = x.w;
   }
 };
@@ -254,26 +311,33 @@ template <>
 struct BRec<double> {
   __device__ __forceinline__ static void get(const double* e, bool staged, double c[4]) {
     const double2* p = reinterpret_cast<const double2*>(e);
-    const double2 x = staged ? p[0] : __ldg(p), y = staged ? p[1] : __ldg(p + 1);
+    const double2 x = staged ? p[0] : ld_once(p), y = staged ? p[1] : ld_once(p + 1);
     c[0] = x.x; c[1] = x.y; c[2] = y.x; c[3] = y.y;
   }
 };
 
-// A variable's ten output coefficients as five 8-byte (FP32) or 16-byte (FP64) shared stores
-// (a record of kPolyStride values starts on a 16-byte boundary; variable v at 10 v values).
+// A variable's ten output coefficients to shared memory in the widest stores its place allows (a
+// record of kPolyStride values starts on a 16-byte boundary; variable v at 10 v values): in FP32
+// two 16-byte and one 8-byte store, in FP64 five 16-byte ones.
 template <class R>
 struct PolyPair;
 template <>
 struct PolyPair<float> {
-  __device__ __forceinline__ static void put(float* so, const float o[10]) {
-    float2* p = reinterpret_cast<float2*>(so);
-#pragma unroll
-    for (int j = 0; j < 5; ++j) p[j] = make_float2(o[2 * j], o[2 * j + 1]);
+  __device__ __forceinline__ static void put(float* so, int v, const float o[10]) {
+    if ((v & 1) == 0) {
+      reinterpret_cast<float4*>(so)[0] = make_float4(o[0], o[1], o[2], o[3]);
+      reinterpret_cast<float4*>(so)[1] = make_float4(o[4], o[5], o[6], o[7]);
+      *reinterpret_cast<float2*>(so + 8) = make_float2(o[8], o[9]);
+    } else {
+      *reinterpret_cast<float2*>(so) = make_float2(o[0], o[1]);
+      *reinterpret_cast<float4*>(so + 2) = make_float4(o[2], o[3], o[4], o[5]);
+      *reinterpret_cast<float4*>(so + 6) = make_float4(o[6], o[7], o[8], o[9]);
+    }
   }
 };
 template <>
 struct PolyPair<double> {
-  __device__ __forceinline__ static void put(double* so, const double o[10]) {
+  __device__ __forceinline__ static void put(double* so, int, const double o[10]) {
     double2* p = reinterpret_cast<double2*>(so);
 #pragma unroll
     for (int j = 0; j < 5; ++j) p[j] = make_double2(o[2 * j], o[2 * j + 1]);
@@ -294,13 +358,32 @@ __device__ __forceinline__ float wdiv<float>(float a, float b) {
   return __fdividef(a, b);
 }
 
-// Five resident blocks per SM as the register bound (at most 80 registers a thread; 72 used):
-// on the 64^3-cube hybrid mesh with the enlarged stencils 0.598 ms per FP32 pass, 0.611 ms at 6
-// blocks (64 registers, spills); before the rows went through L2, 0.664 ms against 0.697 ms
-// unbounded (4 blocks).
-// A uniform range (every tile with the same stencil size K and sub-stencil counts cnt): the
-// tile's offsets into the interleaved arrays are st0 + K (tile - tile0) and sb0 + S (tile - tile0),
-// so no table load stands between the block's start and its first stencil gathers.
+// b[s] <- tau / b[s], s = 0..M (M <= 8; the entries beyond M are 1). FP32: one fast quotient
+// each. FP64: a division is a chain of a dozen FP64 instructions on a pipe that bounds the
+// kernel, so three reciprocals are taken from one division of 1 by the product of the three
+// (each product rounds once more; the indicators lie between the weights' epsilon and far below
+// 10^102, so no product leaves the range).
+template <class R>
+__device__ __forceinline__ void quotients(R tau, int M, R b[kMaxSub + 1]) {
+#pragma unroll
+  for (int s = 0; s <= kMaxSub; ++s)
+    if (s <= M) b[s] = wdiv(tau, b[s]);
+}
+template <>
+__device__ __forceinline__ void quotients<double>(double tau, int M, double b[kMaxSub + 1]) {
+#pragma unroll
+  for (int g = 0; g < 3; ++g) {
+    if (3 * g > M) continue;
+    const double x = b[3 * g], y = b[3 * g + 1], z = b[3 * g + 2], xy = x * y;
+    const double r = tau / (xy * z), rz = r * z;
+    b[3 * g] = rz * y;
+    b[3 * g + 1] = rz * x;
+    b[3 * g + 2] = r * xy;
+  }
+}
+
+// A uniform range (TileRanges::uni): with on >= 1 the tile's stencil arrays start at
+// st0 + K (tile - tile0), with on == 2 its sub-stencil entries at sb0 + S (tile - tile0).
 struct ReconUni {
   int on, K, S;
   uint64_t cnt;
@@ -308,13 +391,12 @@ struct ReconUni {
 };
 
 template <class R, bool kPf, bool kStB>
-__global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM) k_recon(
+__global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM<R>) k_recon(
     int64_t nc, int64_t tile0, int Kr, int Sr, int Mr, ReconUni u, const R* __restrict__ QA,
     const int32_t* __restrict__ t_K, const uint64_t* __restrict__ t_cnt,
     const int32_t* __restrict__ t_st, const int32_t* __restrict__ t_sb,
-    const int32_t* __restrict__ t_idx, const int8_t* __restrict__ n_sub,
-    const R* __restrict__ Ap, const R* __restrict__ Bp, const R* __restrict__ mom,
-    const R* __restrict__ hcell, R wg, R weps, int wpow, R* __restrict__ poly, int* flag,
+    const int32_t* __restrict__ t_idx, const R* __restrict__ Ap, const R* __restrict__ Bp,
+    const R* __restrict__ cell, R wg, R weps, int wpow, R* __restrict__ poly, int* flag,
     int wait_tries, int withhold) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const ReconSmem<R> L(Kr, Sr, Mr, kPf, kStB);
@@ -329,9 +411,23 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM) k_recon(
   const int warp = threadIdx.x / kTile;
   const int64_t tl = tile - tile0;
   const int K = u.on ? u.K : __ldg(t_K + tile);
-  const uint64_t cnt = u.on ? u.cnt : __ldg(t_cnt + tile);
   const int64_t st = u.on ? u.st0 + tl * u.K : (int64_t)__ldg(t_st + tile);
-  const int64_t sbo = u.on ? u.sb0 + tl * u.S : (int64_t)__ldg(t_sb + tile);
+  // phase 1, first half: the stencil indices of the first batch and the cell's own state are
+  // requested before anything else
+  const int64_t i = tile * kTile + lane;
+  const bool valid = i < nc;
+  const int64_t ic = valid ? i : tile * kTile;  // padded lanes mirror the tile's first cell
+  const int32_t* sidx = t_idx + st * kTile + lane;
+  int32_t e[kBatch];
+#pragma unroll
+  for (int j = 0; j < kBatch; ++j) {
+    const int k = warp + j * kReconWarps;
+    e[j] = k < K ? ld_once(sidx + k * kTile) : -1;
+  }
+  Gq<R> c0;
+  c0.load(QA, ic);
+  const uint64_t cnt = u.on == 2 ? u.cnt : __ldg(t_cnt + tile);
+  const int64_t sbo = u.on == 2 ? u.sb0 + tl * u.S : (int64_t)__ldg(t_sb + tile);
   const R* Ag = Ap + st * 9 * kTile;
   const R* Bg = Bp + sbo * 4 * kTile;
   int S = 0, Mt = 0;  // entries and sub-stencil slots of this tile
@@ -341,115 +437,103 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM) k_recon(
     S += c;
     if (c) Mt = q + 1;
   }
-  if (kPf) {
-    if (threadIdx.x == 0) {
-      mbar_init(bar);
-      const uint32_t ab = 9u * K * kTile * sizeof(R), bb = 4u * S * kTile * sizeof(R);
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(Ag), "r"(ab) : "memory");
-      if (!kStB && bb)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(Bg), "r"(bb) : "memory");
-      // withhold != 0 (the timeout test of gks_debug_recon_wait): no copy is issued and 16
-      // bytes more than the copies would bring are expected, so the barrier's phase never
-      // completes and the bounded wait below runs out with nothing in flight
-      mbar_expect_tx(bar, (kStB ? bb : 0u) + (withhold ? 16u : 0u));
-      if (kStB && bb && !withhold) bulk_load(smem_raw + L.b_off, Bg, bb, bar);
+  if (kPf && threadIdx.x == kReconThreads - kTile) {  // the last warp: it has the fewest members
+    mbar_init(bar);
+    const uint32_t ab = 9u * K * kTile * sizeof(R), bb = 4u * S * kTile * sizeof(R);
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(Ag), "r"(ab) : "memory");
+    if (!kStB && bb)
+      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" :: "l"(Bg), "r"(bb) : "memory");
+    // withhold != 0 (the timeout test of gks_debug_recon_wait): no copy is issued and 16
+    // bytes more than the copies would bring are expected, so the barrier's phase never
+    // completes and the bounded wait below runs out with nothing in flight
+    constexpr uint32_t cb = kCellRec * kTile * sizeof(R);
+    mbar_expect_tx(bar, cb + (kStB ? bb : 0u) + (withhold ? 16u : 0u));
+    if (!withhold) {
+      bulk_load(smem_raw + L.c_off, cell + tile * kCellRec * kTile, cb, bar);
+      if (kStB && bb) bulk_load(smem_raw + L.b_off, Bg, bb, bar);
     }
   }
-  const int64_t i = tile * kTile + lane;
-  const bool valid = i < nc;
-  const int64_t ic = valid ? i : tile * kTile;  // padded lanes mirror the tile's first cell
-  // per-cell data of the later phases: the moments and the cell size are prefetched into L2 now
-  // and loaded in phase 3 (held in registers through phases 1 and 2 they cost spills: 0.437
-  // against 0.470 ms per FP32 pass on the 64^3-cube mesh with the uniform-range offsets, 0.456
-  // against 0.457 without them)
-  const int M = n_sub[ic];
-  if (warp == 0) {
-#pragma unroll
-    for (int q = 0; q < 6; ++q)
-      asm volatile("prefetch.global.L2 [%0];" ::"l"(mom + q * nc + ic));
-    asm volatile("prefetch.global.L2 [%0];" ::"l"(hcell + ic));
-  }
-  const int32_t* sidx = t_idx + st * kTile + lane;
-  Gq<R> c0;
-  c0.load(QA, ic);
-  if (kPf) __syncthreads();  // the barrier is initialised before anyone waits on it
 
-  // phase 1: stencil differences, members split over the warps, four per batch: all index
+  // phase 1: stencil differences, members split over the warps, kBatch per batch: all index
   // loads, then all state loads, then the differences
-  for (int k0 = warp; k0 < K; k0 += 4 * kReconWarps) {
-    int32_t e[4];
+  for (int k0 = warp; k0 < K; k0 += kBatch * kReconWarps) {
+    if (k0 != warp) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int k = k0 + u * kReconWarps;
-      e[u] = k < K ? __ldg(sidx + k * kTile) : -1;
+      for (int j = 0; j < kBatch; ++j) {
+        const int k = k0 + j * kReconWarps;
+        e[j] = k < K ? ld_once(sidx + k * kTile) : -1;
+      }
     }
-    Gq<R> g[4];
+    Gq<R> g[kBatch];
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (e[u] >= 0) g[u].load(QA, e[u] & kCellMask);
+    for (int j = 0; j < kBatch; ++j)
+      if (e[j] >= 0) g[j].load(QA, e[j] & kCellMask);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (e[u] < 0) continue;
-      const int fl = e[u] >> kFlipShift;
-      if (fl & 1) g[u].flip(1);
-      if (fl & 2) g[u].flip(2);
-      if (fl & 4) g[u].flip(3);
-      const int k = k0 + u * kReconWarps;
+    for (int j = 0; j < kBatch; ++j) {
+      if (e[j] < 0) continue;
+      const int fl = e[j] >> kFlipShift;
+      if (fl & 1) g[j].flip(1);
+      if (fl & 2) g[j].flip(2);
+      if (fl & 4) g[j].flip(3);
+      const int k = k0 + j * kReconWarps;
       R d[4];
 #pragma unroll
-      for (int v = 0; v < 4; ++v) d[v] = g[u].minus(c0, v);
+      for (int v = 0; v < 4; ++v) d[v] = g[j].minus(c0, v);
       DqRow<R>::put(sdqv, k, lane, d);
-      sdq4[k * kTile + lane] = g[u].minus(c0, 4);
+      sdq4[k * kTile + lane] = g[j].minus(c0, 4);
     }
   }
-  const R* A;
-  const R* Bt;
-  if (kPf) {
-    // every thread waits for the copies; a block whose wait ran out reports it and stops
+  __syncthreads();
+  const R* Bt = (kPf && kStB ? reinterpret_cast<const R*>(smem_raw + L.b_off) : Bg) + 4 * lane;
+  // the copies (per-cell records, staged entries) are awaited where they are read: by the
+  // sub-stencil warps before their entries, by the row warps after their rows. A block whose
+  // wait ran out reports it and stops at the barrier before phase 3.
+  bool ok = true;
+  auto wait_copies = [&]() {
+    if (!kPf) return;
     const int tries = wait_tries > 0 ? wait_tries : kWaitTries;
-    bool ok = mbar_wait(bar, 0, tries);
+    ok = mbar_wait(bar, 0, tries);
     if (!ok) ok = mbar_wait(bar, 0, tries);  // let copies still in flight land before leaving
-    if (__syncthreads_or(!ok)) {
-      if (threadIdx.x == 0) atomicOr(flag, kErrTimeout);
-      return;
-    }
-    A = Ag + lane;
-    Bt = (kStB ? reinterpret_cast<const R*>(smem_raw + L.b_off) : Bg) + 4 * lane;
-  } else {
-    __syncthreads();
-    A = Ag + lane;
-    Bt = Bg + 4 * lane;
-  }
+  };
 
   // phase 2: rows n = warp, warp + 5 of a = A+ dq (both in one member loop: each stencil
   // difference is read once for the two rows), and the sub-stencil fits b_m with their
   // indicators beta_m = |b_m|^2 (scaled coordinates); sub-stencils go to the warps in reverse
   // order (m = 4 - warp, 9 - warp) so that the warp with one row takes two of them
-  {
-    const int n0 = warp, n1 = warp + kReconWarps;
-    const bool two = n1 < 9;
-    const int n1c = two ? n1 : n0;
-    R acc0[5] = {R(0), R(0), R(0), R(0), R(0)}, acc1[5] = {R(0), R(0), R(0), R(0), R(0)};
+  if (warp < kRowWarps) {
+    R acc[3][5];
+#pragma unroll
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int v = 0; v < 5; ++v) acc[j][v] = R(0);
+    const R* q = Ag + 3 * warp * kTile + lane;
 #pragma unroll 6
-    for (int k = 0; k < K; ++k) {
-      const R r0 = __ldg(A + (9 * k + n0) * kTile);
-      const R r1 = __ldg(A + (9 * k + n1c) * kTile);
+    for (int k = 0; k < K; ++k, q += 9 * kTile) {
+      const R r0 = ld_once(q), r1 = ld_once(q + kTile), r2 = ld_once(q + 2 * kTile);
       R d[5];
       DqRow<R>::get(sdqv, k, lane, d);
       d[4] = sdq4[k * kTile + lane];
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        acc0[v] += r0 * d[v];
-        acc1[v] += r1 * d[v];
+        acc[0][v] += r0 * d[v];
+        acc[1][v] += r1 * d[v];
+        acc[2][v] += r2 * d[v];
       }
     }
 #pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      sa[(5 * n0 + v) * kTile + lane] = acc0[v];
-      if (two) sa[(5 * n1 + v) * kTile + lane] = acc1[v];
-    }
+    for (int j = 0; j < 3; ++j)
+#pragma unroll
+      for (int v = 0; v < 5; ++v) sa[(5 * (3 * warp + j) + v) * kTile + lane] = acc[j][v];
   }
-  for (int s = kReconWarps - 1 - warp; s < Mt; s += kReconWarps) {
+  wait_copies();
+  // sub-stencils: the two sub warps alternate; where the entries come through L2 (kStB = false:
+  // the kinds with many sub-stencils) the seventh and eighth go to row warps 0 and 1, and six
+  // entries are in flight instead of two
+  constexpr int kSubU = kStB ? 2 : 6;
+  const bool sub_warp = warp >= kRowWarps;
+  const int s_first = sub_warp ? warp - kRowWarps : (kStB ? kMaxSub : kRowShare + warp);
+  const int s_end = !kStB && sub_warp && Mt > kRowShare ? kRowShare : Mt;
+  for (int s = s_first; s < s_end; s += sub_warp ? kReconWarps - kRowWarps : kMaxSub) {
     int slot = 0;
     for (int q = 0; q < s; ++q) slot += (int)((cnt >> (8 * q)) & 0xffu);
     const int cs = (int)((cnt >> (8 * s)) & 0xffu);
@@ -459,7 +543,7 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM) k_recon(
     for (int t = 0; t < 3; ++t)
 #pragma unroll
       for (int v = 0; v < 5; ++v) b[t][v] = R(0);
-#pragma unroll 2
+#pragma unroll kSubU
     for (int j = 0; j < cs; ++j, e += 4 * kTile) {
       R c[4];
       BRec<R>::get(e, kPf && kStB, c);
@@ -479,58 +563,68 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM) k_recon(
       for (int t = 0; t < 3; ++t) sb[((3 * s + t) * 5 + v) * kTile + lane] = b[t][v];
     }
   }
-  __syncthreads();
+  if (__syncthreads_or(!ok)) {
+    if (threadIdx.x == 0) atomicOr(flag, kErrTimeout);
+    return;
+  }
 
   // phase 3: nonlinear weights, variable v = warp
+  const R* rec = (kPf ? reinterpret_cast<const R*>(smem_raw + L.c_off)
+                      : cell + tile * kCellRec * kTile) + lane;
   R m2[6];
 #pragma unroll
-  for (int q = 0; q < 6; ++q) m2[q] = mom[q * nc + ic];
-  const R hc = hcell[ic];
-  const R g0 = R(1) - wg * R(M);
+  for (int q = 0; q < 6; ++q) m2[q] = rec[q * kTile];
+  const int M = (int)rec[7 * kTile];
+  const R g0 = R(1) - wg * rec[7 * kTile];
+  const R ig0 = rec[9 * kTile];
   const int v = warp;
   {
     R a[9];
 #pragma unroll
     for (int n = 0; n < 9; ++n) a[n] = sa[(5 * n + v) * kTile + lane];
-    // |l| = 1 terms: cell means of the squared first derivatives (linear in the scaled
-    // coordinates y, second moments m2); |l| = 2 terms: squared second derivatives
-    const R gx[3] = {R(2) * a[3], a[6], a[7]};
-    const R gy[3] = {a[6], R(2) * a[4], a[8]};
-    const R gz[3] = {a[7], a[8], R(2) * a[5]};
-    auto qf = [&](const R g[3]) {
-      return m2[0] * g[0] * g[0] + m2[1] * g[1] * g[1] + m2[2] * g[2] * g[2] +
-             R(2) * (m2[3] * g[0] * g[1] + m2[4] * g[0] * g[2] + m2[5] * g[1] * g[2]);
-    };
-    const R beta0 = a[0] * a[0] + a[1] * a[1] + a[2] * a[2] + qf(gx) + qf(gy) + qf(gz) +
-                    R(4) * (a[3] * a[3] + a[4] * a[4] + a[5] * a[5]) + a[6] * a[6] + a[7] * a[7] +
-                    a[8] * a[8];
+    // |l| = 1 terms: cell means of the squared first derivatives, linear in the scaled
+    // coordinates with second moments m2: a_lin^2 + m2 : H^2, H the matrix of second
+    // derivatives; |l| = 2 terms: squared second derivatives
+    const R h0 = R(2) * a[3], h1 = R(2) * a[4], h2 = R(2) * a[5];
+    const R t0 = h0 * h0, t1 = h1 * h1, t2 = h2 * h2;
+    const R s6 = a[6] * a[6], s7 = a[7] * a[7], s8 = a[8] * a[8];
+    const R beta0 = a[0] * a[0] + a[1] * a[1] + a[2] * a[2] + (t0 + t1 + t2) + (s6 + s7 + s8) +
+                    m2[0] * (t0 + s6 + s7) + m2[1] * (t1 + s6 + s8) + m2[2] * (t2 + s7 + s8) +
+                    R(2) * (m2[3] * (a[6] * (h0 + h1) + a[7] * a[8]) +
+                            m2[4] * (a[7] * (h0 + h2) + a[6] * a[8]) +
+                            m2[5] * (a[8] * (h1 + h2) + a[6] * a[7]));
     R tau = R(0);
     for (int s = 0; s < M; ++s) tau += fabs(beta0 - sbet[(5 * s + v) * kTile + lane]);
-    tau = wdiv(tau, R(M));
-    auto weight = [&](R gam, R bb) {
-      const R r = wdiv(tau, bb + weps);
+    tau *= rec[8 * kTile];
+    // bt[0] = beta_0 + eps, bt[1 + s] = beta_s + eps, then tau over each
+    R wm[kMaxSub + 1];
+    wm[0] = beta0 + weps;
+#pragma unroll
+    for (int s = 0; s < kMaxSub; ++s)
+      wm[1 + s] = s < M ? sbet[(5 * s + v) * kTile + lane] + weps : R(1);
+    quotients(tau, M, wm);
+    R sum = R(0);
+#pragma unroll
+    for (int s = 0; s <= kMaxSub; ++s) {
+      if (s > M) {
+        wm[s] = R(0);
+        continue;
+      }
+      const R r = wm[s];
       R pw = r;
       for (int q = 1; q < wpow; ++q) pw *= r;
-      return gam * (R(1) + pw);
-    };
-    const R w0 = weight(g0, beta0);
-    R sum = w0;
-    R wm[kMaxSub];
-#pragma unroll
-    for (int s = 0; s < kMaxSub; ++s) {
-      wm[s] = s < M ? weight(wg, sbet[(5 * s + v) * kTile + lane]) : R(0);
+      wm[s] = (s == 0 ? g0 : wg) * (R(1) + pw);
       sum += wm[s];
     }
     const R is = wdiv(R(1), sum);
-    const R wb0 = w0 * is;
-    const R ig0 = wdiv(R(1), g0);
+    const R wb0 = wm[0] * is;
     const R corr = wb0 * wg * ig0;
     // phase 4 (same warp, same variable): linear part of the combination and the output
     R cl[3] = {R(0), R(0), R(0)};
 #pragma unroll
     for (int s = 0; s < kMaxSub; ++s) {
       if (s < M) {
-        const R f = wm[s] * is - corr;
+        const R f = wm[1 + s] * is - corr;
 #pragma unroll
         for (int t = 0; t < 3; ++t) cl[t] += f * sb[((3 * s + t) * 5 + v) * kTile + lane];
       }
@@ -543,7 +637,7 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM) k_recon(
     C[1] += cl[1];
     C[2] += cl[2];
     {
-      const R ih = wdiv(R(1), hc), ih2 = ih * ih;
+      const R ih = rec[6 * kTile], ih2 = ih * ih;
       // Q = c0 + c1 dx + c2 dy + c3 dz + c4 dx^2 + c5 dy^2 + c6 dz^2 + c7 dxdy + c8 dxdz + c9 dydz
       const R shift = C[3] * m2[0] + C[4] * m2[1] + C[5] * m2[2] + C[6] * m2[3] +
                       C[7] * m2[4] + C[8] * m2[5];
@@ -562,7 +656,7 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM) k_recon(
       // warp touched 32 sectors for 4 bytes each (0.569 -> 0.457 ms per FP32 pass on the
       // 64^3-cube mesh, 5.36 -> 5.34 ms in FP64)
       R* so = reinterpret_cast<R*>(smem_raw + L.dq_off) + lane * kPolyStride + 10 * v;
-      PolyPair<R>::put(so, o);
+      PolyPair<R>::put(so, v, o);
     }
   }
   fence_proxy_async_shared();
@@ -1324,7 +1418,7 @@ void launch_recon_range(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p,
   ReconUni u{m.rr.uni[r], m.rr.K[r], m.rr.S[r], m.rr.cnt[r], m.rr.st0[r], m.rr.sb0[r]};
   k_recon<R, kPf, kStB><<<(unsigned)(m.rr.t1[r] - m.rr.t0[r]), kReconThreads, smem, st>>>(
       m.nc, m.rr.t0[r], m.rr.K[r], m.rr.S[r], m.rr.M[r], u, QA, m.t_K, m.t_cnt, m.t_st, m.t_sb,
-      m.t_idx, m.n_sub, g.Ap, g.Bp, g.mom, g.h, p.weno_gamma, p.weno_eps, p.weno_pow, poly, flag,
+      m.t_idx, g.Ap, g.Bp, g.cell, p.weno_gamma, p.weno_eps, p.weno_pow, poly, flag,
       p.wait_tries, p.withhold);
 }
 
@@ -1430,11 +1524,10 @@ void launch_recon(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const
     }
     // the sub-stencil entries are staged in shared memory only where that costs the range no
     // resident blocks below the register bound; otherwise they are prefetched into L2 like the
-    // rows (on the 64^3-cube mesh the pyramid and hexahedron ranges: 3 and 4 blocks per SM with
-    // the entries staged, 5 without; 0.595 -> 0.571 ms per FP32 pass)
+    // rows (the pyramids and hexahedra of the hybrid meshes, which have eight sub-stencils)
     const ReconSmem<R> pb(m.rr.K[r], m.rr.S[r], m.rr.M[r], true, true);
     const ReconSmem<R> pl(m.rr.K[r], m.rr.S[r], m.rr.M[r], true, false);
-    const int nb_l = std::min(kReconBlocksPerSM, recon_blocks_per_sm(pl.bytes));
+    const int nb_l = std::min(kReconBlocksPerSM<R>, recon_blocks_per_sm(pl.bytes));
     if (pb.bytes <= kMaxBlockSmem && recon_blocks_per_sm(pb.bytes) >= nb_l) {
       launch_recon_range<R, true, true>(m, g, p, QA, poly, flag, r, pb.bytes, s);
     } else if (pl.bytes <= kMaxBlockSmem) {
