@@ -954,9 +954,7 @@ gks_status gks_kernel_bytes(const gks_solver* s, double bytes[3]) {
 
 gks_status gks_launches_per_pass(const gks_solver* s, int64_t launches[3]) {
   if (!s || !launches) return GKS_E_INVAL;
-  launches[0] = 0;
-  for (int r = 0; r < s->m.rr.n; ++r) launches[0] += s->m.rr.t1[r] > s->m.rr.t0[r] ? 1 : 0;
-  if (s->m.ng > 0) launches[0] += 1;  // the ghost refresh of moving no-slip walls
+  launches[0] = recon_launches(s->m);
   launches[1] = 1;
   launches[2] = 1;
   return GKS_OK;

@@ -183,6 +183,8 @@ struct ForkJoin {
 template <class R>
 void launch_recon(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* QA,
                   R* poly, int* flag, cudaStream_t st, const ForkJoin* fj = nullptr);
+// Kernel launches of one launch_recon.
+int recon_launches(const DevMesh& m);
 template <class R>
 void launch_flux(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* poly,
                  const R* QA, double dt, R* fface, int* flag, cudaStream_t st);

@@ -387,12 +387,30 @@ __device__ __forceinline__ void quotients<double>(double tau, int M, double b[kM
 struct ReconUni {
   int on, K, S;
   uint64_t cnt;
-  int64_t st0, sb0;
+  int64_t st0, sb0, tile0;
+};
+// The ranges of one launch: one range per launch on large meshes, every range in one launch on
+// small ones (launch_recon), where a block finds its range by its tile.
+struct ReconSet {
+  int n;
+  ReconUni r[kMaxTileRanges];
 };
 
-template <class R, bool kPf, bool kStB>
+__device__ __forceinline__ ReconUni range_of(const ReconUni& u, int64_t) { return u; }
+__device__ __forceinline__ ReconUni range_of(const ReconSet& set, int64_t tile) {
+  ReconUni u = set.r[0];
+#pragma unroll
+  for (int r = 1; r < kMaxTileRanges; ++r)
+    if (r < set.n && tile >= set.r[r].tile0) u = set.r[r];
+  return u;
+}
+
+// kMany: one launch over several ranges (set), else one range.
+template <class R, bool kPf, bool kStB, bool kMany>
 __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM<R>) k_recon(
-    int64_t nc, int64_t tile0, int Kr, int Sr, int Mr, ReconUni u, const R* __restrict__ QA,
+    int64_t nc, int64_t tile0, int Kr, int Sr, int Mr,
+    const __grid_constant__ std::conditional_t<kMany, ReconSet, ReconUni> set,
+    const R* __restrict__ QA,
     const int32_t* __restrict__ t_K, const uint64_t* __restrict__ t_cnt,
     const int32_t* __restrict__ t_st, const int32_t* __restrict__ t_sb,
     const int32_t* __restrict__ t_idx, const R* __restrict__ Ap, const R* __restrict__ Bp,
@@ -409,7 +427,8 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM<R>) k_recon(
   const int64_t tile = tile0 + blockIdx.x;
   const int lane = threadIdx.x & (kTile - 1);
   const int warp = threadIdx.x / kTile;
-  const int64_t tl = tile - tile0;
+  const ReconUni u = range_of(set, tile);
+  const int64_t tl = tile - (kMany ? u.tile0 : tile0);
   const int K = u.on ? u.K : __ldg(t_K + tile);
   const int64_t st = u.on ? u.st0 + tl * u.K : (int64_t)__ldg(t_st + tile);
   // phase 1, first half: the stencil indices of the first batch and the cell's own state are
@@ -845,63 +864,115 @@ __device__ __forceinline__ bool physical(const double q[5]) {
 }
 
 // Sum of the signed face fluxes of one cell (the owner loses the outward flux), in the cell's
-// fixed face order. FP64 path: FP64 sums. FP32 path: each component is accumulated as an
-// unevaluated pair hi + lo of floats with the error-free TwoSum (Knuth), so the sum is exact to
-// about 2^-48 relative without FP64 arithmetic (GB300 runs FP64 at 1/64 of the FP32 rate).
-template <class R>
-__device__ __forceinline__ void face_sums(int k0, int k1, const int32_t* __restrict__ cf_idx,
-                                          const R* __restrict__ fface, double s[10]);
-template <>
-__device__ __forceinline__ void face_sums<double>(int k0, int k1, const int32_t* __restrict__ cf_idx,
-                                                  const double* __restrict__ fface, double s[10]) {
+// fixed face order: add(q, x) for the components q = kQ0..9 of each face. A cell's chain is a
+// CSR entry, then a face record: kB of each are requested together before any is summed. On small
+// meshes the stage kernels wait on that chain (8.5 us for 2,048 cells, one face at a time), so
+// they take all faces of a cell at once (kFaceBatch; ten stage-pairs of the 8^3-cube mesh 582 ->
+// 465 us together with the merged reconstruction launch, 495 with two or five at a time); on
+// large ones occupancy is worth more (64^3 cubes, FP32: 66.5 us per stage one at a time, 70.0
+// with three), so kB = 1.
+constexpr int kFaceBatch = 6;
+template <int kQ0, int kB, class F>
+__device__ __forceinline__ void face_loop(int k0, int k1, const int32_t* __restrict__ cf_idx,
+                                          const float* __restrict__ fface, F add) {
+  for (int k = k0; k < k1; k += kB) {
+    int32_t e[kB];
+    float4 a[kB], b[kB];
+    float2 c[kB];
 #pragma unroll
-  for (int q = 0; q < 10; ++q) s[q] = 0.0;
-  for (int k = k0; k < k1; ++k) {
-    const int32_t e = __ldg(cf_idx + k);
-    const double* fp = fface + (int64_t)kFaceStride * (e >> 1);
-    const double sg = (e & 1) ? 1.0 : -1.0;
+    for (int j = 0; j < kB; ++j) e[j] = k + j < k1 ? __ldg(cf_idx + k + j) : -1;
 #pragma unroll
-    for (int q = 0; q < 10; ++q) s[q] += sg * __ldg(fp + q);
-  }
-}
-template <>
-__device__ __forceinline__ void face_sums<float>(int k0, int k1, const int32_t* __restrict__ cf_idx,
-                                                 const float* __restrict__ fface, double s[10]) {
-  float hi[10], lo[10];
+    for (int j = 0; j < kB; ++j) {
+      if (e[j] < 0) continue;
+      const float* fp = fface + (int64_t)kFaceStride * (e[j] >> 1);
+      if (kQ0 < 4) a[j] = __ldg(reinterpret_cast<const float4*>(fp));
+      b[j] = __ldg(reinterpret_cast<const float4*>(fp) + 1);
+      c[j] = __ldg(reinterpret_cast<const float2*>(fp) + 4);
+    }
 #pragma unroll
-  for (int q = 0; q < 10; ++q) hi[q] = lo[q] = 0.f;
-  for (int k = k0; k < k1; ++k) {
-    const int32_t e = __ldg(cf_idx + k);
-    const float4* fp = reinterpret_cast<const float4*>(fface + (int64_t)kFaceStride * (e >> 1));
-    const float4 a = __ldg(fp), b = __ldg(fp + 1), c = __ldg(fp + 2);
-    float x[10] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y};
-    const bool neg = !(e & 1);
+    for (int j = 0; j < kB; ++j) {
+      if (e[j] < 0) continue;
+      const float x[10] = {a[j].x, a[j].y, a[j].z, a[j].w, b[j].x,
+                           b[j].y, b[j].z, b[j].w, c[j].x, c[j].y};
+      const bool neg = !(e[j] & 1);
 #pragma unroll
-    for (int q = 0; q < 10; ++q) {
-      const float xv = neg ? -x[q] : x[q];
-      const float t = __fadd_rn(hi[q], xv);
-      const float bb = __fsub_rn(t, hi[q]);
-      const float err = __fadd_rn(__fsub_rn(hi[q], __fsub_rn(t, bb)), __fsub_rn(xv, bb));
-      hi[q] = t;
-      lo[q] = __fadd_rn(lo[q], err);
+      for (int q = kQ0; q < 10; ++q) add(q, neg ? -x[q] : x[q]);
     }
   }
+}
+template <int kQ0, int kB, class F>
+__device__ __forceinline__ void face_loop(int k0, int k1, const int32_t* __restrict__ cf_idx,
+                                          const double* __restrict__ fface, F add) {
+  for (int k = k0; k < k1; k += kB) {
+    int32_t e[kB];
+    double2 x[kB][5];
 #pragma unroll
-  for (int q = 0; q < 10; ++q) s[q] = (double)hi[q] + (double)lo[q];
+    for (int j = 0; j < kB; ++j) e[j] = k + j < k1 ? __ldg(cf_idx + k + j) : -1;
+#pragma unroll
+    for (int j = 0; j < kB; ++j) {
+      if (e[j] < 0) continue;
+      const double2* fp =
+          reinterpret_cast<const double2*>(fface + (int64_t)kFaceStride * (e[j] >> 1));
+#pragma unroll
+      for (int q = kQ0 / 2; q < 5; ++q) x[j][q] = __ldg(fp + q);
+    }
+#pragma unroll
+    for (int j = 0; j < kB; ++j) {
+      if (e[j] < 0) continue;
+      const bool neg = !(e[j] & 1);
+#pragma unroll
+      for (int q = kQ0; q < 10; ++q) {
+        const double v = (q & 1) ? x[j][q / 2].y : x[j][q / 2].x;
+        add(q, neg ? -v : v);
+      }
+    }
+  }
+}
+// FP64 sums of FP64 face fluxes.
+template <int kQ0, int kB>
+__device__ __forceinline__ void face_sums(int k0, int k1, const int32_t* __restrict__ cf_idx,
+                                          const double* __restrict__ fface, double s[10]) {
+#pragma unroll
+  for (int q = kQ0; q < 10; ++q) s[q] = 0.0;
+  face_loop<kQ0, kB>(k0, k1, cf_idx, fface, [&](int q, double x) { s[q] += x; });
+}
+// FP64 sums of FP32 face fluxes without FP64 arithmetic in the loop (GB300 runs FP64 at 1/64 of
+// the FP32 rate): each component is an unevaluated sum h + l + r of floats, TwoSum (Knuth)
+// carrying the rounding errors of h into l and those of l into r, so nothing above 2^-72 of the
+// sum is lost and the value handed on is the exact sum rounded to FP64 (a double accumulation
+// rounds at every face). r is zero unless the fluxes of a cell differ by more than 2^20.
+template <int kQ0, int kB>
+__device__ __forceinline__ void face_sums(int k0, int k1, const int32_t* __restrict__ cf_idx,
+                                          const float* __restrict__ fface, double s[10]) {
+  float h[10], l[10], r[10];
+#pragma unroll
+  for (int q = kQ0; q < 10; ++q) h[q] = l[q] = r[q] = 0.f;
+  face_loop<kQ0, kB>(k0, k1, cf_idx, fface, [&](int q, float x) {
+    const ff t = two_sum(h[q], x), u = two_sum(l[q], t.l);
+    h[q] = t.h;
+    l[q] = u.h;
+    r[q] = __fadd_rn(r[q], u.l);
+  });
+#pragma unroll
+  for (int q = kQ0; q < 10; ++q) {
+    double lo = (double)l[q];
+    if (r[q] != 0.f) lo += (double)r[q];
+    s[q] = (double)h[q] + lo;
+  }
 }
 
 // Per cell: L = -(1/|Omega|) sum_f s_f F_f in the cell's fixed face order, and Lt from dF/dt
 // (the residual of gks_residual), in FP64.
-template <class R>
+template <class R, int kB>
 __global__ void __launch_bounds__(256) k_gather(
     int64_t nc, const int32_t* __restrict__ cf_ptr, const int32_t* __restrict__ cf_idx,
     const R* __restrict__ fface, const double* __restrict__ ivol, double* __restrict__ L,
     double* __restrict__ Lt) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= nc) return;
-  double s[10];
-  face_sums(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, s);
   const double iv = ivol[i];
+  double s[10];
+  face_sums<0, kB>(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, s);
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     L[v * nc + i] = s[v] * iv;
@@ -919,29 +990,21 @@ __global__ void __launch_bounds__(256) k_gather(
 // FP32 path: every operation in float-float arithmetic, so the update is conservative to about
 // 2^-46 relative and issues no FP64 instruction.
 
-// Face sums as float-float pairs, components q0..9 (FP32 path).
+// Face sums as float-float pairs, components kQ0..9 (FP32 path).
+template <int kQ0, int kB>
 __device__ __forceinline__ void face_sums_ff(int k0, int k1, const int32_t* __restrict__ cf_idx,
-                                             const float* __restrict__ fface, int q0, ff s[10]) {
+                                             const float* __restrict__ fface, ff s[10]) {
 #pragma unroll
-  for (int q = 0; q < 10; ++q) s[q] = ff{0.f, 0.f};
-  for (int k = k0; k < k1; ++k) {
-    const int32_t e = __ldg(cf_idx + k);
-    const float4* fp = reinterpret_cast<const float4*>(fface + (int64_t)kFaceStride * (e >> 1));
-    const float4 a = __ldg(fp), b = __ldg(fp + 1), c = __ldg(fp + 2);
-    const float x[10] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y};
-    const bool neg = !(e & 1);
+  for (int q = kQ0; q < 10; ++q) s[q] = ff{0.f, 0.f};
+  face_loop<kQ0, kB>(k0, k1, cf_idx, fface, [&](int q, float x) {
+    const ff t = two_sum(s[q].h, x);
+    s[q] = ff{t.h, __fadd_rn(s[q].l, t.l)};
+  });
 #pragma unroll
-    for (int q = 0; q < 10; ++q) {
-      if (q < q0) continue;
-      const ff t = two_sum(s[q].h, neg ? -x[q] : x[q]);
-      s[q] = ff{t.h, __fadd_rn(s[q].l, t.l)};
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 10; ++q) s[q] = two_sum(s[q].h, s[q].l);
+  for (int q = kQ0; q < 10; ++q) s[q] = two_sum(s[q].h, s[q].l);
 }
 
-template <bool kSecond>
+template <bool kSecond, int kB>
 __global__ void __launch_bounds__(256) k_stage_f(
     int64_t nc, const int32_t* __restrict__ cf_ptr, const int32_t* __restrict__ cf_idx,
     const float* __restrict__ fface, const ff* __restrict__ ivol, ff c1, ff c2,
@@ -949,11 +1012,17 @@ __global__ void __launch_bounds__(256) k_stage_f(
     int* flag) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= nc) return;
-  ff s[10];
-  face_sums_ff(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, kSecond ? 5 : 0, s);
-  const ff iv = ivol[i];
   Gq<float> g;
-  g.load(QA, i);
+  ff iv, s[10];
+  if (kB > 1) {  // requested before the chain of the face sums
+    iv = ivol[i];
+    g.load(QA, i);
+  }
+  face_sums_ff<kSecond ? 5 : 0, kB>(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, s);
+  if (kB == 1) {
+    iv = ivol[i];
+    g.load(QA, i);
+  }
   ff q[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
@@ -979,7 +1048,7 @@ __global__ void __launch_bounds__(256) k_stage_f(
 // accumulate the FP32 face fluxes in FP64, and the update reads and writes the FP64 state
 // [5][nc], which is the master copy in this mode; the gather copies the reconstruction reads
 // (float pairs) are written from it: Q* by stage 1, Q^{n+1} by stage 2.
-template <bool kSecond>
+template <bool kSecond, int kB>
 __global__ void __launch_bounds__(256) k_stage_fd(
     int64_t nc, const int32_t* __restrict__ cf_ptr, const int32_t* __restrict__ cf_idx,
     const float* __restrict__ fface, const double* __restrict__ ivol, double c1, double c2,
@@ -988,17 +1057,7 @@ __global__ void __launch_bounds__(256) k_stage_fd(
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= nc) return;
   double s[10];
-#pragma unroll
-  for (int q = 0; q < 10; ++q) s[q] = 0.0;
-  for (int k = cf_ptr[i]; k < cf_ptr[i + 1]; ++k) {
-    const int32_t e = __ldg(cf_idx + k);
-    const float4* fp = reinterpret_cast<const float4*>(fface + (int64_t)kFaceStride * (e >> 1));
-    const float4 a = __ldg(fp), b = __ldg(fp + 1), c = __ldg(fp + 2);
-    const float x[10] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, c.x, c.y};
-    const double sg = (e & 1) ? 1.0 : -1.0;
-#pragma unroll
-    for (int q = 0; q < 10; ++q) s[q] += sg * (double)x[q];
-  }
+  face_sums<kSecond ? 5 : 0, kB>(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, s);
   const double iv = ivol[i];
   double q[5];
 #pragma unroll
@@ -1019,7 +1078,7 @@ __global__ void __launch_bounds__(256) k_stage_fd(
   if (!physical(q)) atomicOr(flag, kErrNonphysical);
 }
 
-template <bool kSecond>
+template <bool kSecond, int kB>
 __global__ void __launch_bounds__(256) k_stage_d(
     int64_t nc, const int32_t* __restrict__ cf_ptr, const int32_t* __restrict__ cf_idx,
     const double* __restrict__ fface, const double* __restrict__ ivol, double c1, double c2,
@@ -1027,11 +1086,11 @@ __global__ void __launch_bounds__(256) k_stage_d(
     double* __restrict__ QsA, int* flag) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= nc) return;
-  double s[10];
-  face_sums<double>(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, s);
   const double iv = ivol[i];
   Gq<double> g;
   g.load(QA, i);
+  double s[10];
+  face_sums<kSecond ? 5 : 0, kB>(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, s);
   double q[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
@@ -1221,7 +1280,7 @@ __global__ void __launch_bounds__(256) k_jacobi_init(
   R res[5];
   if constexpr (std::is_same<R, float>::value) {
     ff s[10];
-    face_sums_ff(k0, k1, cf_idx, fface, 0, s);
+    face_sums_ff<0, 1>(k0, k1, cf_idx, fface, s);
     const ff h = ff_from(0.5 * dt);
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
@@ -1230,7 +1289,7 @@ __global__ void __launch_bounds__(256) k_jacobi_init(
     }
   } else {
     double s[10];
-    face_sums<double>(k0, k1, cf_idx, fface, s);
+    face_sums<0, 1>(k0, k1, cf_idx, fface, s);
 #pragma unroll
     for (int v = 0; v < 5; ++v) res[v] = s[v] + 0.5 * dt * s[5 + v];
   }
@@ -1409,17 +1468,27 @@ inline int recon_blocks_per_sm(size_t smem) {
   return (int)(kSmemPerSM / (smem + kSmemPerBlockReserved));
 }
 
+// One launch over the tiles of ranges r0 .. r1 - 1 with stencil, entry and slot bounds K, S, M.
 template <class R, bool kPf, bool kStB>
-void launch_recon_range(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* QA,
-                        R* poly, int* flag, int r, size_t smem, cudaStream_t st) {
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_recon<R, kPf, kStB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
-  ReconUni u{m.rr.uni[r], m.rr.K[r], m.rr.S[r], m.rr.cnt[r], m.rr.st0[r], m.rr.sb0[r]};
-  k_recon<R, kPf, kStB><<<(unsigned)(m.rr.t1[r] - m.rr.t0[r]), kReconThreads, smem, st>>>(
-      m.nc, m.rr.t0[r], m.rr.K[r], m.rr.S[r], m.rr.M[r], u, QA, m.t_K, m.t_cnt, m.t_st, m.t_sb,
-      m.t_idx, g.Ap, g.Bp, g.cell, p.weno_gamma, p.weno_eps, p.weno_pow, poly, flag,
-      p.wait_tries, p.withhold);
+void launch_recon_ranges(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* QA,
+                         R* poly, int* flag, int r0, int r1, int K, int S, int M, size_t smem,
+                         cudaStream_t st) {
+  ReconSet set;
+  set.n = r1 - r0;
+  for (int r = r0; r < r1; ++r)
+    set.r[r - r0] = ReconUni{m.rr.uni[r], m.rr.K[r],  m.rr.S[r], m.rr.cnt[r],
+                             m.rr.st0[r], m.rr.sb0[r], m.rr.t0[r]};
+  auto run = [&](auto kern, const auto& arg) {
+    if (smem > 48 * 1024)
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    kern<<<(unsigned)(m.rr.t1[r1 - 1] - m.rr.t0[r0]), kReconThreads, smem, st>>>(
+        m.nc, m.rr.t0[r0], K, S, M, arg, QA, m.t_K, m.t_cnt, m.t_st, m.t_sb, m.t_idx, g.Ap, g.Bp,
+        g.cell, p.weno_gamma, p.weno_eps, p.weno_pow, poly, flag, p.wait_tries, p.withhold);
+  };
+  if (r1 - r0 > 1)
+    run(k_recon<R, kPf, kStB, true>, set);
+  else
+    run(k_recon<R, kPf, kStB, false>, set.r[0]);
 }
 
 // Ghost slots of moving no-slip walls and far-field planes: QA[nc + g] = the image's flow
@@ -1501,8 +1570,26 @@ __global__ void __launch_bounds__(128) k_ghost_fill(int64_t nc, int64_t ng,
   }
 }
 
-// One launch per tile range, the bulk-copy variant whenever its shared memory fits a block. The
-// ranges are independent: with fj, range r > 0 runs on auxiliary stream r - 1, forked from and
+// Threads per block of the per-cell kernels: 256, or 64 where 256 would leave SMs without a block.
+inline int cell_threads(int64_t nc) { return nc < 256 * 152 ? 64 : 256; }
+// Largest number of tiles reconstructed by one launch over all ranges: one wave of the FP32
+// kernel (5 blocks on each of 152 SMs). Below it the launches and the streams' events cost more
+// than the ranges gain from shared memory of their own size: ten steps of the 8^3-cube mesh 564
+// (four launches) -> 485 us, of the 16^3-cube mesh (512 tiles) 700 -> 663 us; at 24^3 cubes
+// (1,728 tiles) 1.299 against 1.278 ms, at 64^3 cubes a pass takes 0.381 ms in one launch against
+// 0.356.
+constexpr int64_t kReconMergeTiles = 760;
+inline bool recon_merged(const TileRanges& rr) {
+  return rr.n > 1 && rr.t1[rr.n - 1] - rr.t0[0] <= kReconMergeTiles;
+}
+int recon_launches(const DevMesh& m) {
+  int n = m.ng > 0 ? 1 : 0;  // the ghost refresh of moving no-slip walls and far-field planes
+  if (recon_merged(m.rr)) return n + 1;
+  for (int r = 0; r < m.rr.n; ++r) n += m.rr.t1[r] > m.rr.t0[r] ? 1 : 0;
+  return n;
+}
+// One launch per tile range (one over all of them on small meshes), the bulk-copy variant
+// whenever its shared memory fits a block. The ranges are independent: with fj, range r > 0 runs on auxiliary stream r - 1, forked from and
 // joined back into st, so that the ranges' blocks share the GPU.
 template <class R>
 void launch_recon(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* QA,
@@ -1512,30 +1599,43 @@ void launch_recon(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const
     k_ghost_fill<R><<<blocks_for(m.ng, 128), 128, 0, st>>>(
         m.nc, m.ng, m.g_src, m.g_map, m.g_mapf, m.g_chain, m.bcs, flux_params(p),
         wall_table<R>(m), const_cast<R*>(QA));
+  const TileRanges& rr = m.rr;
+  auto launch = [&](int r0, int r1, cudaStream_t s) {
+    int K = 0, S = 0, M = 0;
+    for (int r = r0; r < r1; ++r) {
+      K = std::max(K, rr.K[r]);
+      S = std::max(S, rr.S[r]);
+      M = std::max(M, rr.M[r]);
+    }
+    // the sub-stencil entries are staged in shared memory only where that costs the range no
+    // resident blocks below the register bound; otherwise they are prefetched into L2 like the
+    // rows (the pyramids and hexahedra of the hybrid meshes, which have eight sub-stencils)
+    const ReconSmem<R> pb(K, S, M, true, true), pl(K, S, M, true, false);
+    const int nb_l = std::min(kReconBlocksPerSM<R>, recon_blocks_per_sm(pl.bytes));
+    if (pb.bytes <= kMaxBlockSmem && recon_blocks_per_sm(pb.bytes) >= nb_l) {
+      launch_recon_ranges<R, true, true>(m, g, p, QA, poly, flag, r0, r1, K, S, M, pb.bytes, s);
+    } else if (pl.bytes <= kMaxBlockSmem) {
+      launch_recon_ranges<R, true, false>(m, g, p, QA, poly, flag, r0, r1, K, S, M, pl.bytes, s);
+    } else {
+      const ReconSmem<R> np(K, S, M, false, false);
+      launch_recon_ranges<R, false, false>(m, g, p, QA, poly, flag, r0, r1, K, S, M, np.bytes, s);
+    }
+  };
+  if (recon_merged(rr)) {  // the ranges are consecutive and cover all tiles
+    launch(0, rr.n, st);
+    return;
+  }
   int used = 0;
-  const bool fork = fj && fj->n > 0 && m.rr.n > 1;
+  const bool fork = fj && fj->n > 0 && rr.n > 1;
   if (fork) cudaEventRecord(fj->fork, st);
-  for (int r = 0; r < m.rr.n; ++r) {
-    if (m.rr.t1[r] <= m.rr.t0[r]) continue;
+  for (int r = 0; r < rr.n; ++r) {
+    if (rr.t1[r] <= rr.t0[r]) continue;
     cudaStream_t s = st;
     if (fork && r > 0 && used < fj->n) {
       s = fj->aux[used];
       cudaStreamWaitEvent(s, fj->fork, 0);
     }
-    // the sub-stencil entries are staged in shared memory only where that costs the range no
-    // resident blocks below the register bound; otherwise they are prefetched into L2 like the
-    // rows (the pyramids and hexahedra of the hybrid meshes, which have eight sub-stencils)
-    const ReconSmem<R> pb(m.rr.K[r], m.rr.S[r], m.rr.M[r], true, true);
-    const ReconSmem<R> pl(m.rr.K[r], m.rr.S[r], m.rr.M[r], true, false);
-    const int nb_l = std::min(kReconBlocksPerSM<R>, recon_blocks_per_sm(pl.bytes));
-    if (pb.bytes <= kMaxBlockSmem && recon_blocks_per_sm(pb.bytes) >= nb_l) {
-      launch_recon_range<R, true, true>(m, g, p, QA, poly, flag, r, pb.bytes, s);
-    } else if (pl.bytes <= kMaxBlockSmem) {
-      launch_recon_range<R, true, false>(m, g, p, QA, poly, flag, r, pl.bytes, s);
-    } else {
-      const ReconSmem<R> np(m.rr.K[r], m.rr.S[r], m.rr.M[r], false, false);
-      launch_recon_range<R, false, false>(m, g, p, QA, poly, flag, r, np.bytes, s);
-    }
+    launch(r, r + 1, s);
     if (s != st) {
       cudaEventRecord(fj->join[used], s);
       cudaStreamWaitEvent(st, fj->join[used], 0);
@@ -1558,46 +1658,38 @@ void launch_flux(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const 
 template <class R>
 void launch_gather(const DevMesh& m, const Geo64& g, const R* fface, double* L, double* Lt,
                    cudaStream_t st) {
-  k_gather<R><<<blocks_for(m.nc, 256), 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, g.ivol, L,
-                                                       Lt);
+  const int nt = cell_threads(m.nc);
+  auto kern = nt < 256 ? k_gather<R, kFaceBatch> : k_gather<R, 1>;
+  kern<<<blocks_for(m.nc, nt), nt, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, g.ivol, L, Lt);
 }
 template <class R>
 void launch_stage(const DevMesh& m, const GeoR<R>& g, const R* fface, int stage, double dt,
                   void* L, void* Lt, R* QA, R* QsA, int* flag, cudaStream_t st, double* Q64,
                   const double* ivol64) {
-  const unsigned nb = blocks_for(m.nc, 256);
+  const int nt = cell_threads(m.nc);
+  const bool small = nt < 256;
+  const unsigned nb = blocks_for(m.nc, nt);
   // stage 1: c1 = dt/2, c2 = dt^2/8; stage 2: c1 = dt, c2 = dt^2/6
   const double c1 = stage == 1 ? 0.5 * dt : dt, c2 = stage == 1 ? dt * dt / 8.0 : dt * dt / 6.0;
+  constexpr int kB = kFaceBatch;
   if constexpr (std::is_same<R, float>::value) {
     if (Q64) {  // FP64 update of the FP64 master state
-      double* l = static_cast<double*>(L);
-      double* lt = static_cast<double*>(Lt);
-      if (stage == 1)
-        k_stage_fd<false><<<nb, 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, ivol64, c1, c2, l,
-                                              lt, Q64, QA, QsA, flag);
-      else
-        k_stage_fd<true><<<nb, 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, ivol64, c1, c2, l,
-                                             lt, Q64, QA, QsA, flag);
+      auto kern = stage == 1 ? k_stage_fd<false, kB> : k_stage_fd<true, kB>;
+      kern<<<nb, nt, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, ivol64, c1, c2,
+                              static_cast<double*>(L), static_cast<double*>(Lt), Q64, QA, QsA,
+                              flag);
       return;
     }
-    ff* l = static_cast<ff*>(L);
-    ff* lt = static_cast<ff*>(Lt);
-    const ff* iv = reinterpret_cast<const ff*>(g.ivol);
-    if (stage == 1)
-      k_stage_f<false><<<nb, 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, iv, ff_from(c1),
-                                           ff_from(c2), l, lt, QA, QsA, flag);
-    else
-      k_stage_f<true><<<nb, 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, iv, ff_from(c1),
-                                          ff_from(c2), l, lt, QA, QsA, flag);
+    auto kern = stage == 1 ? (small ? k_stage_f<false, kB> : k_stage_f<false, 1>)
+                           : (small ? k_stage_f<true, kB> : k_stage_f<true, 1>);
+    kern<<<nb, nt, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface,
+                            reinterpret_cast<const ff*>(g.ivol), ff_from(c1), ff_from(c2),
+                            static_cast<ff*>(L), static_cast<ff*>(Lt), QA, QsA, flag);
   } else {
-    double* l = static_cast<double*>(L);
-    double* lt = static_cast<double*>(Lt);
-    if (stage == 1)
-      k_stage_d<false><<<nb, 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, g.ivol, c1, c2, l, lt,
-                                           QA, QsA, flag);
-    else
-      k_stage_d<true><<<nb, 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, g.ivol, c1, c2, l, lt,
-                                          QA, QsA, flag);
+    auto kern = stage == 1 ? (small ? k_stage_d<false, kB> : k_stage_d<false, 1>)
+                           : (small ? k_stage_d<true, kB> : k_stage_d<true, 1>);
+    kern<<<nb, nt, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, g.ivol, c1, c2,
+                            static_cast<double*>(L), static_cast<double*>(Lt), QA, QsA, flag);
   }
 }
 void launch_s2o4_stage(int64_t n, int stage, double dt, const double* Q, const double* L,
