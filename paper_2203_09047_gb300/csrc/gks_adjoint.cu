@@ -212,191 +212,214 @@ __global__ void k_vjp_poly(int64_t nc, const int32_t* __restrict__ cf_ptr,
   for (int q = 0; q < 50; ++q) o[q] = s[q];
 }
 
-// Reverse of the reconstruction of one cell, one variable at a time (the variables are
-// independent: each has its own weights).
-__global__ void __launch_bounds__(64) k_vjp_recon(
+// Reverse of the reconstruction, one block of five warps per 32-cell tile, warp = variable, lane =
+// cell (the variables are independent: each has its own weights), no thread reads another's
+// values. The stencil differences of a thread are a column of shared memory, which its cotangents
+// take over once the forward part is done; nothing is indexed in local memory. Bound by the FP64
+// pipe (about 770 FP64 instructions per thread and 18-member stencil). One thread per cell with
+// the differences, fits and cotangents in local arrays moved 4.1 GB per launch through them: 2.18
+// -> 1.44 ms at 131,072 cells, 478 -> 213 us at 16,384 cells (256 blocks of 64
+// threads left most of the GPU idle).
+constexpr int kVjpThreads = 5 * kTile;
+__global__ void __launch_bounds__(kVjpThreads) k_vjp_recon(
     int64_t nc, const double* __restrict__ QA, const int32_t* __restrict__ t_K,
     const uint64_t* __restrict__ t_cnt, const int32_t* __restrict__ t_st,
     const int32_t* __restrict__ t_sb, const int32_t* __restrict__ t_idx,
-    const int32_t* __restrict__ st_ptr, const int8_t* __restrict__ n_sub,
-    const double* __restrict__ Ap, const double* __restrict__ Bp, const double* __restrict__ mom,
-    const double* __restrict__ hcell, double wg, double weps, int wpow,
-    const double* __restrict__ gpc, double* __restrict__ gdq, double* __restrict__ gq0) {
-  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+    const int32_t* __restrict__ st_ptr, const double* __restrict__ Ap,
+    const double* __restrict__ Bp, const double* __restrict__ cell, double wg, double weps,
+    int wpow, const double* __restrict__ gpc, double* __restrict__ gdq,
+    double* __restrict__ gq0) {
+  extern __shared__ double col_s[];
+  const int64_t tile = blockIdx.x;
+  const int lane = threadIdx.x & (kTile - 1), v = threadIdx.x / kTile;
+  const int64_t i = tile * kTile + lane;
   if (i >= nc) return;
-  const int64_t tile = i / kTile;
-  const int lane = (int)(i % kTile);
-  const int K = st_ptr[i + 1] - st_ptr[i];  // the cell's own members (tile padding excluded)
   const int KT = t_K[tile];
   const uint64_t cnt = t_cnt[tile];
-  const int M = n_sub[i];
   const int64_t row0 = t_st[tile];
   const int32_t* sidx = t_idx + row0 * kTile + lane;
   const double* A = Ap + row0 * 9 * kTile + lane;
   const double* Bt = Bp + ((int64_t)t_sb[tile] * kTile + lane) * 4;  // [slot][lane][4]
-  double* gdqc = gdq + row0 * 5 * kTile + lane;
-  double m2[6];
-  for (int q = 0; q < 6; ++q) m2[q] = mom[q * nc + i];
-  const double h = hcell[i], ih = 1.0 / h, ih2 = ih * ih;
-  const double g0 = 1.0 - wg * M;
-  double c0q[5];
-  for (int v = 0; v < 5; ++v) c0q[v] = QA[6 * i + v];
-  for (int v = 0; v < 5; ++v) {
-    // ---- forward: stencil differences, a, b_m, indicators, weights
-    double dq[kMaxStencil];
-    for (int k = 0; k < KT; ++k) {
-      const int32_t e = sidx[k * kTile];
-      double q = QA[6 * (int64_t)(e & kCellMask) + v];
-      if (v >= 1 && v <= 3 && ((e >> (kFlipShift + v - 1)) & 1)) q = -q;
-      dq[k] = q - c0q[v];
-    }
-    double a[9];
-    for (int n = 0; n < 9; ++n) {
-      double s = 0.0;
-      for (int k = 0; k < KT; ++k) s += A[(9 * k + n) * kTile] * dq[k];
-      a[n] = s;
-    }
-    double b[kMaxSub][3], bet[kMaxSub];
-    {
-      const double* e = Bt;
-      for (int s = 0; s < kMaxSub; ++s) {
-        const int cs = (int)((cnt >> (8 * s)) & 0xffu);
-        b[s][0] = b[s][1] = b[s][2] = 0.0;
-        for (int j = 0; j < cs; ++j, e += 4 * kTile) {
-          const int k = (int)e[3];
-          for (int t = 0; t < 3; ++t) b[s][t] += e[t] * dq[k];
-        }
-        bet[s] = b[s][0] * b[s][0] + b[s][1] * b[s][1] + b[s][2] * b[s][2];
-      }
-    }
-    const double gx[3] = {2 * a[3], a[6], a[7]};
-    const double gy[3] = {a[6], 2 * a[4], a[8]};
-    const double gz[3] = {a[7], a[8], 2 * a[5]};
-    auto mv = [&](const double g[3], double o[3]) {
-      o[0] = m2[0] * g[0] + m2[3] * g[1] + m2[4] * g[2];
-      o[1] = m2[3] * g[0] + m2[1] * g[1] + m2[5] * g[2];
-      o[2] = m2[4] * g[0] + m2[5] * g[1] + m2[2] * g[2];
-    };
-    double hx[3], hy[3], hz[3];
-    mv(gx, hx);
-    mv(gy, hy);
-    mv(gz, hz);
-    const double beta0 = a[0] * a[0] + a[1] * a[1] + a[2] * a[2] +
-                         (gx[0] * hx[0] + gx[1] * hx[1] + gx[2] * hx[2]) +
-                         (gy[0] * hy[0] + gy[1] * hy[1] + gy[2] * hy[2]) +
-                         (gz[0] * hz[0] + gz[1] * hz[1] + gz[2] * hz[2]) +
-                         4 * (a[3] * a[3] + a[4] * a[4] + a[5] * a[5]) + a[6] * a[6] +
-                         a[7] * a[7] + a[8] * a[8];
-    double tau = 0.0;
-    for (int s = 0; s < M; ++s) tau += fabs(beta0 - bet[s]);
-    tau /= M;
-    auto ratio_pow = [&](double r) {
-      double p = r;
-      for (int e = 1; e < wpow; ++e) p *= r;
-      return p;
-    };
-    double w[kMaxSub + 1], rr[kMaxSub + 1];
-    rr[0] = tau / (beta0 + weps);
-    w[0] = g0 * (1.0 + ratio_pow(rr[0]));
-    double S = w[0];
-    for (int s = 0; s < M; ++s) {
-      rr[s + 1] = tau / (bet[s] + weps);
-      w[s + 1] = wg * (1.0 + ratio_pow(rr[s + 1]));
-      S += w[s + 1];
-    }
-    const double wb0 = w[0] / S;
-    const double ca = wb0 / g0;
-    double cs[kMaxSub];
-    for (int s = 0; s < M; ++s) cs[s] = w[s + 1] / S - wb0 * wg / g0;
-    // ---- reverse
-    const double* go = gpc + (int64_t)kPolyStride * i + 10 * v;
-    double gQ0 = go[0];
-    double gC[9];
-    for (int n = 0; n < 3; ++n) gC[n] = go[1 + n] * ih;
-    for (int n = 3; n < 9; ++n) gC[n] = go[1 + n] * ih2 - go[0] * m2[n - 3];
-    double ga[9], gb[kMaxSub][3];
-    double gca = 0.0;
-    for (int n = 0; n < 9; ++n) {
-      ga[n] = ca * gC[n];
-      gca += gC[n] * a[n];
-    }
-    double gcs[kMaxSub];
-    for (int s = 0; s < kMaxSub; ++s) {
-      gb[s][0] = gb[s][1] = gb[s][2] = 0.0;
-      gcs[s] = 0.0;
-    }
-    for (int s = 0; s < M; ++s)
-      for (int t = 0; t < 3; ++t) {
-        gb[s][t] = cs[s] * gC[t];
-        gcs[s] += gC[t] * b[s][t];
-      }
-    // ca = wb0/g0, cs_s = wb_s - wb0 wg/g0
-    double gwb[kMaxSub + 1];
-    gwb[0] = gca / g0;
-    for (int s = 0; s < M; ++s) {
-      gwb[0] -= gcs[s] * wg / g0;
-      gwb[s + 1] = gcs[s];
-    }
-    // wb_j = w_j / S
-    double dotw = 0.0;
-    for (int j = 0; j <= M; ++j) dotw += gwb[j] * (w[j] / S);
-    double gtau = 0.0, gbeta0 = 0.0, gbet[kMaxSub];
-    for (int s = 0; s < kMaxSub; ++s) gbet[s] = 0.0;
-    for (int j = 0; j <= M; ++j) {
-      const double gw = (gwb[j] - dotw) / S;
-      const double gam = j == 0 ? g0 : wg;
-      const double r = rr[j];
-      double dpow = wpow;  // d(r^p)/dr = p r^(p-1)
-      for (int e = 1; e < wpow; ++e) dpow *= r;
-      const double gr = gw * gam * dpow;
-      const double bb = j == 0 ? beta0 : bet[j - 1];
-      gtau += gr / (bb + weps);
-      const double gbb = -gr * tau / ((bb + weps) * (bb + weps));
-      if (j == 0)
-        gbeta0 += gbb;
-      else
-        gbet[j - 1] += gbb;
-    }
-    // tau = sum_s |beta0 - beta_s| / M  (derivative of |x| taken as +1 at x = 0)
-    for (int s = 0; s < M; ++s) {
-      const double sg = (beta0 - bet[s]) < 0.0 ? -1.0 : 1.0;
-      gbeta0 += sg * gtau / M;
-      gbet[s] -= sg * gtau / M;
-    }
-    // beta_s = |b_s|^2
-    for (int s = 0; s < M; ++s)
-      for (int t = 0; t < 3; ++t) gb[s][t] += 2.0 * b[s][t] * gbet[s];
-    // beta0
-    for (int n = 0; n < 3; ++n) ga[n] += 2.0 * a[n] * gbeta0;
-    ga[3] += (2.0 * (2.0 * hx[0]) + 8.0 * a[3]) * gbeta0;
-    ga[4] += (2.0 * (2.0 * hy[1]) + 8.0 * a[4]) * gbeta0;
-    ga[5] += (2.0 * (2.0 * hz[2]) + 8.0 * a[5]) * gbeta0;
-    ga[6] += (2.0 * hx[1] + 2.0 * hy[0] + 2.0 * a[6]) * gbeta0;
-    ga[7] += (2.0 * hx[2] + 2.0 * hz[0] + 2.0 * a[7]) * gbeta0;
-    ga[8] += (2.0 * hy[2] + 2.0 * hz[1] + 2.0 * a[8]) * gbeta0;
-    // a = A+ dq, b_s = B_s dq|S_s
-    double gd[kMaxStencil];
-    for (int k = 0; k < KT; ++k) {
-      double s = 0.0;
-      for (int n = 0; n < 9; ++n) s += A[(9 * k + n) * kTile] * ga[n];
-      gd[k] = s;
-    }
-    {
-      const double* e = Bt;
-      for (int s = 0; s < kMaxSub; ++s) {
-        const int csn = (int)((cnt >> (8 * s)) & 0xffu);
-        for (int j = 0; j < csn; ++j, e += 4 * kTile) {
-          const int k = (int)e[3];
-          for (int t = 0; t < 3; ++t) gd[k] += e[t] * gb[s][t];
-        }
-      }
-    }
-    for (int k = 0; k < KT; ++k) {
-      gQ0 -= gd[k];
-      gdqc[(5 * k + v) * kTile] = k < K ? gd[k] : 0.0;
-    }
-    gq0[v * nc + i] = gQ0;
+  const double* rec = cell + tile * kCellRec * kTile + lane;
+  double* col = col_s + v * kTile + lane;  // col[5 kTile k]: member k
+  constexpr int kS = kVjpThreads;
+  // ---- forward: stencil differences, a, b_m, indicators, weights
+  const double c0 = QA[6 * i + v];
+#pragma unroll 4
+  for (int k = 0; k < KT; ++k) {
+    const int32_t e = sidx[k * kTile];
+    double q = QA[6 * (int64_t)(e & kCellMask) + v];
+    if (v >= 1 && v <= 3 && ((e >> (kFlipShift + v - 1)) & 1)) q = -q;
+    col[kS * k] = q - c0;
   }
+  double a[9];
+#pragma unroll
+  for (int n = 0; n < 9; ++n) a[n] = 0.0;
+#pragma unroll 2
+  for (int k = 0; k < KT; ++k) {
+    const double d = col[kS * k];
+#pragma unroll
+    for (int n = 0; n < 9; ++n) a[n] += A[(9 * k + n) * kTile] * d;
+  }
+  double b[kMaxSub][3], inv[kMaxSub + 2], bet[kMaxSub];
+  {
+    const double* e = Bt;
+#pragma unroll
+    for (int s = 0; s < kMaxSub; ++s) {
+      const int cs = (int)((cnt >> (8 * s)) & 0xffu);
+      b[s][0] = b[s][1] = b[s][2] = 0.0;
+      for (int j = 0; j < cs; ++j, e += 4 * kTile) {
+        const double2 x = *reinterpret_cast<const double2*>(e);
+        const double2 y = *reinterpret_cast<const double2*>(e + 2);
+        const double d = col[kS * (int)y.y];
+        b[s][0] += x.x * d;
+        b[s][1] += x.y * d;
+        b[s][2] += y.x * d;
+      }
+      bet[s] = b[s][0] * b[s][0] + b[s][1] * b[s][1] + b[s][2] * b[s][2];
+    }
+  }
+  double m2[6];
+#pragma unroll
+  for (int q = 0; q < 6; ++q) m2[q] = rec[q * kTile];
+  const double ih = rec[6 * kTile], ih2 = ih * ih, iM = rec[8 * kTile], ig0 = rec[9 * kTile];
+  const int M = (int)rec[7 * kTile];
+  const double g0 = 1.0 - wg * rec[7 * kTile];
+  const double gx[3] = {2 * a[3], a[6], a[7]};
+  const double gy[3] = {a[6], 2 * a[4], a[8]};
+  const double gz[3] = {a[7], a[8], 2 * a[5]};
+  auto mv = [&](const double g[3], double o[3]) {
+    o[0] = m2[0] * g[0] + m2[3] * g[1] + m2[4] * g[2];
+    o[1] = m2[3] * g[0] + m2[1] * g[1] + m2[5] * g[2];
+    o[2] = m2[4] * g[0] + m2[5] * g[1] + m2[2] * g[2];
+  };
+  double hx[3], hy[3], hz[3];
+  mv(gx, hx);
+  mv(gy, hy);
+  mv(gz, hz);
+  const double beta0 = a[0] * a[0] + a[1] * a[1] + a[2] * a[2] +
+                       (gx[0] * hx[0] + gx[1] * hx[1] + gx[2] * hx[2]) +
+                       (gy[0] * hy[0] + gy[1] * hy[1] + gy[2] * hy[2]) +
+                       (gz[0] * hz[0] + gz[1] * hz[1] + gz[2] * hz[2]) +
+                       4 * (a[3] * a[3] + a[4] * a[4] + a[5] * a[5]) + a[6] * a[6] +
+                       a[7] * a[7] + a[8] * a[8];
+  double tau = 0.0;
+#pragma unroll
+  for (int s = 0; s < kMaxSub; ++s)
+    if (s < M) tau += fabs(beta0 - bet[s]);
+  tau *= iM;
+  // inv[j] = 1 / (beta_j + eps) (j = 0: beta_0), three reciprocals from one division
+  inv[0] = beta0 + weps;
+#pragma unroll
+  for (int s = 0; s < kMaxSub; ++s) inv[s + 1] = s < M ? bet[s] + weps : 1.0;
+#pragma unroll
+  for (int g = 0; g < 3; ++g) {
+    if (3 * g > M) continue;
+    const double x = inv[3 * g], y = inv[3 * g + 1], z = inv[3 * g + 2], xy = x * y;
+    const double r = 1.0 / (xy * z), rz = r * z;
+    inv[3 * g] = rz * y;
+    inv[3 * g + 1] = rz * x;
+    inv[3 * g + 2] = r * xy;
+  }
+  // w_j = gam_j (1 + r_j^p), r_j = tau inv_j; dw_j/dr_j = gam_j p r_j^(p-1)
+  double w[kMaxSub + 1], S = 0.0;
+#pragma unroll
+  for (int j = 0; j <= kMaxSub; ++j) {
+    w[j] = 0.0;
+    if (j > M) continue;
+    const double r = tau * inv[j];
+    double p = r;
+    for (int e = 1; e < wpow; ++e) p *= r;
+    w[j] = (j == 0 ? g0 : wg) * (1.0 + p);
+    S += w[j];
+  }
+  const double iS = 1.0 / S, wb0 = w[0] * iS, ca = wb0 * ig0, corr = wb0 * wg * ig0;
+  // ---- reverse
+  const double* go = gpc + (int64_t)kPolyStride * i + 10 * v;
+  double gQ0 = go[0], ga[9], gC[3], gca = 0.0;
+#pragma unroll
+  for (int n = 0; n < 9; ++n) {
+    const double x = n < 3 ? go[1 + n] * ih : go[1 + n] * ih2 - go[0] * m2[n < 3 ? 0 : n - 3];
+    if (n < 3) gC[n] = x;
+    ga[n] = ca * x;
+    gca += x * a[n];
+  }
+  // c_s = wb_s - wb0 wg / g0 multiplies b_s; ca = wb0 / g0 multiplies a; wb_j = w_j / S
+  double gcs[kMaxSub], gwb0 = gca * ig0, dotw = 0.0;
+#pragma unroll
+  for (int s = 0; s < kMaxSub; ++s) {
+    gcs[s] = 0.0;
+    if (s >= M) continue;
+    gcs[s] = gC[0] * b[s][0] + gC[1] * b[s][1] + gC[2] * b[s][2];
+    gwb0 -= gcs[s] * wg * ig0;
+    dotw += gcs[s] * w[s + 1];
+  }
+  dotw = (dotw + gwb0 * w[0]) * iS;
+  double gtau = 0.0, gbeta0 = 0.0, gbet[kMaxSub];
+#pragma unroll
+  for (int j = 0; j <= kMaxSub; ++j) {
+    if (j > 0) gbet[j > 0 ? j - 1 : 0] = 0.0;
+    if (j > M) continue;
+    const double gw = ((j == 0 ? gwb0 : gcs[j > 0 ? j - 1 : 0]) - dotw) * iS;
+    const double r = tau * inv[j];
+    double dpow = wpow;
+    for (int e = 1; e < wpow; ++e) dpow *= r;
+    const double x = gw * (j == 0 ? g0 : wg) * dpow * inv[j];  // cotangent of r over bb
+    gtau += x;
+    if (j == 0)
+      gbeta0 -= x * r;
+    else
+      gbet[j > 0 ? j - 1 : 0] = -x * r;
+  }
+  // tau = sum_s |beta0 - beta_s| / M  (derivative of |x| taken as +1 at x = 0)
+  gtau *= iM;
+#pragma unroll
+  for (int s = 0; s < kMaxSub; ++s) {
+    if (s >= M) continue;
+    const double g = (beta0 - bet[s]) < 0.0 ? -gtau : gtau;
+    gbeta0 += g;
+    // beta_s = |b_s|^2; b_s becomes its own cotangent
+    const double x = 2.0 * (gbet[s] - g), cs = w[s + 1] * iS - corr;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) b[s][t] = cs * gC[t] + x * b[s][t];
+  }
+  // beta0
+#pragma unroll
+  for (int n = 0; n < 3; ++n) ga[n] += 2.0 * a[n] * gbeta0;
+  ga[3] += (4.0 * hx[0] + 8.0 * a[3]) * gbeta0;
+  ga[4] += (4.0 * hy[1] + 8.0 * a[4]) * gbeta0;
+  ga[5] += (4.0 * hz[2] + 8.0 * a[5]) * gbeta0;
+  ga[6] += (2.0 * hx[1] + 2.0 * hy[0] + 2.0 * a[6]) * gbeta0;
+  ga[7] += (2.0 * hx[2] + 2.0 * hz[0] + 2.0 * a[7]) * gbeta0;
+  ga[8] += (2.0 * hy[2] + 2.0 * hz[1] + 2.0 * a[8]) * gbeta0;
+  // a = A+ dq, b_s = B_s dq|S_s
+#pragma unroll 2
+  for (int k = 0; k < KT; ++k) {
+    double s = 0.0;
+#pragma unroll
+    for (int n = 0; n < 9; ++n) s += A[(9 * k + n) * kTile] * ga[n];
+    col[kS * k] = s;
+  }
+  {
+    const double* e = Bt;
+#pragma unroll
+    for (int s = 0; s < kMaxSub; ++s) {
+      const int cs = (int)((cnt >> (8 * s)) & 0xffu);
+      for (int j = 0; j < cs; ++j, e += 4 * kTile) {
+        const double2 x = *reinterpret_cast<const double2*>(e);
+        const double2 y = *reinterpret_cast<const double2*>(e + 2);
+        if (s < M) col[kS * (int)y.y] += x.x * b[s][0] + x.y * b[s][1] + y.x * b[s][2];
+      }
+    }
+  }
+  const int K = st_ptr[i + 1] - st_ptr[i];  // the cell's own members (tile padding excluded)
+  double* gdqc = gdq + (row0 * 5 + v) * kTile + lane;
+  for (int k = 0; k < KT; ++k) {
+    const double g = col[kS * k];
+    gQ0 -= g;
+    gdqc[5 * k * kTile] = k < K ? g : 0.0;
+  }
+  gq0[v * nc + i] = gQ0;
 }
 
 // One boundary plane's map of a ghost cell's flow variables (as k_ghost_fill applies it):
@@ -515,10 +538,14 @@ void launch_vjp(const DevMesh& m, const Geo64& g64, const GeoR<double>& g, const
                                                   gL, gLt, g64.vol, m.nc, fp, m.wall64, dt,
                                                   p.gp_fallback, g64.mom, g64.h, gpf, flag);
   k_vjp_poly<<<blocks_for(m.nc, 128), 128, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, gpf, gpc);
-  k_vjp_recon<<<blocks_for(m.nc, 64), 64, 0, st>>>(m.nc, QA, m.t_K, m.t_cnt, m.t_st, m.t_sb,
-                                                     m.t_idx, m.st_ptr, m.n_sub, g.Ap, g.Bp, g64.mom,
-                                                     g64.h, p.weno_gamma, p.weno_eps, p.weno_pow, gpc,
-                                                     gdq, gq0);
+  int kmax = 0;  // largest stencil of a tile: a column of each thread's differences
+  for (int r = 0; r < m.rr.n; ++r) kmax = m.rr.K[r] > kmax ? m.rr.K[r] : kmax;
+  const size_t smem = sizeof(double) * kVjpThreads * kmax;
+  if (smem > 48 * 1024)
+    cudaFuncSetAttribute(k_vjp_recon, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  k_vjp_recon<<<(unsigned)m.n_tiles, kVjpThreads, smem, st>>>(
+      m.nc, QA, m.t_K, m.t_cnt, m.t_st, m.t_sb, m.t_idx, m.st_ptr, g.Ap, g.Bp, g.cell,
+      p.weno_gamma, p.weno_eps, p.weno_pow, gpc, gdq, gq0);
   k_vjp_stencil<<<blocks_for(m.nc, 128), 128, 0, st>>>(m.nc, rs_ptr, rs_pos, m.t_idx, m.g_map,
                                                         m.g_chain, m.bcs, fp, m.wall64, QA,
                                                         gdq, gq0, gQ);
