@@ -518,7 +518,9 @@ void launch_vjp(const DevMesh& m, const Geo64& g64, const GeoR<double>& g, const
                 const double* QA, const double* poly, const double* gL, const double* gLt,
                 double dt, double* gpf, double* gpc, double* gdq, double* gq0, double* gQ,
                 const int32_t* rs_ptr, const int32_t* rs_pos, int* flag, cudaStream_t st) {
-  const FluxParams<double> fp = flux_params(p);
+  FluxParams<double> fp = flux_params(p);
+  fp.erfc_tab = m.erfc_tab;
+  fp.idt = 1.0 / dt;
   using Kern = decltype(&k_vjp_flux<true, true, true>);
   const Kern tab[2][2][2] = {
       {{k_vjp_flux<false, false, false>, k_vjp_flux<false, false, true>},

@@ -641,6 +641,7 @@ gks_status gks_init(const gks_mesh* mesh, const gks_params* p, void* stream, gks
     int S = 0, M = 0;
     for (int q = 0; q < kMaxSub; ++q) {
       const int c = (int)((h.t_cnt[t] >> (8 * q)) & 0xffu);
+    if ((e = supload(s, &m.erfc_tab, erfc_table())) != cudaSuccess) return bad("upload");
       S += c;
       if (c) M = q + 1;
     }

@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <vector>
 
 #include "gks_internal.h"
 
@@ -110,6 +111,7 @@ struct DevMesh {
   // [6][kPlaneStride] in FP64 and FP32 (see WallData)
   double* wall64 = nullptr;
   float* wall32 = nullptr;
+  double* erfc_tab = nullptr;  // table of half_erfc (FP64 flux and its adjoint)
 };
 template <class R>
 inline const R* wall_table(const DevMesh& m);
@@ -183,6 +185,9 @@ struct ForkJoin {
 template <class R>
 void launch_recon(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* QA,
                   R* poly, int* flag, cudaStream_t st, const ForkJoin* fj = nullptr);
+// The table of half_erfc (gks_kinetic.cuh): a constant of 41 KB, computed on the host in extended
+// precision at the first use (1.3 ms).
+const std::vector<double>& erfc_table();
 // Kernel launches of one launch_recon.
 int recon_launches(const DevMesh& m);
 template <class R>

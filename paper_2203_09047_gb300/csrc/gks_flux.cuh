@@ -45,7 +45,7 @@ GKS_HD R dotU(const Prim<R>& w, R x, R y, R z) {
 
 // s is an int, or a packed pair of signs when R carries both sides.
 template <class R, class Sg>
-GKS_HD void side_init(const R n[3], Sg s, Side<R>& h) {
+GKS_HD void side_init(const double*, const R n[3], Sg s, Side<R>& h) {
   const Prim<R>& w = h.w;
   h.Un = dotU(w, n[0], n[1], n[2]);
   h.u2h = R(0.5) * dotU(w, w.U, w.V, w.W);
@@ -53,6 +53,24 @@ GKS_HD void side_init(const R n[3], Sg s, Side<R>& h) {
   const R x = sl * h.Un;
   h.A = R(0.5) * k_erfc(-R(s) * x);
   h.sB = R(s) * k_div(R(0.28209479177387814) * k_exp(-x * x), sl);  // 1/(2 sqrt(pi))
+  h.be = w.rho * h.sB;
+}
+GKS_HD void side_init(const double* tab, const double n[3], int s, Side<double>& h) {
+  const Prim<double>& w = h.w;
+  h.Un = dotU(w, n[0], n[1], n[2]);
+  h.u2h = 0.5 * dotU(w, w.U, w.V, w.W);
+#ifdef __CUDA_ARCH__
+  const double rs = rsqrt(w.lam);
+#else
+  const double rs = 1.0 / sqrt(w.lam);
+#endif
+  const double x = w.lam * rs * h.Un;
+  double d;
+  if (!half_erfc(tab, -s * x, h.A, d)) {
+    h.A = 0.5 * erfc(-s * x);
+    d = -0.56418958354775629 * exp(-x * x);  // 1/sqrt(pi)
+  }
+  h.sB = -0.5 * s * d * rs;
   h.be = w.rho * h.sB;
 }
 // dA0 = s B z and d(s B) = -s B (Un z + dlam / (2 lam)), z = lam (2 dUn + Un dlam / lam).
@@ -99,10 +117,10 @@ GKS_HD void time_slope(const Prim<R>& w, R Ep, const Advect<R>& a, const R dp[3]
 // form the non-equilibrium terms N[0] = F+(W), N[1] = sum_d D<u c_d psi>[dq_d],
 // N[2] = DF+[rho <A psi>]. The caller formed h.w from q (to_prim).
 template <class R, class Sg>
-GKS_HD void side_terms(int full, R gm1, const R q[5], const R g[5][3], const R n[3], Sg s,
-                       Side<R>& h, R q0[5], R dW[5][3], R N[3][5]) {
+GKS_HD void side_terms(int full, const double* tab, R gm1, const R q[5], const R g[5][3],
+                       const R n[3], Sg s, Side<R>& h, R q0[5], R dW[5][3], R N[3][5]) {
   const Prim<R>& w = h.w;
-  side_init(n, s, h);
+  side_init(tab, n, s, h);
   const R hU = R(0.5) * h.Un;
   q0[0] = h.A * q[0];
 #pragma unroll
@@ -196,10 +214,10 @@ struct FitWeights {
   R n[3], t[3];
 };
 template <class R>
-GKS_HD void fit_weights(R tau, R dt, FitWeights<R>& f) {
+GKS_HD void fit_weights(R tau, R dt, R idt0, FitWeights<R>& f) {
   const R e = tau > R(0) ? k_exp(k_div(R(-0.5) * dt, tau)) : R(0);
   const R x = R(1) - e, s = x * x, m = x * (R(2) + x);
-  const R idt = k_div(R(1), dt), a = tau * idt, b = R(4) * a * idt;
+  const R idt = idt0 != R(0) ? idt0 : R(k_div(R(1), dt)), a = tau * idt, b = R(4) * a * idt;
   f.n[0] = a * m;
   f.t[0] = -b * s;
   f.n[2] = -tau * f.n[0];
@@ -239,7 +257,7 @@ GKS_HD bool interface_flux(const FluxParams<R>& P, const R q0[5], const R dW[5][
     E2[4] = r * w.ir * Ep + Un * (t[4] + dpt);
   }
   const R x = k_abs(k_div(pl - pr, pl + pr));
-  const R tau = collision_time(P, p, w.ir, x, dt);
+  const R tau = collision_time(P, p, w.ip, w.ir, x, dt);
   // E1 = rho0 <u (ab . c) psi>_0; multiplied by tau, so zero without a collision-time model
   if (P.tau_model != 0) {
     R Nn[5];
@@ -272,7 +290,7 @@ GKS_HD bool interface_flux(const FluxParams<R>& P, const R q0[5], const R dW[5][
   }
   if (full_terms(P)) {
     FitWeights<R> f;
-    fit_weights(tau, dt, f);
+    fit_weights(tau, dt, P.idt, f);
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
       const R d0 = N[0][q] - E0[q], d1 = N[1][q] - E1[q], d2 = N[2][q] - E2[q];
@@ -308,10 +326,10 @@ GKS_HD bool gp_flux_global(const FluxParams<R>& P, const R vl[5], const R gl[5][
   const R gm1 = P.gamma - R(1);
   const bool full = full_terms(P);
   R q0[5], dW[5][3], N[3][5];
-  side_terms(full, gm1, vl, gl, n, +1, hl, q0, dW, N);
+  side_terms(full, P.erfc_tab, gm1, vl, gl, n, +1, hl, q0, dW, N);
   {
     R q[5], d[5][3], M[3][5];
-    side_terms(full, gm1, vr, gr, n, -1, hr, q, d, M);
+    side_terms(full, P.erfc_tab, gm1, vr, gr, n, -1, hr, q, d, M);
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       q0[v] += q[v];

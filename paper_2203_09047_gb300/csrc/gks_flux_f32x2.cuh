@@ -29,7 +29,7 @@ __device__ __forceinline__ bool gp_flux_global2(const FluxParams<float>& P, cons
     Side<P2> h;
     if (!to_prim(q, P2(P.gamma), h.w)) return false;
     P2 Q[5], D[5][3], M[3][5];
-    side_terms(full, P2(P.gamma - 1.f), q, g, n, sg, h, Q, D, M);
+    side_terms(full, nullptr, P2(P.gamma - 1.f), q, g, n, sg, h, Q, D, M);
     pl = h.w.p.lo();
     pr = h.w.p.hi();
 #pragma unroll

@@ -385,10 +385,10 @@ GKS_HD bool gp_flux_global_vjp(const FluxParams<double>& P, const double vl[5],
   Side<double> hl, hr;
   if (!(to_prim(vl, P.gamma, hl.w) & to_prim(vr, P.gamma, hr.w))) return false;
   double q0[5], dW[5][3], N[3][5];
-  side_terms(full, gm1, vl, gl, n, +1, hl, q0, dW, N);
+  side_terms(full, P.erfc_tab, gm1, vl, gl, n, +1, hl, q0, dW, N);
   {
     double q[5], d[5][3], M[3][5];
-    side_terms(full, gm1, vr, gr, n, -1, hr, q, d, M);
+    side_terms(full, P.erfc_tab, gm1, vr, gr, n, -1, hr, q, d, M);
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       q0[v] += q[v];
@@ -424,7 +424,7 @@ GKS_HD bool gp_flux_global_vjp(const FluxParams<double>& P, const double vl[5],
     const double dpt = gm1 * (t[4] - dotU(w, t[1], t[2], t[3]) + u2h * t[0]);
     const double sdp = hl.w.p >= hr.w.p ? 1.0 : -1.0, spp = hl.w.p + hr.w.p;
     const double jump = sdp * (hl.w.p - hr.w.p) / spp;
-    const double tau = collision_time(P, p, w.ir, jump, dt);
+    const double tau = collision_time(P, p, w.ip, w.ir, jump, dt);
     // ---- reverse of the combination
     double gE0[5], gE1[5], gE2[5], gtau = 0.0;
     double Nn[5] = {0, 0, 0, 0, 0}, rj[3], Np = 0, nH = 0, E10 = 0;
@@ -456,7 +456,7 @@ GKS_HD bool gp_flux_global_vjp(const FluxParams<double>& P, const double vl[5],
       }
       FitWeights<double> f, df;
       if (full) {
-        fit_weights(tau, dt, f);
+        fit_weights(tau, dt, P.idt, f);
         fit_weights_dtau(tau, dt, df);
       }
 #pragma unroll

@@ -3,12 +3,42 @@
 // hand-written adjoint be checked on a CPU (against the oracle and finite differences). One
 // device entry runs the FP32 Gauss-point flux in its scalar and its packed f32x2 instantiation
 // side by side, a direct test of the pair arithmetic.
+#include <cmath>
 #include <cstdint>
+#include <vector>
 
 #include <cuda_runtime.h>
 
+#include "gks_device.cuh"
 #include "gks_flux_f32x2.cuh"
 #include "gks_kinetic_adj.cuh"
+
+// Taylor coefficients of erfc(z)/2 about z = i/64: c_0 = erfc(z)/2 and
+// c_(k+1) = -(-1)^k H_k(z) exp(-z^2) / (sqrt(pi) (k+1)!), H_k the Hermite polynomials.
+static std::vector<double> make_erfc_table() {
+  using namespace gks;
+  typedef long double L;
+  std::vector<double> tab((size_t)kErfcTerms * kErfcRecords);
+  for (int i = 0; i < kErfcRecords; ++i) {
+    const L z = (L)(i - kErfcSteps * kErfcMax) / kErfcSteps;
+    double* c = tab.data() + (size_t)kErfcTerms * i;
+    c[0] = (double)(0.5L * erfcl(z));
+    const L d1 = -expl(-z * z) / sqrtl(acosl(-1.0L));
+    L hm = 0, h = 1, fact = 1;
+    for (int k = 0; k + 1 < kErfcTerms; ++k) {
+      fact *= k + 1;
+      c[k + 1] = (double)(d1 * ((k & 1) ? -h : h) / fact);
+      const L hn = 2 * z * h - 2 * k * hm;
+      hm = h;
+      h = hn;
+    }
+  }
+  return tab;
+}
+const std::vector<double>& gks::erfc_table() {
+  static const std::vector<double> tab = make_erfc_table();
+  return tab;
+}
 
 namespace {
 gks::FluxParams<double> params_from(const double* p) {
@@ -25,6 +55,7 @@ gks::FluxParams<double> params_from(const double* p) {
   P.pr_fix = 1.0 / p[6] - 1.0;
   P.T_ref = p[7];
   P.mu_pow = p[8];
+  P.erfc_tab = gks::erfc_table().data();  // as the kernels
   return P;
 }
 // the wall plane of `code` from p's wall_u[6][3], wall_T[6]
@@ -111,6 +142,14 @@ extern "C" int gks_gp_face_host(const double* p, const double* vl, const double*
       ggr[3 * v + a] = gGR[v][a];
     }
   return 0;
+}
+
+// half_erfc at n points: f = erfc(z)/2, d = -exp(-z^2)/sqrt(pi); returns the number of points the
+// table does not cover (left as they are).
+extern "C" int gks_half_erfc_host(int n, const double* z, double* f, double* d) {
+  int out = 0;
+  for (int i = 0; i < n; ++i) out += gks::half_erfc(gks::erfc_table().data(), z[i], f[i], d[i]) ? 0 : 1;
+  return out;
 }
 
 // The wall ghost at a Gauss point (value, gradient [5][3]) for wall code `code`, and, when gvg is

@@ -757,7 +757,8 @@ __device__ __forceinline__ void first_order_if_nonphysical(const R* __restrict__
 // gradients rotated to the normal and two tangents, one moment derivative per axis), per
 // launch: FP32 smooth 0.418 -> 0.326 ms (64^3-cube mesh, 2.39 M faces), FP32 full 326 -> 231 us
 // (48^3-cube explosion, 1.02 M faces), FP64 smooth 2.53 -> 1.77 ms (32^3 cubes, 299 k faces),
-// FP64 full 2.05 -> 1.31 ms (124 k faces of tetrahedra). Resident blocks per SM, measured on
+// FP64 full 2.05 -> 1.31 ms (124 k faces of tetrahedra); with erfc and exp from one table and one
+// division per state (half_erfc, to_prim) FP64 1.49 and 1.20 ms. Resident blocks per SM, measured on
 // the same meshes: FP32 smooth 6 (0.326 ms; 4, 5, 7 and 8 blocks 0.380, 0.354, 0.333 and
 // 0.356); FP32 full 4 (231 us; 3 and 5 blocks 254 and 254); FP64 unbounded (2 blocks equal; 3
 // and 4 blocks 1 and 3 % slower).
@@ -1646,7 +1647,9 @@ void launch_recon(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const
 template <class R>
 void launch_flux(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* poly,
                  const R* QA, double dt, R* fface, int* flag, cudaStream_t st) {
-  const FluxParams<R> fp = flux_params(p);
+  FluxParams<R> fp = flux_params(p);
+  fp.erfc_tab = m.erfc_tab;
+  fp.idt = (R)(1.0 / dt);
   const unsigned nb = blocks_for(4 * m.nf, 128);
   // without a collision time the full form is the smooth one (its non-equilibrium terms carry
   // the weight tau = 0)

@@ -61,6 +61,55 @@ GKS_HD bool to_prim(const R q[5], R gamma, Prim<R>& w) {
   w.hil = w.p * w.ir;
   return (w.rho > R(0)) && (w.p > R(0));  // false also for NaN
 }
+// FP64: both reciprocals from one division, 1 / (rho rho p) (a division is a chain of about ten
+// instructions on the FP64 pipe, which bounds the FP64 kernels).
+GKS_HD bool to_prim(const double q[5], double gamma, Prim<double>& w) {
+  w.rho = q[0];
+  const double rp = (gamma - 1.0) *
+                    (q[0] * q[4] - 0.5 * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]));  // rho p
+  const double r = 1.0 / (q[0] * rp);
+  w.ir = rp * r;
+  w.U = q[1] * w.ir;
+  w.V = q[2] * w.ir;
+  w.W = q[3] * w.ir;
+  w.p = rp * w.ir;
+  w.ip = q[0] * q[0] * r;
+  w.lam = 0.5 * w.rho * w.ip;
+  w.hil = w.p * w.ir;
+  return (w.rho > 0.0) && (w.p > 0.0);
+}
+
+// erfc(z) / 2 and its derivative -exp(-z^2) / sqrt(pi) in FP64 from one table: Taylor
+// polynomials of degree 9 about the points i / 64, |i| <= 256 (coefficients f^(k) / k! from the
+// Hermite recurrence, filled on the host in extended precision). |z - i/64| <= 1/128, so the
+// remainder is below 2^-53 of either value up to |z| = 4; beyond it the library functions. Both
+// values take 17 FMAs and one record of 80 bytes, where erfc and exp take about five times that
+// on the FP64 pipe (k_flux FP64 1.77 -> 1.49 ms with the single division of to_prim, smooth form,
+// 299 k faces); largest errors over 20,000 points 1.9 and 2.8 times 2^-53.
+constexpr int kErfcSteps = 64, kErfcMax = 4, kErfcTerms = 10;
+constexpr int kErfcRecords = 2 * kErfcSteps * kErfcMax + 1;
+GKS_HD bool half_erfc(const double* tab, double z, double& f, double& d) {
+  if (!(tab && k_abs(z) < (double)kErfcMax)) return false;
+  const int i = (int)(z * kErfcSteps + (z < 0.0 ? -0.5 : 0.5));
+  const double t = z - (double)i * (1.0 / kErfcSteps);
+  const double2* c = reinterpret_cast<const double2*>(tab + kErfcTerms * (i + kErfcSteps * kErfcMax));
+  double k[kErfcTerms];
+#pragma unroll
+  for (int j = 0; j < kErfcTerms / 2; ++j) {
+    const double2 x = c[j];
+    k[2 * j] = x.x;
+    k[2 * j + 1] = x.y;
+  }
+  f = k[kErfcTerms - 1];
+  d = f;
+  f = f * t + k[kErfcTerms - 2];
+#pragma unroll
+  for (int j = kErfcTerms - 3; j >= 0; --j) {
+    d = d * t + f;
+    f = f * t + k[j];
+  }
+  return true;
+}
 
 template <class R>
 struct FluxParams {
@@ -68,6 +117,8 @@ struct FluxParams {
   int full, tau_model;
   R pr_fix = R(0);  // 1/Pr - 1 (heat-flux correction of the smooth flux; 0 for the BGK value)
   R T_ref = R(1), mu_pow = R(0.7);  // power law mu (T / T_ref)^mu_pow (collision time 3)
+  const double* erfc_tab = nullptr; // table of half_erfc (FP64 path; null: the library functions)
+  R idt = R(0);                     // 1/dt where the caller has it (0: formed per point)
 };
 
 // One boundary plane: no-slip wall velocity and temperature (<= 0: adiabatic), far-field state
@@ -113,11 +164,11 @@ inline FluxParams<R> flux_params(const KP<R>& p) {
 // Collision time of the interface (Section 5): zero; inviscid (eps + C dp) dt; viscous
 // mu / p0 + C dp dt, with mu constant or the power law of Section 5.4 at T0 = p0 / rho0.
 template <class R>
-GKS_HD R collision_time(const FluxParams<R>& P, R p0, R ir0, R dp, R dt) {
+GKS_HD R collision_time(const FluxParams<R>& P, R p0, R ip0, R ir0, R dp, R dt) {
   if (P.tau_model == 1) return (P.tau_eps + P.tau_C * dp) * dt;
-  if (P.tau_model == 2) return k_div(P.mu, p0) + P.tau_C * dp * dt;
+  if (P.tau_model == 2) return P.mu * ip0 + P.tau_C * dp * dt;
   if (P.tau_model == 3)
-    return k_div(P.mu * k_pow(k_div(p0 * ir0, P.T_ref), P.mu_pow), p0) + P.tau_C * dp * dt;
+    return P.mu * k_pow(k_div(p0 * ir0, P.T_ref), P.mu_pow) * ip0 + P.tau_C * dp * dt;
   return R(0);
 }
 
