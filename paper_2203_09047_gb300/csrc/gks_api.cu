@@ -50,7 +50,6 @@ struct gks_solver {
   // Q is its FP64 [5][nc] form, refreshed from QA when a call needs it (q_stale after steps).
   double* Q = nullptr;      // [5][nc]
   bool q_stale = false;
-  double* Qs = nullptr;     // staging for the residual calls
   double* L = nullptr;      // stage-1 L, Lt [5][nc]: 8 bytes per value (FP64, or a float-float
   double* Lt = nullptr;     // pair on the FP32 path)
   double* tmp = nullptr;    // staging in caller order [5][nc]
@@ -77,8 +76,7 @@ struct gks_solver {
   // adjoint (allocated on the first gks_residual_vjp call)
   bool vjp_ready = false;
   GeoR<double> gv;             // FP64 geometry (the solver's own in FP64 mode)
-  double* vQ = nullptr;        // internal-order state [5][nc]
-  double* vQA = nullptr;       // its FP64 gather copy [nc][6]
+  double* vQA = nullptr;       // FP64 gather copy of the state [nc][6]
   double* vpoly = nullptr;     // FP64 polynomials [nc][kPolyStride]
   double* vgL = nullptr;       // internal-order cotangents [5][nc]
   double* vgLt = nullptr;
@@ -233,11 +231,36 @@ void residual_any(gks_solver* s, const void* QinA, double dt, int mode, double* 
 }
 
 // Caller-order state -> internal order (dst) and its gather copy (gq).
-void permute_in_any(gks_solver* s, const double* src, double* dst, void* gq) {
+void permute_in_any(gks_solver* s, const double* src, double* dst, void* gq, int* flag) {
   if (s->mixed)
-    launch_permute_in<float>(s->m.nc, s->m.perm, src, dst, (float*)gq, s->st);
+    launch_permute_in<float>(s->m.nc, s->m.perm, src, dst, (float*)gq, flag, s->st);
   else
-    launch_permute_in<double>(s->m.nc, s->m.perm, src, dst, (double*)gq, s->st);
+    launch_permute_in<double>(s->m.nc, s->m.perm, src, dst, (double*)gq, flag, s->st);
+}
+
+// Whether the kernels may read and write a caller's state array in place: ordinary device memory
+// of the solver's device from its first to its last byte, aligned to its values. Anything else
+// (host, managed, another device's, unaligned, too short) goes through a staging buffer and a
+// copy, which reports what it cannot reach.
+bool in_place(const gks_solver* s, const void* p) {
+  if (((uintptr_t)p & (sizeof(double) - 1)) != 0) return false;
+  const char* ends[2] = {(const char*)p, (const char*)p + sizeof(double) * 5 * s->m.nc - 1};
+  for (const char* q : ends) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeDevice || a.device != s->device) return false;
+  }
+  return true;
+}
+// A caller's input array on the device: itself, or its copy in stage.
+cudaError_t input_of(gks_solver* s, const double* p, double* stage, const double** out) {
+  *out = p;
+  if (in_place(s, p)) return cudaSuccess;
+  *out = stage;
+  return cudaMemcpyAsync(stage, p, sizeof(double) * 5 * s->m.nc, cudaMemcpyDefault, s->st);
 }
 
 // Refresh the FP64 form of the state from its gather copy after steps.
@@ -618,6 +641,7 @@ gks_status gks_init(const gks_mesh* mesh, const gks_params* p, void* stream, gks
     for (size_t k = 0; k < w64.size(); ++k) w32[k] = (float)w64[k];
     if ((e = supload(s, &m.wall64, w64)) != cudaSuccess) return bad("upload");
     if ((e = supload(s, &m.wall32, w32)) != cudaSuccess) return bad("upload");
+    if ((e = supload(s, &m.erfc_tab, erfc_table())) != cudaSuccess) return bad("upload");
     m.ng = (int64_t)gsrc.size();
     if (m.ng > 0) {
       if ((e = supload(s, &m.g_src, gsrc)) != cudaSuccess) return bad("upload");
@@ -641,7 +665,6 @@ gks_status gks_init(const gks_mesh* mesh, const gks_params* p, void* stream, gks
     int S = 0, M = 0;
     for (int q = 0; q < kMaxSub; ++q) {
       const int c = (int)((h.t_cnt[t] >> (8 * q)) & 0xffu);
-    if ((e = supload(s, &m.erfc_tab, erfc_table())) != cudaSuccess) return bad("upload");
       S += c;
       if (c) M = q + 1;
     }
@@ -691,7 +714,6 @@ gks_status gks_init(const gks_mesh* mesh, const gks_params* p, void* stream, gks
   if ((e = salloc(s, &s->g.hdt, nc)) != cudaSuccess) return bad("alloc");
   if ((e = salloc(s, &s->g.farea, nf)) != cudaSuccess) return bad("alloc");
   if ((e = salloc(s, &s->Q, 5 * nc)) != cudaSuccess) return bad("alloc");
-  if ((e = salloc(s, &s->Qs, 5 * nc)) != cudaSuccess) return bad("alloc");
   if ((e = salloc(s, &s->L, 5 * nc)) != cudaSuccess) return bad("alloc");
   if ((e = salloc(s, &s->Lt, 5 * nc)) != cudaSuccess) return bad("alloc");
   if ((e = salloc(s, &s->tmp, 5 * nc)) != cudaSuccess) return bad("alloc");
@@ -737,10 +759,10 @@ gks_status gks_init(const gks_mesh* mesh, const gks_params* p, void* stream, gks
 
 gks_status gks_set_state(gks_solver* s, const double* Q) {
   if (!s || !Q) return GKS_E_INVAL;
-  const int64_t nc = s->m.nc;
-  cudaError_t e = cudaMemcpyAsync(s->tmp, Q, sizeof(double) * 5 * nc, cudaMemcpyDefault, s->st);
+  const double* q = nullptr;
+  cudaError_t e = input_of(s, Q, s->tmp, &q);
   if (e != cudaSuccess) return s->cuda_fail(e, "set_state copy");
-  permute_in_any(s, s->tmp, s->Q, s->QA);
+  permute_in_any(s, q, s->Q, s->QA, nullptr);
   s->q_stale = false;
   e = cudaGetLastError();
   return e == cudaSuccess ? GKS_OK : s->cuda_fail(e, "set_state");
@@ -749,9 +771,17 @@ gks_status gks_set_state(gks_solver* s, const double* Q) {
 gks_status gks_get_state(gks_solver* s, double* Q) {
   if (!s || !Q) return GKS_E_INVAL;
   const int64_t nc = s->m.nc;
-  sync_q(s);
-  launch_permute_out(nc, s->m.perm, s->Q, s->tmp, s->st);
-  cudaError_t e = cudaMemcpyAsync(Q, s->tmp, sizeof(double) * 5 * nc, cudaMemcpyDefault, s->st);
+  const bool direct = in_place(s, Q);
+  double* dst = direct ? Q : s->tmp;
+  if (!s->q_stale)
+    launch_permute_out(nc, s->m.perm, s->Q, dst, s->st);
+  else if (s->mixed)
+    launch_unpack_out<float>(nc, s->m.perm, (const float*)s->QA, dst, s->st);
+  else
+    launch_unpack_out<double>(nc, s->m.perm, (const double*)s->QA, dst, s->st);
+  cudaError_t e = cudaGetLastError();
+  if (e == cudaSuccess && !direct)
+    e = cudaMemcpyAsync(Q, dst, sizeof(double) * 5 * nc, cudaMemcpyDefault, s->st);
   if (e != cudaSuccess) return s->cuda_fail(e, "get_state copy");
   e = cudaStreamSynchronize(s->st);
   return e == cudaSuccess ? GKS_OK : s->cuda_fail(e, "get_state");
@@ -759,18 +789,25 @@ gks_status gks_get_state(gks_solver* s, double* Q) {
 
 gks_status gks_max_dt(gks_solver* s, double cfl, double* dt) {
   if (!s || !dt || !(cfl > 0)) return GKS_E_INVAL;
-  sync_q(s);
-  launch_check_state(s->m.nc, s->Q, s->prm.gamma, s->flag, s->st);
+  // the gather copy is the state, except that the FP64-update mode steps an FP64 master copy
+  if (s->fp64upd) sync_q(s);
   const int nb = dt_blocks(s->m.nc);
-  launch_dt(s->m.nc, s->Q, s->g.hdt, s->prm.gamma, s->prm.mu,
-            s->prm.tau_model == GKS_TAU_POWER_LAW, s->prm.T_ref, s->prm.mu_pow, s->dt_part, nb,
-            s->dt_out, s->st);
+  const gks_params& p = s->prm;
+  const int power = p.tau_model == GKS_TAU_POWER_LAW;
+  if (s->mixed)
+    launch_dt<float>(s->m.nc, (const float*)s->QA, s->fp64upd ? s->Q : nullptr, s->g.hdt, p.gamma,
+                     p.mu, power, p.T_ref, p.mu_pow, s->dt_part, nb, s->dt_out, s->flag, s->st);
+  else
+    launch_dt<double>(s->m.nc, (const double*)s->QA, nullptr, s->g.hdt, p.gamma, p.mu, power,
+                      p.T_ref, p.mu_pow, s->dt_part, nb, s->dt_out, s->flag, s->st);
+  // the bound and the status word in one wait
+  double bound = 0.0;
+  cudaError_t e = cudaMemcpyAsync(s->h_dt + 1, s->dt_out, sizeof(double), cudaMemcpyDeviceToHost, s->st);
+  if (e != cudaSuccess) return s->cuda_fail(e, "max_dt");
   gks_status r = check_and_clear(s);
   if (r != GKS_OK) return r;
-  cudaError_t e = cudaMemcpyAsync(s->h_dt, s->dt_out, sizeof(double), cudaMemcpyDeviceToHost, s->st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
-  if (e != cudaSuccess) return s->cuda_fail(e, "max_dt");
-  *dt = cfl * s->h_dt[0];
+  bound = s->h_dt[1];
+  *dt = cfl * bound;
   return GKS_OK;
 }
 
@@ -843,18 +880,18 @@ gks_status gks_check(gks_solver* s) {
 gks_status gks_residual(gks_solver* s, const double* Q, double dt, double* L, double* Lt) {
   if (!s || !Q || !L || !Lt || !(dt > 0)) return GKS_E_INVAL;
   const int64_t nc = s->m.nc;
-  cudaError_t e = cudaMemcpyAsync(s->tmp, Q, sizeof(double) * 5 * nc, cudaMemcpyDefault, s->st);
+  const double* q = nullptr;
+  cudaError_t e = input_of(s, Q, s->tmp, &q);
   if (e != cudaSuccess) return s->cuda_fail(e, "residual copy");
-  permute_in_any(s, s->tmp, s->Qs, s->QsA);
-  launch_check_state(nc, s->Qs, s->prm.gamma, s->flag, s->st);
-  residual_any(s, s->QsA, dt, 0, s->tmp, s->tmp2);
-  // tmp, tmp2 hold L, Lt in internal order; write them out in caller order
-  launch_permute_out(nc, s->m.perm, s->tmp, s->Qs, s->st);
-  e = cudaMemcpyAsync(L, s->Qs, sizeof(double) * 5 * nc, cudaMemcpyDefault, s->st);
-  if (e != cudaSuccess) return s->cuda_fail(e, "residual copy out");
-  launch_permute_out(nc, s->m.perm, s->tmp2, s->tmp, s->st);
-  e = cudaMemcpyAsync(Lt, s->tmp, sizeof(double) * 5 * nc, cudaMemcpyDefault, s->st);
-  if (e != cudaSuccess) return s->cuda_fail(e, "residual copy out");
+  permute_in_any(s, q, nullptr, s->QsA, s->flag);
+  // L and Lt leave the face sums in caller order, in place or through a staging buffer
+  const bool inL = in_place(s, L), inLt = in_place(s, Lt);
+  residual_any(s, s->QsA, dt, 0, inL ? L : s->tmp, inLt ? Lt : s->tmp2);
+  const size_t bytes = sizeof(double) * 5 * nc;
+  if (!inL && (e = cudaMemcpyAsync(L, s->tmp, bytes, cudaMemcpyDefault, s->st)) != cudaSuccess)
+    return s->cuda_fail(e, "residual copy out");
+  if (!inLt && (e = cudaMemcpyAsync(Lt, s->tmp2, bytes, cudaMemcpyDefault, s->st)) != cudaSuccess)
+    return s->cuda_fail(e, "residual copy out");
   e = cudaGetLastError();
   if (e != cudaSuccess) return s->cuda_fail(e, "residual launch");
   return check_and_clear(s);
@@ -875,8 +912,7 @@ gks_status gks_residual_vjp(gks_solver* s, const double* Q, double dt, const dou
     } else {
       s->gv = s->gd;
     }
-    if ((e = salloc(s, &s->vQ, 5 * nc)) != cudaSuccess ||
-        (e = salloc(s, &s->vQA, 6 * (nc + s->m.ng))) != cudaSuccess ||
+    if ((e = salloc(s, &s->vQA, 6 * (nc + s->m.ng))) != cudaSuccess ||
         (e = salloc(s, &s->vpoly, (int64_t)kPolyStride * nc)) != cudaSuccess ||
         (e = salloc(s, &s->vgL, 5 * nc)) != cudaSuccess ||
         (e = salloc(s, &s->vgLt, 5 * nc)) != cudaSuccess ||
@@ -888,25 +924,23 @@ gks_status gks_residual_vjp(gks_solver* s, const double* Q, double dt, const dou
       return s->cuda_fail(e, "vjp buffers");
     s->vjp_ready = true;
   }
-  const size_t bytes = sizeof(double) * 5 * nc;
-  // inputs to internal order
-  if ((e = cudaMemcpyAsync(s->tmp, Q, bytes, cudaMemcpyDefault, s->st)) != cudaSuccess)
-    return s->cuda_fail(e, "vjp copy");
-  launch_permute_in<double>(nc, s->m.perm, s->tmp, s->vQ, s->vQA, s->st);
-  launch_check_state(nc, s->vQ, s->prm.gamma, s->flag, s->st);
-  if ((e = cudaMemcpyAsync(s->tmp, gL, bytes, cudaMemcpyDefault, s->st)) != cudaSuccess)
-    return s->cuda_fail(e, "vjp copy");
-  launch_permute_in<double>(nc, s->m.perm, s->tmp, s->vgL, (double*)nullptr, s->st);
-  if ((e = cudaMemcpyAsync(s->tmp, gLt, bytes, cudaMemcpyDefault, s->st)) != cudaSuccess)
-    return s->cuda_fail(e, "vjp copy");
-  launch_permute_in<double>(nc, s->m.perm, s->tmp, s->vgLt, (double*)nullptr, s->st);
+  // inputs to internal order (a staged copy is read before the next one is made)
+  const double* in = nullptr;
+  if ((e = input_of(s, Q, s->tmp, &in)) != cudaSuccess) return s->cuda_fail(e, "vjp copy");
+  launch_permute_in<double>(nc, s->m.perm, in, nullptr, s->vQA, s->flag, s->st);
+  if ((e = input_of(s, gL, s->tmp, &in)) != cudaSuccess) return s->cuda_fail(e, "vjp copy");
+  launch_permute_in<double>(nc, s->m.perm, in, s->vgL, nullptr, nullptr, s->st);
+  if ((e = input_of(s, gLt, s->tmp, &in)) != cudaSuccess) return s->cuda_fail(e, "vjp copy");
+  launch_permute_in<double>(nc, s->m.perm, in, s->vgLt, nullptr, nullptr, s->st);
   // forward reconstruction in FP64, then the reverse passes
   const KParams<double> kp = kparams<double>(s->prm);
   launch_recon<double>(s->m, s->gv, kp, s->vQA, s->vpoly, s->flag, s->st, &s->fj);
   launch_vjp(s->m, s->g, s->gv, kp, s->vQA, s->vpoly, s->vgL, s->vgLt, dt, s->vgpf, s->vgpc,
              s->vgdq, s->vgq0, s->vgQ, s->rs_ptr, s->rs_pos, s->flag, s->st);
-  launch_permute_out(nc, s->m.perm, s->vgQ, s->tmp, s->st);
-  if ((e = cudaMemcpyAsync(gQ, s->tmp, bytes, cudaMemcpyDefault, s->st)) != cudaSuccess)
+  const bool direct = in_place(s, gQ);
+  launch_permute_out(nc, s->m.perm, s->vgQ, direct ? gQ : s->tmp, s->st);
+  if (!direct && (e = cudaMemcpyAsync(gQ, s->tmp, sizeof(double) * 5 * nc, cudaMemcpyDefault,
+                                      s->st)) != cudaSuccess)
     return s->cuda_fail(e, "vjp copy out");
   e = cudaGetLastError();
   if (e != cudaSuccess) return s->cuda_fail(e, "vjp launch");

@@ -193,7 +193,8 @@ int recon_launches(const DevMesh& m);
 template <class R>
 void launch_flux(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* poly,
                  const R* QA, double dt, R* fface, int* flag, cudaStream_t st);
-// Residual output: L = -(1/|Omega|) sum_f s_f F_f and Lt likewise from dF/dt, in FP64.
+// Residual output: L = -(1/|Omega|) sum_f s_f F_f and Lt likewise from dF/dt, in FP64 and in
+// caller order.
 template <class R>
 void launch_gather(const DevMesh& m, const Geo64& g, const R* fface, double* L, double* Lt,
                    cudaStream_t st);
@@ -229,15 +230,22 @@ void launch_jacobi_sweep(const DevMesh& m, const R* fn, const R* QA, const R* Rv
 // The state [5][nc] in FP64 (internal order) from its gather copy.
 template <class R>
 void launch_unpack(int64_t nc, const R* QA, double* Q, cudaStream_t st);
+// The same in caller order.
+template <class R>
+void launch_unpack_out(int64_t nc, const int32_t* perm, const R* QA, double* dst, cudaStream_t st);
+// Caller order -> internal order (dst) and gather copy (gq), either may be null; flag != null
+// checks the state on the way.
 template <class R>
 void launch_permute_in(int64_t nc, const int32_t* perm, const double* src, double* dst, R* gq,
-                       cudaStream_t st);
+                       int* flag, cudaStream_t st);
 void launch_permute_out(int64_t nc, const int32_t* perm, const double* src, double* dst,
                         cudaStream_t st);
-void launch_check_state(int64_t nc, const double* Q, double gamma, int* flag, cudaStream_t st);
-void launch_dt(int64_t nc, const double* Q, const double* hdt, double gamma, double mu, int power,
-               double T_ref, double mu_pow, double* partial, int nblocks, double* out,
-               cudaStream_t st);
+// State check and smallest time-step bound of the state in the gather copy QA (Q64 != null: its
+// FP64 values are Q64 [5][nc]).
+template <class R>
+void launch_dt(int64_t nc, const R* QA, const double* Q64, const double* hdt, double gamma,
+               double mu, int power, double T_ref, double mu_pow, double* partial, int nblocks,
+               double* out, int* flag, cudaStream_t st);
 int dt_blocks(int64_t nc);
 
 // ---- adjoint (gks_adjoint.cu) --------------------------------------------------------------
