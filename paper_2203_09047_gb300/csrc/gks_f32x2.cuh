@@ -1,6 +1,6 @@
 // A pair of FP32 values on Blackwell's packed f32x2 arithmetic (FFMA2, FMUL2, FADD2: two FP32
 // operations per instruction and lane), usable as the scalar type R of the flux templates so
-// that one instantiation computes both sides of a face at once (one side in each half). A
+// that one instantiation computes two Gauss points, or both sides of one, at once. A
 // product is kept pending (M2) and fused into the addition or subtraction that consumes it,
 // since the packed intrinsics are not contracted by the compiler; a pending product used any
 // other way is rounded into a P2 first. Division, square root, exp and erfc run per half.
@@ -61,7 +61,7 @@ __device__ __forceinline__ P2& operator+=(P2& a, const M2& b) { return a = a + b
 __device__ __forceinline__ P2& operator-=(P2& a, const P2& b) { return a = a - b; }
 __device__ __forceinline__ P2& operator-=(P2& a, const M2& b) { return a = a - b; }
 __device__ __forceinline__ P2& operator*=(P2& a, const P2& b) { return a = P2(a * b); }
-// true when it holds in both halves (both sides)
+// true when it holds in both halves
 __device__ __forceinline__ bool operator>(const P2& a, const P2& b) {
   return (a.v.x > b.v.x) && (a.v.y > b.v.y);
 }
@@ -77,6 +77,9 @@ __device__ __forceinline__ P2 k_sqrt(const P2& x) { return P2(sqrtf(x.v.x), sqrt
 __device__ __forceinline__ P2 k_exp(const P2& x) { return P2(expf(x.v.x), expf(x.v.y)); }
 __device__ __forceinline__ P2 k_erfc(const P2& x) { return P2(erfcf(x.v.x), erfcf(x.v.y)); }
 __device__ __forceinline__ P2 k_abs(const P2& x) { return P2(fabsf(x.v.x), fabsf(x.v.y)); }
+__device__ __forceinline__ P2 k_pow(const P2& x, const P2& y) {
+  return P2(powf(x.v.x, y.v.x), powf(x.v.y, y.v.y));
+}
 __device__ __forceinline__ float hsum(const P2& a) { return a.v.x + a.v.y; }
 
 }  // namespace gks

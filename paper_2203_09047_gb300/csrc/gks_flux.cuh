@@ -115,17 +115,29 @@ GKS_HD void time_slope(const Prim<R>& w, R Ep, const Advect<R>& a, const R dp[3]
 
 // One side's part of the interface state q0 and of its gradient dW[v][axis], and for the full
 // form the non-equilibrium terms N[0] = F+(W), N[1] = sum_d D<u c_d psi>[dq_d],
-// N[2] = DF+[rho <A psi>]. The caller formed h.w from q (to_prim).
-template <class R, class Sg>
-GKS_HD void side_terms(int full, const double* tab, R gm1, const R q[5], const R g[5][3],
+// N[2] = DF+[rho <A psi>]; kAdd adds them to the other side's. The caller formed h.w from q
+// (to_prim).
+template <bool kAdd, class R>
+GKS_HD void put(R& x, const R& y) {
+  if (kAdd)
+    x += y;
+  else
+    x = y;
+}
+template <bool kAdd, class R, class Sg>
+GKS_HD void side_terms(bool full, const double* tab, R gm1, const R q[5], const R g[5][3],
                        const R n[3], Sg s, Side<R>& h, R q0[5], R dW[5][3], R N[3][5]) {
   const Prim<R>& w = h.w;
   side_init(tab, n, s, h);
-  const R hU = R(0.5) * h.Un;
-  q0[0] = h.A * q[0];
+  const R hU = R(0.5) * h.Un, hb = R(0.5) * h.be;
+  // sums start from the other side's value, so that adding it costs nothing
+  auto first = [](const R& x, const R& a, const R& b) -> R {
+    return kAdd ? R(x + a * b) : R(a * b);
+  };
+  q0[0] = first(q0[0], h.A, q[0]);
 #pragma unroll
-  for (int a = 0; a < 3; ++a) q0[1 + a] = h.A * q[1 + a] + h.be * n[a];
-  q0[4] = h.A * q[4] + hU * h.be;
+  for (int a = 0; a < 3; ++a) q0[1 + a] = first(q0[1 + a], h.A, q[1 + a]) + h.be * n[a];
+  q0[4] = first(q0[4], h.A, q[4]) + hU * h.be;
   const R U[3] = {w.U, w.V, w.W};
   R dp[3], dA1[3];  // full form only
   R UA, UsB, nA, nsB, nUn;
@@ -134,10 +146,11 @@ GKS_HD void side_terms(int full, const double* tab, R gm1, const R q[5], const R
     SideD<R> e;
     side_der(h, gm1, n, g[0][d], g[1][d], g[2][d], g[3][d], g[4][d], e);
     const R dbe = h.sB * g[0][d] + w.rho * e.dsB;
-    dW[0][d] = e.dA * q[0] + h.A * g[0][d];
+    dW[0][d] = first(dW[0][d], e.dA, q[0]) + h.A * g[0][d];
 #pragma unroll
-    for (int a = 0; a < 3; ++a) dW[1 + a][d] = e.dA * q[1 + a] + h.A * g[1 + a][d] + dbe * n[a];
-    dW[4][d] = e.dA * q[4] + h.A * g[4][d] + hU * dbe + R(0.5) * h.be * e.dUn;
+    for (int a = 0; a < 3; ++a)
+      dW[1 + a][d] = first(dW[1 + a][d], e.dA, q[1 + a]) + h.A * g[1 + a][d] + dbe * n[a];
+    dW[4][d] = first(dW[4][d], e.dA, q[4]) + h.A * g[4][d] + hU * dbe + hb * e.dUn;
     if (full) {
       dp[d] = e.dp;
       dA1[d] = e.dUn * h.A + h.Un * e.dA + e.dsB;
@@ -151,10 +164,10 @@ GKS_HD void side_terms(int full, const double* tab, R gm1, const R q[5], const R
   if (!full) return;
   const R A = h.A, A1 = h.Un * h.A + h.sB, E = q[4], p = w.p;
   const R F4 = R(0.5) * (A1 + h.Un * A);
-  N[0][0] = A1 * q[0];
+  N[0][0] = first(N[0][0], A1, q[0]);
 #pragma unroll
-  for (int a = 0; a < 3; ++a) N[0][1 + a] = A1 * q[1 + a] + (p * A) * n[a];
-  N[0][4] = A1 * E + p * F4;
+  for (int a = 0; a < 3; ++a) N[0][1 + a] = first(N[0][1 + a], A1, q[1 + a]) + (p * A) * n[a];
+  N[0][4] = first(N[0][4], A1, E) + p * F4;
   Advect<R> c;
   advect(w, g, dp, c);
   {
@@ -167,17 +180,18 @@ GKS_HD void side_terms(int full, const double* tab, R gm1, const R q[5], const R
     const R pn = A * Np + p * nA;                   // n . grad (p A0)
     // div (p A0 U) + n . grad (p s B)
     const R pd = p * (A * c.divU + UA) + A * c.Gp + h.sB * Np + p * nsB;
-    N[1][0] = A1 * c.divm + w.rho * UA1 + pn;
+    const R N10 = A1 * c.divm + w.rho * UA1 + pn;
+    put<kAdd>(N[1][0], N10);
     const R Ah = A * w.hil;
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      N[1][1 + j] = U[j] * N[1][0] + A1 * (c.H[j] + dp[j]) + Ah * (Nn[1 + j] - U[j] * Nn[0]) +
-                    n[j] * pd + p * dA1[j];
+      N[1][1 + j] = first(N[1][1 + j], U[j], N10) + A1 * (c.H[j] + dp[j]) +
+                    Ah * (Nn[1 + j] - U[j] * Nn[0]) + n[j] * pd + p * dA1[j];
     const R E3 = E + R(1.5) * p, Ep = E + p;
     const R X = E3 * A1 + (p * A) * hU;
     const R Y = Ep * A + hU * h.be;
     const R nbe = h.sB * Nn[0] + w.rho * nsB;
-    N[1][4] = X * c.divU + (c.G[4] + R(1.5) * c.Gp) * A1 + E3 * UA1 +
+    N[1][4] = first(N[1][4], X, c.divU) + (c.G[4] + R(1.5) * c.Gp) * A1 + E3 * UA1 +
               R(0.5) * (p * (UUn * A + h.Un * UA) + h.Un * A * c.Gp) +
               (Np - w.hil * Nn[0]) * w.ir * Y +
               w.hil * ((Nn[4] + Np) * A + Ep * nA + R(0.5) * (nUn * h.be + h.Un * nbe));
@@ -188,10 +202,11 @@ GKS_HD void side_terms(int full, const double* tab, R gm1, const R q[5], const R
   side_der(h, gm1, n, t[0], t[1], t[2], t[3], t[4], e);
   const R x = e.dUn * A + h.Un * e.dA, y = x + e.dsB;  // d(Un A0), dA1
   const R z = A * e.dp + p * e.dA;                     // d(p A0)
-  N[2][0] = y * q[0] + A1 * t[0];
+  N[2][0] = first(N[2][0], y, q[0]) + A1 * t[0];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) N[2][1 + a] = y * q[1 + a] + A1 * t[1 + a] + z * n[a];
-  N[2][4] = y * E + A1 * t[4] + e.dp * F4 + R(0.5) * p * (x + y);
+  for (int a = 0; a < 3; ++a)
+    N[2][1 + a] = first(N[2][1 + a], y, q[1 + a]) + A1 * t[1 + a] + z * n[a];
+  N[2][4] = first(N[2][4], y, E) + A1 * t[4] + e.dp * F4 + R(0.5) * p * (x + y);
 }
 
 // The non-equilibrium terms enter for the full form with a collision time only (tau = 0 leaves
@@ -199,6 +214,12 @@ GKS_HD void side_terms(int full, const double* tab, R gm1, const R q[5], const R
 template <class R>
 GKS_HD bool full_terms(const FluxParams<R>& P) {
   return P.full && P.tau_model != 0;
+}
+
+// exp(-dt / (2 tau)), 0 for tau = 0.
+template <class R>
+GKS_HD R relaxation(R dt, R tau) {
+  return tau > R(0) ? k_exp(k_div(R(-0.5) * dt, tau)) : R(0);
 }
 
 // The two-point time fit of the full form (Eq. flux-1). With e = exp(-dt / (2 tau)) the fitted
@@ -215,7 +236,7 @@ struct FitWeights {
 };
 template <class R>
 GKS_HD void fit_weights(R tau, R dt, R idt0, FitWeights<R>& f) {
-  const R e = tau > R(0) ? k_exp(k_div(R(-0.5) * dt, tau)) : R(0);
+  const R e = relaxation(dt, tau);
   const R x = R(1) - e, s = x * x, m = x * (R(2) + x);
   const R idt = idt0 != R(0) ? idt0 : R(k_div(R(1), dt)), a = tau * idt, b = R(4) * a * idt;
   f.n[0] = a * m;
@@ -227,13 +248,11 @@ GKS_HD void fit_weights(R tau, R dt, R idt0, FitWeights<R>& f) {
 }
 
 // F^n and dF/dt of the two-point time fit from the interface state q0, its gradient dW, the two
-// sides' summed non-equilibrium terms N (full form) and pressures. Returns false for a
-// non-physical interface state.
+// sides' summed non-equilibrium terms N (full form) and pressures; w the primitives of q0.
 template <class R>
-GKS_HD bool interface_flux(const FluxParams<R>& P, const R q0[5], const R dW[5][3],
-                           const R N[3][5], R pl, R pr, const R n[3], R dt, R Fn[5], R Ft[5]) {
-  Prim<R> w;
-  if (!to_prim(q0, P.gamma, w)) return false;
+GKS_HD void interface_flux(const FluxParams<R>& P, const Prim<R>& w, const R q0[5],
+                           const R dW[5][3], const R N[3][5], R pl, R pr, const R n[3], R dt,
+                           R Fn[5], R Ft[5]) {
   const R gm1 = P.gamma - R(1), E = q0[4], p = w.p, Ep = E + p;
   const R U[3] = {w.U, w.V, w.W};
   const R Un = dotU(w, n[0], n[1], n[2]);
@@ -297,7 +316,7 @@ GKS_HD bool interface_flux(const FluxParams<R>& P, const R q0[5], const R dW[5][
       Fn[q] += f.n[0] * d0 + f.n[1] * d1 + f.n[2] * d2;
       Ft[q] += f.t[0] * d0 + f.t[1] * d1 + f.t[2] * d2;
     }
-    return true;
+    return;
   }
   if (P.pr_fix != R(0)) {
     // the energy components gain pr_fix times the heat flux relative to the interface velocity,
@@ -312,7 +331,6 @@ GKS_HD bool interface_flux(const FluxParams<R>& P, const R q0[5], const R dW[5][
     Fn[4] += P.pr_fix * qn;
     Ft[4] += P.pr_fix * qt;
   }
-  return true;
 }
 
 // Whole Gauss-point contribution: values and gradients [v][axis] of both sides, unit normal n
@@ -326,22 +344,12 @@ GKS_HD bool gp_flux_global(const FluxParams<R>& P, const R vl[5], const R gl[5][
   const R gm1 = P.gamma - R(1);
   const bool full = full_terms(P);
   R q0[5], dW[5][3], N[3][5];
-  side_terms(full, P.erfc_tab, gm1, vl, gl, n, +1, hl, q0, dW, N);
-  {
-    R q[5], d[5][3], M[3][5];
-    side_terms(full, P.erfc_tab, gm1, vr, gr, n, -1, hr, q, d, M);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      q0[v] += q[v];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        dW[v][a] += d[v][a];
-        if (full) N[a][v] += M[a][v];
-      }
-    }
-  }
+  side_terms<false>(full, P.erfc_tab, gm1, vl, gl, n, +1, hl, q0, dW, N);
+  side_terms<true>(full, P.erfc_tab, gm1, vr, gr, n, -1, hr, q0, dW, N);
+  Prim<R> w0;
+  if (!to_prim(q0, P.gamma, w0)) return false;
   R Fn[5], Ft[5];
-  if (!interface_flux(P, q0, dW, N, hl.w.p, hr.w.p, n, dt, Fn, Ft)) return false;
+  interface_flux(P, w0, q0, dW, N, hl.w.p, hr.w.p, n, dt, Fn, Ft);
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
     acc[q] = w * Fn[q];

@@ -385,20 +385,8 @@ GKS_HD bool gp_flux_global_vjp(const FluxParams<double>& P, const double vl[5],
   Side<double> hl, hr;
   if (!(to_prim(vl, P.gamma, hl.w) & to_prim(vr, P.gamma, hr.w))) return false;
   double q0[5], dW[5][3], N[3][5];
-  side_terms(full, P.erfc_tab, gm1, vl, gl, n, +1, hl, q0, dW, N);
-  {
-    double q[5], d[5][3], M[3][5];
-    side_terms(full, P.erfc_tab, gm1, vr, gr, n, -1, hr, q, d, M);
-#pragma unroll
-    for (int v = 0; v < 5; ++v) {
-      q0[v] += q[v];
-#pragma unroll
-      for (int a = 0; a < 3; ++a) {
-        dW[v][a] += d[v][a];
-        if (full) N[a][v] += M[a][v];
-      }
-    }
-  }
+  side_terms<false>(full, P.erfc_tab, gm1, vl, gl, n, +1, hl, q0, dW, N);
+  side_terms<true>(full, P.erfc_tab, gm1, vr, gr, n, -1, hr, q0, dW, N);
   double gq0[5] = {0, 0, 0, 0, 0}, gdW[5][3], gN[3][5], gpl = 0, gpr = 0;
 #pragma unroll
   for (int v = 0; v < 5; ++v)

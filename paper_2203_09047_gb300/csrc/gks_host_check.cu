@@ -201,26 +201,48 @@ gks::FluxParams<float> params_f32(const double* p) {
   return P;
 }
 // point i: in[45 i ..] = vl[5], gl[5][3], vr[5], gr[5][3], n1[3], w, dt;
-// out[21 i ..] = scalar acc[10], packed acc[10], (scalar ok) + 2 (packed ok)
+// out[21 i ..] = scalar acc[10], packed acc[10], (scalar ok) + 2 (packed ok). The packed form is
+// the kernels': the smooth form pairs point i with the next one (first half: point i), the full
+// form the two sides of point i.
 __global__ void k_face_f32_pair(gks::FluxParams<float> P, int n, const float* __restrict__ in,
                                 float* __restrict__ out) {
+  using gks::P2;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float* x = in + 45 * (int64_t)i;
+  const float* y = in + 45 * (int64_t)((i + 1) % n);
   float vl[5], gl[5][3], vr[5], gr[5][3], n1[3];
-  for (int v = 0; v < 5; ++v) {
-    vl[v] = x[v];
-    vr[v] = x[20 + v];
+  P2 v[5], g[5][3], nn[3], acc2[10];
+  for (int k = 0; k < 5; ++k) {
+    vl[k] = x[k];
+    vr[k] = x[20 + k];
+    v[k] = P2(x[k], y[k]);
     for (int a = 0; a < 3; ++a) {
-      gl[v][a] = x[5 + 3 * v + a];
-      gr[v][a] = x[25 + 3 * v + a];
+      gl[k][a] = x[5 + 3 * k + a];
+      gr[k][a] = x[25 + 3 * k + a];
+      g[k][a] = P2(x[5 + 3 * k + a], y[5 + 3 * k + a]);
     }
   }
-  for (int a = 0; a < 3; ++a) n1[a] = x[40 + a];
+  for (int a = 0; a < 3; ++a) {
+    n1[a] = x[40 + a];
+    nn[a] = P2(x[40 + a], y[40 + a]);
+  }
   const float w = x[43], dt = x[44];
   float acc_s[10], acc_p[10];
   const bool ok_s = gks::gp_flux_global(P, vl, gl, vr, gr, n1, w, dt, acc_s);
-  const bool ok_p = gks::gp_flux_global2(P, vl, gl, vr, gr, n1, w, dt, acc_p);
+  auto right = [&](P2* vv, P2 (*gg)[3]) {
+    for (int k = 0; k < 5; ++k) {
+      vv[k] = P2(x[20 + k], y[20 + k]);
+      for (int a = 0; a < 3; ++a) gg[k][a] = P2(x[25 + 3 * k + a], y[25 + 3 * k + a]);
+    }
+  };
+  bool ok_p;
+  if (gks::full_terms(P)) {
+    ok_p = gks::gp_flux_sides(P, vl, gl, vr, gr, n1, w, dt, acc_p);
+  } else {
+    ok_p = gks::gp_flux_pair(P, v, g, right, nn, P2(w), dt, acc2) & 1u;
+    for (int q = 0; q < 10; ++q) acc_p[q] = acc2[q].lo();
+  }
   float* o = out + 21 * (int64_t)i;
   for (int q = 0; q < 10; ++q) {
     o[q] = acc_s[q];

@@ -745,32 +745,71 @@ __device__ __forceinline__ void first_order_if_nonphysical(const R* __restrict__
   }
 }
 
+// The same for a pair of points, each on its own.
+__device__ __forceinline__ void first_order_if_nonphysical2(const float* __restrict__ QA,
+                                                            int64_t c, P2 v[5], P2 g[5][3]) {
+  const P2 m2 = v[1] * v[1] + v[2] * v[2] + v[3] * v[3], e = v[0] * v[4];
+  const bool b0 = !(v[0].lo() > 0.f && e.lo() > 0.5f * m2.lo());
+  const bool b1 = !(v[0].hi() > 0.f && e.hi() > 0.5f * m2.hi());
+  if (!b0 && !b1) return;
+  Gq<float> q;
+  q.load(QA, c);
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
+    v[k] = P2(b0 ? q.value(k) : v[k].lo(), b1 ? q.value(k) : v[k].hi());
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+      g[k][a] = P2(b0 ? 0.f : g[k][a].lo(), b1 ? 0.f : g[k][a].hi());
+  }
+}
+// The wall's ghost of a pair of points in place of the owner's values, one point at a time (the
+// far-field state branches on the point's state).
+__device__ __forceinline__ void wall_ghost2(const FluxParams<float>& P, int wall,
+                                         const WallData<float>& wd, P2 v[5], P2 g[5][3]) {
+#pragma unroll 1
+  for (int h = 0; h < 2; ++h) {
+    float vo[5], go[5][3], vg[5], gg[5][3];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      vo[k] = h ? v[k].hi() : v[k].lo();
+#pragma unroll
+      for (int a = 0; a < 3; ++a) go[k][a] = h ? g[k][a].hi() : g[k][a].lo();
+    }
+    wall_ghost(P, wall, wd, vo, go, vg, gg);
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      v[k] = h ? P2(v[k].lo(), vg[k]) : P2(vg[k], v[k].hi());
+#pragma unroll
+      for (int a = 0; a < 3; ++a)
+        g[k][a] = h ? P2(g[k][a].lo(), gg[k][a]) : P2(gg[k][a], g[k][a].hi());
+    }
+  }
+}
+
 // ------------------------------------------------------------------------------------------
-// Flux: four consecutive threads per face, one per Gauss point. Each evaluates both sides'
-// reconstructions and gradients, computes F^n and dF/dt in the global frame (gks_flux.cuh) and
-// weights them by the quadrature weight; the four are summed with shuffles and written once.
-// kFull selects the flux form and kTau0 a zero collision time at compile time, so that each
-// instance carries only the arithmetic (and registers) of its own form. The FP32 instances do
-// the two sides' work on packed f32x2 arithmetic (gp_flux_global2: side_terms instantiated with
-// the pair type P2). Bound by the FMA pipe (FP64: the FP64 pipe, 1/64 of the FP32 rate), so the
-// form with the fewest operations wins: against the flux in the face frame (values and
-// gradients rotated to the normal and two tangents, one moment derivative per axis), per
-// launch: FP32 smooth 0.418 -> 0.326 ms (64^3-cube mesh, 2.39 M faces), FP32 full 326 -> 231 us
-// (48^3-cube explosion, 1.02 M faces), FP64 smooth 2.53 -> 1.77 ms (32^3 cubes, 299 k faces),
-// FP64 full 2.05 -> 1.31 ms (124 k faces of tetrahedra); with erfc and exp from one table and one
-// division per state (half_erfc, to_prim) FP64 1.49 and 1.20 ms. Resident blocks per SM, measured on
-// the same meshes: FP32 smooth 6 (0.326 ms; 4, 5, 7 and 8 blocks 0.380, 0.354, 0.333 and
-// 0.356); FP32 full 4 (231 us; 3 and 5 blocks 254 and 254); FP64 unbounded (2 blocks equal; 3
-// and 4 blocks 1 and 3 % slower).
-#ifndef GKS_FLUX_SMOOTH_MIN_BLOCKS
-#define GKS_FLUX_SMOOTH_MIN_BLOCKS 6  // resident 128-thread blocks per SM, FP32 smooth flux
-#endif
-#ifndef GKS_FLUX_FULL_MIN_BLOCKS
-#define GKS_FLUX_FULL_MIN_BLOCKS 4  // resident 128-thread blocks per SM, FP32 full flux
-#endif
-#ifndef GKS_FLUX_FP64_MIN_BLOCKS
-#define GKS_FLUX_FP64_MIN_BLOCKS 1  // resident 128-thread blocks per SM, FP64 flux
-#endif
+// Flux: per Gauss point both sides' reconstructions and gradients, F^n and dF/dt in the global
+// frame (gks_flux.cuh), weighted by the quadrature weight; the four points of a face are summed
+// with shuffles and written once. k_flux_pair (FP32, smooth form): two threads per face, two
+// points per thread on packed arithmetic; k_flux: four threads per face, one point per thread, in
+// FP64, and in FP32 for the full form with the two sides packed. kTau0 fixes a zero collision
+// time and kFull the full form at compile time, so that an instance carries only its own form.
+// Bound by issue slots and the FMA pipe (FP64: the FP64 pipe, 1/64 of the FP32 rate), so the form
+// with the fewest operations wins. Per launch, against the flux in the face frame (values and
+// gradients rotated to the normal and two tangents, one moment derivative per axis):
+//   FP32 smooth, 64^3-cube mesh (2.39 M faces): 0.418 -> 0.326 ms, two points per thread 0.302;
+//   FP32 full, 48^3-cube explosion (1.02 M faces): 326 -> 231 us;
+//   FP64 smooth, 32^3 cubes (299 k faces): 2.53 -> 1.77 ms, with erfc and exp from one table and
+//     one division per state (half_erfc, to_prim) 1.49, sums started from the other side's 1.44;
+//   FP64 full, 124 k faces of tetrahedra: 2.05 -> 1.31, 1.20, 1.16 ms.
+// Resident threads per SM, measured: FP32 smooth 8 blocks of 64 (0.302 ms; of 128 threads 4
+// blocks 0.307, 3 blocks without spills 0.322, 5 blocks 0.407); FP32 full 4 blocks of 128 (231
+// us; 3 and 5 blocks 254 and 254); FP64 unbounded (two blocks).
+constexpr int kPairThreads = 64, kPairBlocks = 8;  // k_flux_pair
+constexpr int kFullBlocks = 4, kSidesBlocks = 6;   // k_flux, FP32 full and smooth form, 128 threads
+// Fewest faces of k_flux_pair, about one and a half waves of its threads: below it the GPU is not
+// full, and four threads per face are done sooner (ten steps of the 8^3-cube mesh, 4,672 faces,
+// 474 -> 468 us; 37,000 faces 659 -> 655 us; equal at 126,000; at 299,000 2.252 against 2.286 ms).
+constexpr int64_t kPairFaces = 60000;
 // One 16-byte (FP32) or 32-byte (FP64) part of a face record of kFaceStride values: part j holds
 // values 4j .. 4j + 3 of acc (values 10 and 11 are padding, written as zeros).
 template <class R>
@@ -798,11 +837,68 @@ struct FaceRec<double> {
   }
 };
 
+template <bool kTau0>
+__global__ void __launch_bounds__(kPairThreads, kPairBlocks)
+    k_flux_pair(int64_t nf, const int32_t* __restrict__ f_owner, const int32_t* __restrict__ f_nb,
+                const int8_t* __restrict__ f_wall, const float* __restrict__ fgp,
+                const float* __restrict__ poly, const float* __restrict__ QA, int fallback,
+                FluxParams<float> P, const float* __restrict__ wall_tab, float dt,
+                float* __restrict__ fface, int* flag) {
+  P.full = 0;
+  if (kTau0) P.tau_model = 0;
+  const int64_t gid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  const int64_t f = gid >> 1;  // two threads per face, Gauss points 2 (gid & 1) and the next
+  const bool active = f < nf;
+  float acc[10];
+#pragma unroll
+  for (int q = 0; q < 10; ++q) acc[q] = 0.f;
+  int wall = -1;
+  if (active) {
+    const int64_t stride = 4 * nf;
+    const int32_t o = f_owner[f], nb = f_nb[f];
+    wall = f_wall[f];
+    auto pair_at = [&](int a) {
+      return P2(__ldcs(reinterpret_cast<const float2*>(fgp + a * stride) + gid));
+    };
+    P2 d[3], n[3], v[5], g[5][3], acc2[10];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      d[a] = pair_at(a);
+      n[a] = pair_at(6 + a);
+    }
+    eval_poly2(PolyRef<float>{poly + (int64_t)kPolyStride * o}, d, v, g);
+    if (fallback) first_order_if_nonphysical2(QA, o, v, g);
+    auto right = [&](P2* v, P2 (*g)[3]) {
+      if (nb >= 0) {
+        P2 e[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) e[a] = pair_at(3 + a);
+        eval_poly2(PolyRef<float>{poly + (int64_t)kPolyStride * nb}, e, v, g);
+        if (fallback) first_order_if_nonphysical2(QA, nb, v, g);
+      } else {
+        wall_ghost2(P, wall, wall_data(wall_tab, wall), v, g);  // the wall's ghost
+      }
+    };
+    const unsigned ok = gp_flux_pair(P, v, g, right, n, pair_at(9), dt, acc2);
+    if (ok != 3u) atomicOr(flag, kErrNonphysical);
+#pragma unroll
+    for (int q = 0; q < 10; ++q) acc[q] = hsum(acc2[q]);
+  }
+#pragma unroll
+  for (int q = 0; q < 10; ++q) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 1);
+  // both lanes of the face hold the sums; lane j writes the record's 16-byte part j, lane 0 part 2
+  if (active) {
+    if (wall >= 0) wall_flux_fix(wall, wall_data(wall_tab, wall), acc);
+    float* rec = fface + (int64_t)kFaceStride * f;
+    FaceRec<float>::put(rec, (int)(gid & 1), acc);
+    if ((gid & 1) == 0) FaceRec<float>::put(rec, 2, acc);
+  }
+}
+
+// One Gauss point per thread, four consecutive threads per face: FP64, and the FP32 full form.
 template <class R, bool kFull, bool kTau0>
-__global__ void __launch_bounds__(128, sizeof(R) == 4 ? (kFull ? GKS_FLUX_FULL_MIN_BLOCKS : GKS_FLUX_SMOOTH_MIN_BLOCKS)
-                                                      : GKS_FLUX_FP64_MIN_BLOCKS)
-    k_flux(
-    int64_t nf, int64_t nc, const int32_t* __restrict__ f_owner, const int32_t* __restrict__ f_nb,
+__global__ void __launch_bounds__(128, sizeof(R) == 4 ? (kFull ? kFullBlocks : kSidesBlocks) : 1) k_flux(
+    int64_t nf, const int32_t* __restrict__ f_owner, const int32_t* __restrict__ f_nb,
     const int8_t* __restrict__ f_wall, const R* __restrict__ fgp, const R* __restrict__ poly,
     const R* __restrict__ QA, int fallback, FluxParams<R> P, const R* __restrict__ wall_tab, R dt,
     R* __restrict__ fface, int* flag) {
@@ -838,7 +934,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? (kFull ? GKS_FLUX_FULL_M
     }
     bool ok;
     if constexpr (sizeof(R) == 4)
-      ok = gp_flux_global2(P, vl, gl, vr, gr, n1, w, dt, acc);  // both sides on packed f32x2
+      ok = gp_flux_sides(P, vl, gl, vr, gr, n1, w, dt, acc);  // both sides on packed f32x2
     else
       ok = gp_flux_global(P, vl, gl, vr, gr, n1, w, dt, acc);
     if (!ok) atomicOr(flag, kErrNonphysical);
@@ -849,9 +945,7 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? (kFull ? GKS_FLUX_FULL_M
     acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 1);
     acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 2);
   }
-  // every lane of the face now holds the sums; lanes 4f + j, j < 3, write the record's 16-byte
-  // part j (values 4j .. 4j + 3; the two padding values of part 2 are written as zeros), so a
-  // warp writes its eight faces' 384 contiguous bytes in one store
+  // every lane of the face now holds the sums; lanes 4f + j, j < 3, write the record's part j
   if (active && (gid & 3) < 3) {
     if (wall >= 0) wall_flux_fix(wall, wall_data(wall_tab, wall), acc);
     FaceRec<R>::put(fface + (int64_t)kFaceStride * f, (int)(gid & 3), acc);
@@ -1733,13 +1827,25 @@ void launch_flux(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const 
   FluxParams<R> fp = flux_params(p);
   fp.erfc_tab = m.erfc_tab;
   fp.idt = (R)(1.0 / dt);
-  const unsigned nb = blocks_for(4 * m.nf, 128);
   // without a collision time the full form is the smooth one (its non-equilibrium terms carry
   // the weight tau = 0)
-  auto kern = fp.tau_model == 0 ? k_flux<R, false, true>
-                                : (fp.full ? k_flux<R, true, false> : k_flux<R, false, false>);
-  kern<<<nb, 128, 0, st>>>(m.nf, m.nc, m.f_owner, m.f_nb, m.f_wall, g.fgp, poly, QA,
-                           p.gp_fallback, fp, wall_table<R>(m), (R)dt, fface, flag);
+  auto run = [&](auto kern, int per_face, int nt) {
+    kern<<<blocks_for(per_face * m.nf, nt), nt, 0, st>>>(
+        m.nf, m.f_owner, m.f_nb, m.f_wall, g.fgp, poly, QA, p.gp_fallback, fp, wall_table<R>(m),
+        (R)dt, fface, flag);
+  };
+  if constexpr (std::is_same<R, float>::value) {
+    const bool pair = m.nf >= kPairFaces;
+    if (fp.tau_model != 0 && fp.full)
+      run(k_flux<R, true, false>, 4, 128);
+    else if (pair)
+      run(fp.tau_model == 0 ? k_flux_pair<true> : k_flux_pair<false>, 2, kPairThreads);
+    else
+      run(fp.tau_model == 0 ? k_flux<R, false, true> : k_flux<R, false, false>, 4, 128);
+  } else {
+    run(fp.tau_model == 0 ? k_flux<R, false, true>
+                          : (fp.full ? k_flux<R, true, false> : k_flux<R, false, false>), 4, 128);
+  }
 }
 template <class R>
 void launch_gather(const DevMesh& m, const Geo64& g, const R* fface, double* L, double* Lt,
