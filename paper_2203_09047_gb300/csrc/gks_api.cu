@@ -61,11 +61,8 @@ struct gks_solver {
   ForkJoin fj;             // concurrent reconstruction ranges
   // implicit step (allocated on the first gks_step_implicit call), precision R:
   bool imp_ready = false;
-  void* jfn = nullptr;      // [nf][4] unit normal out of the owner, area
-  void* jR = nullptr;       // [5][nc] |Omega| Res
-  void* jD = nullptr;       // [nc] Jacobi diagonal
-  void* jhrs = nullptr;     // [cf entries] r_f S_f / 2
-  void* jdQ[2] = {nullptr, nullptr};  // [5][nc] Jacobi iterates
+  JacobiBuf<double> jd;
+  JacobiBuf<float> jf;
   int* flag = nullptr;      // device status bits
   int* bad_cell = nullptr;
   double* dt_part = nullptr;
@@ -441,28 +438,27 @@ bool valid_params(const gks_params* p, std::string& why) {
 }
 
 template <class R>
-gks_status step_implicit_r(gks_solver* s, GeoR<R>& g, double dt, int nsteps, int kmax) {
-  const int64_t nc = s->m.nc, nf = s->m.nf;
+gks_status step_implicit_r(gks_solver* s, GeoR<R>& g, JacobiBuf<R>& b, double dt, int nsteps,
+                           int kmax) {
+  const int64_t nc = s->m.nc, nf = s->m.nf, ncf = s->m.n_tiles * kTile * kCellFaces;
   cudaError_t e = cudaSuccess;
   if (!s->imp_ready) {
-    R *fn = nullptr, *rv = nullptr, *d = nullptr, *hrs = nullptr, *a = nullptr, *b = nullptr;
-    if ((e = salloc(s, &fn, 4 * nf)) != cudaSuccess || (e = salloc(s, &rv, 5 * nc)) != cudaSuccess ||
-        (e = salloc(s, &d, nc)) != cudaSuccess || (e = salloc(s, &hrs, s->m.ncf)) != cudaSuccess ||
-        (e = salloc(s, &a, 5 * nc)) != cudaSuccess || (e = salloc(s, &b, 5 * nc)) != cudaSuccess)
+    // the face normals are needed for the plan only: they borrow an iterate's buffer
+    const int64_t ndq = (sizeof(R) == 4 ? 8 : 6) * nc;
+    if ((e = salloc(s, &b.nb, ncf)) != cudaSuccess || (e = salloc(s, &b.n, 4 * ncf)) != cudaSuccess ||
+        (e = salloc(s, &b.prim, 4 * nc)) != cudaSuccess || (e = salloc(s, &b.Rv, 5 * nc)) != cudaSuccess ||
+        (e = salloc(s, &b.D, nc)) != cudaSuccess || (e = salloc(s, &b.hrs, ncf)) != cudaSuccess ||
+        (e = salloc(s, &b.dQ[0], ndq)) != cudaSuccess ||
+        (e = salloc(s, &b.dQ[1], std::max(ndq, 4 * nf))) != cudaSuccess)
       return s->cuda_fail(e, "implicit buffers");
-    s->jfn = fn;
-    s->jR = rv;
-    s->jD = d;
-    s->jhrs = hrs;
-    s->jdQ[0] = a;
-    s->jdQ[1] = b;
+    R* fn = b.dQ[1];
     launch_face_normals<R>(s->m, fn, s->st);
+    launch_jacobi_plan<R>(s->m, fn, b.nb, b.n, s->st);
     s->imp_ready = true;
   }
   KParams<R> kp = kparams<R>(s->prm);
   kp.wait_tries = s->dbg_wait_tries;
   kp.withhold = s->dbg_withhold;
-  R* dq[2] = {(R*)s->jdQ[0], (R*)s->jdQ[1]};
   for (int n = 0; n < nsteps; ++n) {
     int t = s->tick(0);
     launch_recon<R>(s->m, g, kp, (const R*)s->QA, (R*)s->poly, s->flag, s->st, &s->fj);
@@ -472,13 +468,10 @@ gks_status step_implicit_r(gks_solver* s, GeoR<R>& g, double dt, int nsteps, int
                    s->st);
     s->tock(t);
     t = s->tick(2);
-    launch_jacobi_init<R>(s->m, (const R*)s->fface, (const R*)s->jfn, s->g.vol, dt,
-                          (const R*)s->QA, (R*)s->jR, (R*)s->jD, (R*)s->jhrs, dq[0], kp,
-                          s->st);
+    launch_jacobi_init<R>(s->m, (const R*)s->fface, b, s->g.vol, dt, (const R*)s->QA, kp, s->st);
     for (int it = 1; it <= kmax; ++it)
-      launch_jacobi_sweep<R>(s->m, (const R*)s->jfn, (const R*)s->QA, (const R*)s->jR,
-                             (const R*)s->jD, (const R*)s->jhrs, dq[(it - 1) & 1], dq[it & 1],
-                             it == kmax, (R*)s->QsA, kp, s->flag, s->st);
+      launch_jacobi_sweep<R>(s->m, b, (const R*)s->QA, it, it == kmax, (R*)s->QsA, kp, s->flag,
+                             s->st);
     s->tock(t);
     std::swap(s->QA, s->QsA);  // Q^{n+1} was written to the other gather copy
   }
@@ -868,8 +861,8 @@ gks_status gks_s2o4_stage_vjp(int64_t n, int stage, double dt, const double* g, 
 
 gks_status gks_step_implicit(gks_solver* s, double dt, int nsteps, int kmax) {
   if (!s || !(dt > 0) || nsteps < 0 || kmax < 1) return GKS_E_INVAL;
-  return s->mixed ? step_implicit_r<float>(s, s->gf, dt, nsteps, kmax)
-                  : step_implicit_r<double>(s, s->gd, dt, nsteps, kmax);
+  return s->mixed ? step_implicit_r<float>(s, s->gf, s->jf, dt, nsteps, kmax)
+                  : step_implicit_r<double>(s, s->gd, s->jd, dt, nsteps, kmax);
 }
 
 gks_status gks_check(gks_solver* s) {

@@ -214,18 +214,30 @@ void launch_stage(const DevMesh& m, const GeoR<R>& g, const R* fface, int stage,
                   double* Q64 = nullptr, const double* ivol64 = nullptr);
 // Implicit step (Section 4) on the gather copy QA (the state), after the reconstruction and
 // flux of Q^n: jacobi_init forms |Omega| Res = s + dt/2 st from the face sums, the diagonal
-// D = |Omega|/dt + 1/2 sum_f r_f S_f, the per-entry factors hrs = 1/2 r_f S_f (cell-face CSR
-// order) and dQ0 = |Omega| Res / D; each jacobi_sweep forms dQ^(k) from dQ^(k-1), the last one
-// (last != 0) writes Q^n + dQ to QAout (the other gather copy) in place of dQ. Buffers are in precision R: Rv, dQ
-// [5][nc], D [nc], hrs [cf entries]; fn is [nf][4] from launch_face_normals.
+// D = |Omega|/dt + 1/2 sum_f r_f S_f, the per-entry factors hrs = 1/2 r_f S_f and
+// dQ0 = |Omega| Res / D; jacobi_sweep number it forms dQ^(it) from dQ^(it-1), the last one
+// (last != 0) writes Q^n + dQ to QAout (the other gather copy) in place of dQ. Buffers in
+// precision R; nb and n are the plan of jacobi_plan (fn: [nf][4] from launch_face_normals), "cf"
+// arrays have kCellFaces entries per cell, tile-interleaved [tile][kCellFaces][32].
+constexpr int kCellFaces = 6;  // most faces of a cell (hexahedra)
 template <class R>
-void launch_jacobi_init(const DevMesh& m, const R* fface, const R* fn, const double* vol,
-                        double dt, const R* QA, R* Rv, R* D, R* hrs, R* dQ0, const KParams<R>& kp,
-                        cudaStream_t st);
+struct JacobiBuf {
+  int32_t* nb = nullptr;  // [cf] cell across the face, -1 - wall code at a boundary
+  R* n = nullptr;         // [cf][4] unit normal out of the cell, face area
+  R* prim = nullptr;      // [nc][4] 1/rho, p, sound speed
+  R* Rv = nullptr;        // [5][nc] |Omega| Res
+  R* D = nullptr;         // [nc] diagonal
+  R* hrs = nullptr;       // [cf]
+  R* dQ[2] = {nullptr, nullptr};  // iterates, one record of 8 (FP32) or 6 (FP64) values per cell
+};
 template <class R>
-void launch_jacobi_sweep(const DevMesh& m, const R* fn, const R* QA, const R* Rv, const R* D,
-                         const R* hrs, const R* dQin, R* dQout, int last, R* QAout,
-                         const KParams<R>& kp, int* flag, cudaStream_t st);
+void launch_jacobi_plan(const DevMesh& m, const R* fn, int32_t* jnb, R* jn, cudaStream_t st);
+template <class R>
+void launch_jacobi_init(const DevMesh& m, const R* fface, const JacobiBuf<R>& b, const double* vol,
+                        double dt, const R* QA, const KParams<R>& kp, cudaStream_t st);
+template <class R>
+void launch_jacobi_sweep(const DevMesh& m, const JacobiBuf<R>& b, const R* QA, int it, int last,
+                         R* QAout, const KParams<R>& kp, int* flag, cudaStream_t st);
 
 // The state [5][nc] in FP64 (internal order) from its gather copy.
 template <class R>

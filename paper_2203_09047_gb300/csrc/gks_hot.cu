@@ -1245,25 +1245,84 @@ __global__ void __launch_bounds__(256) k_s2o4_stage_vjp(int64_t n, int stage, do
 // (du = (dm - u drho)/rho', dp = (gamma - 1)(dE - (m . du + dm . u')/2)), so no two nearly equal
 // fluxes are subtracted.
 
+// Per-cell values of the implicit step at Q^n: 1/rho, p, sound speed.
 template <class R>
-__device__ __forceinline__ void state_of(const R* __restrict__ QA, int64_t c, R q[5]) {
-  Gq<R> g;
-  g.load(QA, c);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) q[v] = (R)g.value(v);
+struct JPrim {
+  R ir, p, c, pad;
+};
+// Four values of R (normal and area of a cell's face, JPrim) in one or two 16-byte loads.
+template <class R>
+struct __align__(16) R4 {
+  R x, y, z, w;
+};
+__device__ __forceinline__ R4<float> ld4(const float* p) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+  return {a.x, a.y, a.z, a.w};
+}
+__device__ __forceinline__ R4<double> ld4(const double* p) {
+  const double2 a = __ldg(reinterpret_cast<const double2*>(p));
+  const double2 b = __ldg(reinterpret_cast<const double2*>(p) + 1);
+  return {a.x, a.y, b.x, b.y};
 }
 template <class R>
-__device__ __forceinline__ R wave_speed(const R q[5], const R n[3], R gm1) {
-  const R ir = R(1) / q[0];
-  const R u[3] = {q[1] * ir, q[2] * ir, q[3] * ir};
-  const R p = gm1 * (q[4] - R(0.5) * (q[1] * u[0] + q[2] * u[1] + q[3] * u[2]));
-  const R c2 = (gm1 + R(1)) * p * ir;
-  return fabs(u[0] * n[0] + u[1] * n[1] + u[2] * n[2]) + sqrt(c2 > R(0) ? c2 : R(0));
+__device__ __forceinline__ JPrim<R> load_prim(const R* __restrict__ prim, int64_t c) {
+  const R4<R> a = ld4(prim + 4 * c);
+  return {a.x, a.y, a.z, R(0)};
+}
+// Iterates: one record of kJdq values per cell.
+template <class R>
+constexpr int kJdq = sizeof(R) == 4 ? 8 : 6;
+__device__ __forceinline__ void load_dq(const float* __restrict__ dQ, int64_t c, float d[5]) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(dQ + 8 * c));
+  d[0] = a.x; d[1] = a.y; d[2] = a.z; d[3] = a.w;
+  d[4] = __ldg(dQ + 8 * c + 4);
+}
+__device__ __forceinline__ void load_dq(const double* __restrict__ dQ, int64_t c, double d[5]) {
+  const double2* p = reinterpret_cast<const double2*>(dQ + 6 * c);
+  const double2 a = __ldg(p), b = __ldg(p + 1);
+  d[0] = a.x; d[1] = a.y; d[2] = b.x; d[3] = b.y;
+  d[4] = __ldg(dQ + 6 * c + 4);
+}
+__device__ __forceinline__ void store_dq(float* __restrict__ dQ, int64_t c, const float d[5]) {
+  *reinterpret_cast<float4*>(dQ + 8 * c) = make_float4(d[0], d[1], d[2], d[3]);
+  dQ[8 * c + 4] = d[4];
+}
+__device__ __forceinline__ void store_dq(double* __restrict__ dQ, int64_t c, const double d[5]) {
+  double2* p = reinterpret_cast<double2*>(dQ + 6 * c);
+  p[0] = make_double2(d[0], d[1]);
+  p[1] = make_double2(d[2], d[3]);
+  dQ[6 * c + 4] = d[4];
+}
+// State of a cell from its gather copy in precision R (the leading parts of float-float pairs).
+__device__ __forceinline__ void state_of(const float* __restrict__ QA, int64_t c, float q[5]) {
+  const float4 a = __ldg(reinterpret_cast<const float4*>(QA + 12 * c));
+  q[0] = a.x; q[1] = a.y; q[2] = a.z; q[3] = a.w;
+  q[4] = __ldg(QA + 12 * c + 4);
+}
+__device__ __forceinline__ void state_of(const double* __restrict__ QA, int64_t c, double q[5]) {
+  const double2* p = reinterpret_cast<const double2*>(QA + 6 * c);
+  const double2 a = __ldg(p), b = __ldg(p + 1);
+  q[0] = a.x; q[1] = a.y; q[2] = b.x; q[3] = b.y;
+  q[4] = __ldg(QA + 6 * c + 4);
 }
 template <class R>
-__device__ __forceinline__ void euler_flux_change(const R q[5], const R d[5], const R n[3], R gm1,
-                                                  R out[5]) {
-  const R ir = R(1) / q[0], ir1 = R(1) / (q[0] + d[0]);
+__device__ __forceinline__ JPrim<R> prim_of(const R q[5], R gm1) {
+  JPrim<R> w;
+  w.ir = R(1) / q[0];
+  w.p = gm1 * (q[4] - R(0.5) * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) * w.ir);
+  const R c2 = (gm1 + R(1)) * w.p * w.ir;
+  w.c = sqrt(c2 > R(0) ? c2 : R(0));
+  w.pad = R(0);
+  return w;
+}
+template <class R>
+__device__ __forceinline__ R wave_speed(const R q[5], const JPrim<R>& w, const R n[3]) {
+  return fabs((q[1] * n[0] + q[2] * n[1] + q[3] * n[2]) * w.ir) + w.c;
+}
+template <class R>
+__device__ __forceinline__ void euler_flux_change(const R q[5], R ir, R p, const R d[5],
+                                                  const R n[3], R gm1, R out[5]) {
+  const R ir1 = R(1) / (q[0] + d[0]);
   R u[3], du[3], u1[3];
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -1273,7 +1332,6 @@ __device__ __forceinline__ void euler_flux_change(const R q[5], const R d[5], co
   }
   const R un = u[0] * n[0] + u[1] * n[1] + u[2] * n[2];
   const R dun = du[0] * n[0] + du[1] * n[1] + du[2] * n[2], un1 = un + dun;
-  const R p = gm1 * (q[4] - R(0.5) * (q[1] * u[0] + q[2] * u[1] + q[3] * u[2]));
   const R dp = gm1 * (d[4] - R(0.5) * (q[1] * du[0] + q[2] * du[1] + q[3] * du[2] +
                                        d[1] * u1[0] + d[2] * u1[1] + d[3] * u1[2]));
   out[0] = d[1] * n[0] + d[2] * n[1] + d[3] * n[2];
@@ -1327,56 +1385,99 @@ __device__ __forceinline__ void wall_cell_ghost_inc(const FluxParams<R>& P, int 
           R(2) * (u0 * d[1] + u1 * d[2] + u2 * d[3]);
 }
 
-// The other side of cell-face entry e seen from cell i: its index (-1: the wall's ghost of cell
-// i, *wall the wall code) and the unit normal out of cell i with the face area.
+// Plan of the implicit step, tile-interleaved [tile][kCellFaces][32] in the order of a cell's
+// faces: the cell across each (nb >= 0, -1 - wall code at a boundary face, kNoFace beyond the
+// cell's faces) and the unit normal out of the cell with the face area. One coalesced read in
+// place of the chain CSR entry -> face -> owner, neighbour, wall and normal of every sweep.
+constexpr int32_t kNoFace = INT32_MIN;
 template <class R>
-__device__ __forceinline__ int64_t other_side(int32_t e, const int32_t* __restrict__ f_owner,
-                                              const int32_t* __restrict__ f_nb,
-                                              const int8_t* __restrict__ f_wall,
-                                              const R* __restrict__ fn, R n[3], R& S, int& wall) {
-  const int64_t f = e >> 1;
-  const bool nbside = e & 1;
-  const R sg = nbside ? R(-1) : R(1);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) n[a] = sg * fn[4 * f + a];
-  S = fn[4 * f + 3];
-  const int64_t p = nbside ? f_owner[f] : f_nb[f];
-  wall = p < 0 ? f_wall[f] : -1;
-  return p;
+__global__ void k_jacobi_plan(int64_t nc, int64_t n_tiles, const int32_t* __restrict__ cf_ptr,
+                              const int32_t* __restrict__ cf_idx,
+                              const int32_t* __restrict__ f_owner,
+                              const int32_t* __restrict__ f_nb, const int8_t* __restrict__ f_wall,
+                              const R* __restrict__ fn, int32_t* __restrict__ jnb,
+                              R* __restrict__ jn) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= n_tiles * kTile) return;
+  const int64_t at = i / kTile * kCellFaces * kTile + i % kTile;
+  const int k0 = i < nc ? cf_ptr[i] : 0, nk = i < nc ? cf_ptr[i + 1] - k0 : 0;
+  for (int j = 0; j < kCellFaces; ++j) {
+    const int64_t o = at + (int64_t)j * kTile;
+    if (j >= nk) {
+      jnb[o] = kNoFace;
+      for (int a = 0; a < 4; ++a) jn[4 * o + a] = R(0);
+      continue;
+    }
+    const int32_t e = cf_idx[k0 + j];
+    const int64_t f = e >> 1;
+    const bool nbside = e & 1;
+    const int32_t p = nbside ? f_owner[f] : f_nb[f];
+    jnb[o] = p >= 0 ? p : -1 - f_wall[f];
+    for (int a = 0; a < 3; ++a) jn[4 * o + a] = nbside ? -fn[4 * f + a] : fn[4 * f + a];
+    jn[4 * o + 3] = fn[4 * f + 3];
+  }
+}
+template <class R>
+__global__ void __launch_bounds__(256) k_jacobi_prim(int64_t nc, const R* __restrict__ QA, R gm1,
+                                                     R* __restrict__ prim) {
+  const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  if (i >= nc) return;
+  R q[5];
+  state_of(QA, i, q);
+  const JPrim<R> w = prim_of(q, gm1);
+  *reinterpret_cast<R4<R>*>(prim + 4 * i) = {w.ir, w.p, w.c, R(0)};
 }
 
+// Both kernels below wait on the gathers of a cell's neighbours in FP32, and on the FP64 pipe in
+// FP64. The plan's coalesced entries, one record per cell for the iterate, and 1/rho, p and c per
+// cell in place of per face took an FP32 step's init and three sweeps from 69 to 58 us (131,072
+// cells), the FP64 one from 256 to 160 us (48,000 cells, where blocks of 256 threads, 188 of
+// them, left every second SM with twice the work of the others: 234 us). Requesting two, three or
+// six faces of a cell together was slower (66, 68, 89 us).
 template <class R>
 __global__ void __launch_bounds__(256) k_jacobi_init(
     int64_t nc, const int32_t* __restrict__ cf_ptr, const int32_t* __restrict__ cf_idx,
-    const int32_t* __restrict__ f_owner, const int32_t* __restrict__ f_nb,
-    const int8_t* __restrict__ f_wall, const R* __restrict__ fface, const R* __restrict__ fn,
-    const double* __restrict__ vol, double dt, const R* __restrict__ QA, FluxParams<R> P,
-    const R* __restrict__ wall_tab, R* __restrict__ Rv, R* __restrict__ D, R* __restrict__ hrs,
-    R* __restrict__ dQ0) {
+    const int32_t* __restrict__ jnb, const R* __restrict__ jn, const R* __restrict__ fface,
+    const double* __restrict__ vol, double dt, const R* __restrict__ QA,
+    R* __restrict__ prim, FluxParams<R> P, const R* __restrict__ wall_tab, R* __restrict__ Rv,
+    R* __restrict__ D, R* __restrict__ hrs, R* __restrict__ dQ0) {
+  constexpr bool kPrimed = sizeof(R) == 8;  // prim filled by k_jacobi_prim
   const R gm1 = P.gamma - R(1);
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= nc) return;
   R qi[5];
   state_of(QA, i, qi);
+  const JPrim<R> wi = kPrimed ? load_prim(prim, i) : prim_of(qi, gm1);
+  if (!kPrimed) *reinterpret_cast<R4<R>*>(prim + 4 * i) = {wi.ir, wi.p, wi.c, R(0)};
   R dsum = R(0);
-  const int k0 = cf_ptr[i], k1 = cf_ptr[i + 1];
-  for (int k = k0; k < k1; ++k) {
-    R n[3], S, qp[5];
-    int wall;
-    const int64_t p = other_side(cf_idx[k], f_owner, f_nb, f_wall, fn, n, S, wall);
-    if (p >= 0) {
-      state_of(QA, p, qp);
+  const int64_t at = i / kTile * kCellFaces * kTile + i % kTile;
+  int32_t nba[kCellFaces];
+#pragma unroll
+  for (int j = 0; j < kCellFaces; ++j) nba[j] = __ldg(jnb + at + j * kTile);
+#pragma unroll
+  for (int j = 0; j < kCellFaces; ++j) {
+    const int32_t nb = nba[j];
+    if (nb == kNoFace) break;
+    const R4<R> n4 = ld4(jn + 4 * (at + j * kTile));
+    const R n[3] = {n4.x, n4.y, n4.z};
+    R q[5];
+    JPrim<R> w;
+    if (nb >= 0) {
+      state_of(QA, nb, q);
+      w = kPrimed ? load_prim(prim, nb) : prim_of(q, gm1);
     } else {
-      wall_cell_ghost(P, wall, wall_data(wall_tab, wall), qi, qp);
+      const int wall = -1 - nb;
+      wall_cell_ghost(P, wall, wall_data(wall_tab, wall), qi, q);
+      w = prim_of(q, gm1);
     }
-    const R r = fmax(wave_speed(qi, n, gm1), wave_speed(qp, n, gm1));
-    hrs[k] = R(0.5) * r * S;
-    dsum += hrs[k];
+    const R h = R(0.5) * fmax(wave_speed(qi, wi, n), wave_speed(q, w, n)) * n4.w;
+    hrs[at + j * kTile] = h;
+    dsum += h;
   }
   R res[5];
   if constexpr (std::is_same<R, float>::value) {
     ff s[10];
-    face_sums_ff<0, 1>(k0, k1, cf_idx, fface, s);
+    face_sums_ff<0, 1>(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, s);
     const ff h = ff_from(0.5 * dt);
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
@@ -1385,25 +1486,26 @@ __global__ void __launch_bounds__(256) k_jacobi_init(
     }
   } else {
     double s[10];
-    face_sums<0, 1>(k0, k1, cf_idx, fface, s);
+    face_sums<0, 1>(cf_ptr[i], cf_ptr[i + 1], cf_idx, fface, s);
 #pragma unroll
     for (int v = 0; v < 5; ++v) res[v] = s[v] + 0.5 * dt * s[5 + v];
   }
   const R d = (R)(vol[i] / dt) + dsum;
   D[i] = d;
   const R id = R(1) / d;
+  R d0[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) {
     Rv[v * nc + i] = res[v];
-    dQ0[v * nc + i] = res[v] * id;
+    d0[v] = res[v] * id;
   }
+  store_dq(dQ0, i, d0);
 }
 
 template <class R, bool kLast>
 __global__ void __launch_bounds__(256) k_jacobi_sweep(
-    int64_t nc, const int32_t* __restrict__ cf_ptr, const int32_t* __restrict__ cf_idx,
-    const int32_t* __restrict__ f_owner, const int32_t* __restrict__ f_nb,
-    const int8_t* __restrict__ f_wall, const R* __restrict__ fn, const R* __restrict__ QA,
+    int64_t nc, const int32_t* __restrict__ jnb, const R* __restrict__ jn,
+    const R* __restrict__ QA, const R* __restrict__ prim,
     const R* __restrict__ Rv, const R* __restrict__ D, const R* __restrict__ hrs,
     const R* __restrict__ dQin, R* __restrict__ dQout, R* __restrict__ QAout, FluxParams<R> P,
     const R* __restrict__ wall_tab, int* flag) {
@@ -1411,38 +1513,46 @@ __global__ void __launch_bounds__(256) k_jacobi_sweep(
   if (i >= nc) return;
   const R gm1 = P.gamma - R(1);
   R acc[5] = {R(0), R(0), R(0), R(0), R(0)};
-  const int k0 = cf_ptr[i], k1 = cf_ptr[i + 1];
-  for (int k = k0; k < k1; ++k) {
-    R n[3], S, qp[5], dp[5], dT[5];
-    int wall;
-    const int64_t p = other_side(cf_idx[k], f_owner, f_nb, f_wall, fn, n, S, wall);
-    const int64_t c = p >= 0 ? p : i;
-    state_of(QA, c, qp);
+  const int64_t at = i / kTile * kCellFaces * kTile + i % kTile;
+  int32_t nba[kCellFaces];
 #pragma unroll
-    for (int v = 0; v < 5; ++v) dp[v] = dQin[v * nc + c];
-    if (p < 0) {  // the wall's ghost of the cell and of its increment
+  for (int j = 0; j < kCellFaces; ++j) nba[j] = __ldg(jnb + at + j * kTile);
+#pragma unroll
+  for (int j = 0; j < kCellFaces; ++j) {
+    const int32_t nb = nba[j];
+    if (nb == kNoFace) break;
+    const int64_t c = nb >= 0 ? nb : i;
+    R q[5], dp[5];
+    state_of(QA, c, q);
+    JPrim<R> w = load_prim(prim, c);
+    load_dq(dQin, c, dp);
+    const R4<R> n4 = ld4(jn + 4 * (at + j * kTile));
+    const R h = __ldg(hrs + at + j * kTile);
+    if (nb < 0) {  // the wall's ghost of the cell and of its increment
+      const int wall = -1 - nb;
       R qg[5], dg[5];
       const WallData<R> wd = wall_data(wall_tab, wall);
-      wall_cell_ghost(P, wall, wd, qp, qg);
-      wall_cell_ghost_inc(P, wall, wd, qp, dp, dg);
+      wall_cell_ghost(P, wall, wd, q, qg);
+      wall_cell_ghost_inc(P, wall, wd, q, dp, dg);
 #pragma unroll
       for (int v = 0; v < 5; ++v) {
-        qp[v] = qg[v];
+        q[v] = qg[v];
         dp[v] = dg[v];
       }
+      w = prim_of(q, gm1);
     }
-    euler_flux_change(qp, dp, n, gm1, dT);
-    const R h = hrs[k];
+    const R n[3] = {n4.x, n4.y, n4.z}, hS = R(0.5) * n4.w;
+    R dT[5];
+    euler_flux_change(q, w.ir, w.p, dp, n, gm1, dT);
 #pragma unroll
-    for (int v = 0; v < 5; ++v) acc[v] += R(0.5) * S * dT[v] - h * dp[v];
+    for (int v = 0; v < 5; ++v) acc[v] += hS * dT[v] - h * dp[v];
   }
   const R id = R(1) / D[i];
   R d[5];
 #pragma unroll
   for (int v = 0; v < 5; ++v) d[v] = (Rv[v * nc + i] - acc[v]) * id;
   if (!kLast) {
-#pragma unroll
-    for (int v = 0; v < 5; ++v) dQout[v * nc + i] = d[v];
+    store_dq(dQout, i, d);
     return;
   }
   // Q^{n+1} = Q^n + dQ, written to the other gather copy (neighbours still read Q^n)
@@ -1896,29 +2006,29 @@ void launch_s2o4_stage_vjp(int64_t n, int stage, double dt, const double* g, dou
   k_s2o4_stage_vjp<<<blocks_for(n, 256), 256, 0, st>>>(n, stage, c1, c2, g, gQ, gL, gLt, gLts);
 }
 
+constexpr int kJacobiThreads = 64;
 template <class R>
-void launch_jacobi_init(const DevMesh& m, const R* fface, const R* fn, const double* vol,
-                        double dt, const R* QA, R* Rv, R* D, R* hrs, R* dQ0,
-                        const KParams<R>& kp, cudaStream_t st) {
-  k_jacobi_init<R><<<blocks_for(m.nc, 256), 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, m.f_owner,
-                                                          m.f_nb, m.f_wall, fface, fn, vol, dt,
-                                                          QA, flux_params(kp), wall_table<R>(m),
-                                                          Rv, D, hrs, dQ0);
+void launch_jacobi_plan(const DevMesh& m, const R* fn, int32_t* jnb, R* jn, cudaStream_t st) {
+  k_jacobi_plan<R><<<blocks_for(m.n_tiles * kTile, 256), 256, 0, st>>>(
+      m.nc, m.n_tiles, m.cf_ptr, m.cf_idx, m.f_owner, m.f_nb, m.f_wall, fn, jnb, jn);
 }
 template <class R>
-void launch_jacobi_sweep(const DevMesh& m, const R* fn, const R* QA, const R* Rv, const R* D,
-                         const R* hrs, const R* dQin, R* dQout, int last, R* QAout,
-                         const KParams<R>& kp, int* flag, cudaStream_t st) {
-  const unsigned nb = blocks_for(m.nc, 256);
+void launch_jacobi_init(const DevMesh& m, const R* fface, const JacobiBuf<R>& b, const double* vol,
+                        double dt, const R* QA, const KParams<R>& kp, cudaStream_t st) {
   const FluxParams<R> fp = flux_params(kp);
-  if (last)
-    k_jacobi_sweep<R, true><<<nb, 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, m.f_owner, m.f_nb,
-                                                m.f_wall, fn, QA, Rv, D, hrs, dQin, dQout, QAout,
-                                                fp, wall_table<R>(m), flag);
-  else
-    k_jacobi_sweep<R, false><<<nb, 256, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, m.f_owner, m.f_nb,
-                                                 m.f_wall, fn, QA, Rv, D, hrs, dQin, dQout, QAout,
-                                                 fp, wall_table<R>(m), flag);
+  if constexpr (sizeof(R) == 8)
+    k_jacobi_prim<R><<<blocks_for(m.nc, 64), 64, 0, st>>>(m.nc, QA, fp.gamma - R(1), b.prim);
+  k_jacobi_init<R><<<blocks_for(m.nc, kJacobiThreads), kJacobiThreads, 0, st>>>(
+      m.nc, m.cf_ptr, m.cf_idx, b.nb, b.n, fface, vol, dt, QA, b.prim, fp, wall_table<R>(m), b.Rv,
+      b.D, b.hrs, b.dQ[0]);
+}
+template <class R>
+void launch_jacobi_sweep(const DevMesh& m, const JacobiBuf<R>& b, const R* QA, int it, int last,
+                         R* QAout, const KParams<R>& kp, int* flag, cudaStream_t st) {
+  auto kern = last ? k_jacobi_sweep<R, true> : k_jacobi_sweep<R, false>;
+  kern<<<blocks_for(m.nc, kJacobiThreads), kJacobiThreads, 0, st>>>(m.nc, b.nb, b.n, QA, b.prim, b.Rv, b.D,
+                                              b.hrs, b.dQ[(it - 1) & 1], b.dQ[it & 1], QAout,
+                                              flux_params(kp), wall_table<R>(m), flag);
 }
 template <class R>
 void launch_unpack(int64_t nc, const R* QA, double* Q, cudaStream_t st) {
@@ -1985,19 +2095,22 @@ template void launch_stage<float>(const DevMesh&, const GeoR<float>&, const floa
                                   void*, void*, float*, float*, int*, cudaStream_t, double*,
                                   const double*);
 template void launch_unpack<double>(int64_t, const double*, double*, cudaStream_t);
-template void launch_jacobi_init<double>(const DevMesh&, const double*, const double*,
-                                         const double*, double, const double*, double*, double*,
-                                         double*, double*, const KParams<double>&, cudaStream_t);
-template void launch_jacobi_init<float>(const DevMesh&, const float*, const float*, const double*,
-                                        double, const float*, float*, float*, float*, float*,
+template void launch_jacobi_plan<double>(const DevMesh&, const double*, int32_t*, double*,
+                                         cudaStream_t);
+template void launch_jacobi_plan<float>(const DevMesh&, const float*, int32_t*, float*,
+                                        cudaStream_t);
+template void launch_jacobi_init<double>(const DevMesh&, const double*, const JacobiBuf<double>&,
+                                         const double*, double, const double*,
+                                         const KParams<double>&, cudaStream_t);
+template void launch_jacobi_init<float>(const DevMesh&, const float*, const JacobiBuf<float>&,
+                                        const double*, double, const float*,
                                         const KParams<float>&, cudaStream_t);
-template void launch_jacobi_sweep<double>(const DevMesh&, const double*, const double*,
-                                          const double*, const double*, const double*,
-                                          const double*, double*, int, double*,
-                                          const KParams<double>&, int*, cudaStream_t);
-template void launch_jacobi_sweep<float>(const DevMesh&, const float*, const float*, const float*,
-                                         const float*, const float*, const float*, float*, int,
-                                         float*, const KParams<float>&, int*, cudaStream_t);
+template void launch_jacobi_sweep<double>(const DevMesh&, const JacobiBuf<double>&, const double*,
+                                          int, int, double*, const KParams<double>&, int*,
+                                          cudaStream_t);
+template void launch_jacobi_sweep<float>(const DevMesh&, const JacobiBuf<float>&, const float*,
+                                         int, int, float*, const KParams<float>&, int*,
+                                         cudaStream_t);
 template void launch_unpack<float>(int64_t, const float*, double*, cudaStream_t);
 
 }  // namespace gks
