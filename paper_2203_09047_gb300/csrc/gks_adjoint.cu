@@ -93,7 +93,7 @@ __global__ void __launch_bounds__(128) k_vjp_flux(
     int64_t nf, const int32_t* __restrict__ f_owner, const int32_t* __restrict__ f_nb,
     const int8_t* __restrict__ f_wall, const double* __restrict__ fgp,
     const double* __restrict__ poly, const double* __restrict__ gL, const double* __restrict__ gLt,
-    const double* __restrict__ vol, int64_t nc, FluxParams<double> P,
+    const double* __restrict__ ivol, int64_t nc, FluxParams<double> P,
     const double* __restrict__ wall_tab, double dt, int fallback, const double* __restrict__ mom,
     const double* __restrict__ hcell, double* __restrict__ gpf, int* flag) {
   P.full = kFull;
@@ -117,14 +117,14 @@ __global__ void __launch_bounds__(128) k_vjp_flux(
     const int wall = f_wall[f];
     // cotangent of the face flux: L_o -= F / |O_o|, L_nb += F / |O_nb|
     double gacc[10];
-    const double io = 1.0 / vol[o];
+    const double io = ivol[o];
 #pragma unroll
     for (int q = 0; q < 5; ++q) {
       gacc[q] = -gL[q * nc + o] * io;
       gacc[5 + q] = -gLt[q * nc + o] * io;
     }
     if (!kWalls || nb >= 0) {
-      const double in = 1.0 / vol[nb];
+      const double in = ivol[nb];
 #pragma unroll
       for (int q = 0; q < 5; ++q) {
         gacc[q] += gL[q * nc + nb] * in;
@@ -219,9 +219,10 @@ __global__ void k_vjp_poly(int64_t nc, const int32_t* __restrict__ cf_ptr,
 // pipe (about 770 FP64 instructions per thread and 18-member stencil). One thread per cell with
 // the differences, fits and cotangents in local arrays moved 4.1 GB per launch through them: 2.18
 // -> 1.44 ms at 131,072 cells, 478 -> 213 us at 16,384 cells (256 blocks of 64
-// threads left most of the GPU idle).
+// threads left most of the GPU idle); at four blocks per SM (96 registers, some spills) a whole
+// VJP of 131,072 cells 11.09 -> 10.64 ms (two, three, five blocks 10.72, 10.68, 10.68).
 constexpr int kVjpThreads = 5 * kTile;
-__global__ void __launch_bounds__(kVjpThreads) k_vjp_recon(
+__global__ void __launch_bounds__(kVjpThreads, 4) k_vjp_recon(
     int64_t nc, const double* __restrict__ QA, const int32_t* __restrict__ t_K,
     const uint64_t* __restrict__ t_cnt, const int32_t* __restrict__ t_st,
     const int32_t* __restrict__ t_sb, const int32_t* __restrict__ t_idx,
@@ -537,7 +538,7 @@ void launch_vjp(const DevMesh& m, const Geo64& g64, const GeoR<double>& g, const
       cudaDeviceGetLimit(&cur, cudaLimitStackSize) == cudaSuccess && at.localSizeBytes > cur)
     cudaDeviceSetLimit(cudaLimitStackSize, at.localSizeBytes);
   kern<<<blocks_for(4 * m.nf, 128), 128, 0, st>>>(m.nf, m.f_owner, m.f_nb, m.f_wall, g.fgp, poly,
-                                                  gL, gLt, g64.vol, m.nc, fp, m.wall64, dt,
+                                                  gL, gLt, g64.ivol, m.nc, fp, m.wall64, dt,
                                                   p.gp_fallback, g64.mom, g64.h, gpf, flag);
   k_vjp_poly<<<blocks_for(m.nc, 128), 128, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, gpf, gpc);
   int kmax = 0;  // largest stencil of a tile: a column of each thread's differences
