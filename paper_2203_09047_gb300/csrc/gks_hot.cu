@@ -22,6 +22,18 @@ inline unsigned blocks_for(int64_t n, int t) { return (unsigned)((n + t - 1) / t
 // from it. FP32 path: each value is kept as hi + lo floats, so Q_k - Q_0 is formed as
 // (hi_k - hi_0) + (lo_k - lo_0) without FP64 arithmetic and is as accurate as rounding the
 // FP64 difference to FP32. FP64 path: the FP64 values themselves.
+// (double)x by integer arithmetic, for every x: the conversion instruction runs at the FP64 rate
+// (1/64 of the FP32 rate) even where it is predicated off. Subnormal numbers are scaled by 2^64
+// first (exact).
+__device__ __forceinline__ double widen(float x) {
+  const bool sub = (__float_as_uint(x) & 0x7fffffffu) < 0x00800000u;  // subnormal or zero
+  const uint32_t u = __float_as_uint(sub ? x * 18446744073709551616.f : x);
+  const uint32_t m = u & 0x7fffffffu;
+  uint32_t hi = (m >> 3) + (sub ? 0x34000000u : 0x38000000u);
+  if (m == 0) hi = 0;
+  if (m >= 0x7f800000u) hi = 0x7ff00000u | ((m >> 3) & 0xfffffu);  // infinite or NaN
+  return __hiloint2double((int)(hi | (u & 0x80000000u)), (int)(u << 29));
+}
 template <class R>
 struct Gq;
 template <>
@@ -45,7 +57,7 @@ struct Gq<float> {
 #pragma unroll
     for (int v = 0; v < 5; ++v) {
       h[v] = (float)q[v];
-      l[v] = (float)(q[v] - (double)h[v]);
+      l[v] = (float)(q[v] - widen(h[v]));
     }
     float4* p = reinterpret_cast<float4*>(QA + 12 * c);
     p[0] = make_float4(h[0], h[1], h[2], h[3]);
@@ -81,7 +93,7 @@ struct Gq<double> {
 
 // FP64 value of variable v of a gather copy.
 __device__ __forceinline__ double unpack_value(const Gq<float>& g, int v) {
-  return (double)g.hi[v] + (double)g.lo[v];
+  return widen(g.hi[v]) + widen(g.lo[v]);
 }
 __device__ __forceinline__ double unpack_value(const Gq<double>& g, int v) { return g.q[v]; }
 
@@ -1048,12 +1060,23 @@ __device__ __forceinline__ void face_sums(int k0, int k1, const int32_t* __restr
     l[q] = u.h;
     r[q] = __fadd_rn(r[q], u.l);
   });
+  bool rest = false;
 #pragma unroll
   for (int q = kQ0; q < 10; ++q) {
-    double lo = (double)l[q];
-    if (r[q] != 0.f) lo += (double)r[q];
-    s[q] = (double)h[q] + lo;
+    rest = rest || r[q] != 0.f;
+    s[q] = widen(l[q]);
   }
+  if (rest) {
+#pragma unroll 1
+    for (int q = kQ0; q < 10; ++q) {
+      // (selected without a dynamic register index)
+#pragma unroll
+      for (int p = kQ0; p < 10; ++p)
+        if (p == q) s[p] += widen(r[p]);
+    }
+  }
+#pragma unroll
+  for (int q = kQ0; q < 10; ++q) s[q] += widen(h[q]);
 }
 
 // Per cell: L = -(1/|Omega|) sum_f s_f F_f in the cell's fixed face order, and Lt from dF/dt
@@ -1171,7 +1194,13 @@ __global__ void __launch_bounds__(256) k_stage_fd(
     }
   }
   Gq<float>::store(kSecond ? QA : QsA, i, q);
-  if (!physical(q)) atomicOr(flag, kErrNonphysical);
+  // the check in FP32 where that is beyond doubt, else in FP64
+  float f[5];
+#pragma unroll
+  for (int v = 0; v < 5; ++v) f[v] = (float)q[v];
+  const float e = f[0] * f[4], m2 = f[1] * f[1] + f[2] * f[2] + f[3] * f[3];
+  if (!(f[0] > 1e-15f && e < 1e30f && e - 0.5f * m2 > 1e-5f * e + 1e-30f) && !physical(q))
+    atomicOr(flag, kErrNonphysical);
 }
 
 template <bool kSecond, int kB>
