@@ -811,8 +811,9 @@ __device__ __forceinline__ void wall_ghost2(const FluxParams<float>& P, int wall
 //   FP32 smooth, 64^3-cube mesh (2.39 M faces): 0.418 -> 0.326 ms, two points per thread 0.302;
 //   FP32 full, 48^3-cube explosion (1.02 M faces): 326 -> 231 us;
 //   FP64 smooth, 32^3 cubes (299 k faces): 2.53 -> 1.77 ms, with erfc and exp from one table and
-//     one division per state (half_erfc, to_prim) 1.49, sums started from the other side's 1.44;
-//   FP64 full, 124 k faces of tetrahedra: 2.05 -> 1.31, 1.20, 1.16 ms.
+//     one division per state (half_erfc, to_prim) 1.49, sums started from the other side's 1.44,
+//     shorter slopes (side_der) and exchanges that halve the four-point sums 1.39;
+//   FP64 full, 124 k faces of tetrahedra: 2.05 -> 1.31, 1.20, 1.16, 1.14 ms.
 // Resident threads per SM, measured: FP32 smooth 8 blocks of 64 (0.302 ms; of 128 threads 4
 // blocks 0.307, 3 blocks without spills 0.322, 5 blocks 0.407); FP32 full 4 blocks of 128 (231
 // us; 3 and 5 blocks 254 and 254); FP64 unbounded (two blocks).
@@ -951,7 +952,24 @@ __global__ void __launch_bounds__(128, sizeof(R) == 4 ? (kFull ? kFullBlocks : k
       ok = gp_flux_global(P, vl, gl, vr, gr, n1, w, dt, acc);
     if (!ok) atomicOr(flag, kErrNonphysical);
   }
-  // sum the four Gauss points of the face (lanes 4f .. 4f+3 of one warp)
+  // sum the four Gauss points of the face (lanes 4f .. 4f+3 of one warp). Away from walls each
+  // exchange halves what a lane carries: lane bit 0 keeps F^n or dF/dt, bit 1 the first three or
+  // the last two of it (8 additions a lane instead of 20, the same sums), and writes those.
+  if (!__any_sync(0xffffffffu, wall >= 0)) {
+    const int b0 = threadIdx.x & 1, b1 = (threadIdx.x >> 1) & 1;
+    R y[6];
+#pragma unroll
+    for (int q = 0; q < 5; ++q)
+      y[q] = (b0 ? acc[5 + q] : acc[q]) + __shfl_xor_sync(0xffffffffu, b0 ? acc[q] : acc[5 + q], 1);
+    y[5] = R(0);
+    R* rec = fface + (int64_t)kFaceStride * f + 5 * b0 + 3 * b1;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+      const R z = (b1 ? y[3 + q] : y[q]) + __shfl_xor_sync(0xffffffffu, b1 ? y[q] : y[3 + q], 2);
+      if (active && (q < 2 || !b1)) rec[q] = z;
+    }
+    return;
+  }
 #pragma unroll
   for (int q = 0; q < 10; ++q) {
     acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], 1);
