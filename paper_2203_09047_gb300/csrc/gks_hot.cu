@@ -1703,15 +1703,18 @@ __device__ __forceinline__ float dt_bound_f32(const float q[5], float h, const D
   return b > 1e-30f && b < 1e30f ? b : 0.f;
 }
 
-// The smallest bound of all cells, bit for bit the FP64 one: a block takes kDtCells cells per
+// The smallest bound of all cells, bit for bit the FP64 one: a block takes kCells cells per
 // thread at a time, bounds them in FP32, and evaluates in FP64 only those within 2^-9 of the
 // block's smallest (or outside the FP32 range), which contain its FP64 minimum as the FP32 error
 // is far below that. The FP64 evaluation of every cell (two divisions, two square roots and a
 // third division on a pipe of 1/64 of the FP32 rate, 44 us for 442,368 cells) and the passes that
-// unpacked and checked the state before it (25 us) are gone: 69 -> GKS_DT us together.
+// unpacked and checked the state before it (25 us) are gone: 69 -> 16 us together. Each block
+// evaluates at least one warp in FP64, so large meshes take four cells per thread (a call on
+// 442,368 cells 31.6 us, 43.2 with one; on 1,048,576 cells 43 and 76 us); below a block per SM
+// that way, one cell per thread spreads the FP64 work where many cells are alike (60,000 cells of
+// the Riemann tube 35 us, 45 with four).
 constexpr int kDtThreads = 256;
-constexpr int kDtCells = 4;
-constexpr int kDtMaxBlocks = 1024;
+constexpr int kDtMaxBlocks = 8192;
 
 // FP64 state of cell i: Q64 (the FP64-update mode's master copy) or the gather copy.
 template <class R>
@@ -1721,18 +1724,18 @@ __device__ __forceinline__ void state64(const Gq<R>& g, const double* Q64, int64
   for (int v = 0; v < 5; ++v) q[v] = Q64 ? Q64[v * nc + i] : unpack_value(g, v);
 }
 
-template <class R>
+template <class R, int kCells>
 __global__ void __launch_bounds__(kDtThreads) k_dt_partial(
     int64_t nc, const R* __restrict__ QA, const double* __restrict__ Q64,
     const double* __restrict__ hdt, DtParams P, double* partial, int* flag) {
   __shared__ double red[kDtThreads / 32];
   __shared__ float redf[kDtThreads / 32];
   double best = DBL_MAX;
-  constexpr int64_t kChunk = (int64_t)kDtThreads * kDtCells;
+  constexpr int64_t kChunk = (int64_t)kDtThreads * kCells;
   for (int64_t base = blockIdx.x * kChunk; base < nc; base += gridDim.x * kChunk) {
-    float b[kDtCells], lo = FLT_MAX;
+    float b[kCells], lo = FLT_MAX;
 #pragma unroll
-    for (int j = 0; j < kDtCells; ++j) {
+    for (int j = 0; j < kCells; ++j) {
       const int64_t i = base + j * kDtThreads + threadIdx.x;
       b[j] = FLT_MAX;
       if (i >= nc) continue;
@@ -1758,7 +1761,7 @@ __global__ void __launch_bounds__(kDtThreads) k_dt_partial(
     __syncthreads();
     lo *= 1.f + 1.f / 512.f;
 #pragma unroll
-    for (int j = 0; j < kDtCells; ++j) {
+    for (int j = 0; j < kCells; ++j) {
       const int64_t i = base + j * kDtThreads + threadIdx.x;
       if (i >= nc || !(b[j] <= lo)) continue;
       Gq<R> g;
@@ -2095,8 +2098,9 @@ void launch_permute_out(int64_t nc, const int32_t* perm, const double* src, doub
                         cudaStream_t st) {
   k_permute_out<<<blocks_for(nc, 256), 256, 0, st>>>(nc, perm, src, dst);
 }
+constexpr int64_t kDtLargeCells = 152 * 4 * kDtThreads;  // from here on four cells per thread
 int dt_blocks(int64_t nc) {
-  constexpr int64_t chunk = (int64_t)kDtThreads * kDtCells;
+  const int64_t chunk = (nc >= kDtLargeCells ? 4 : 1) * kDtThreads;
   const int64_t b = (nc + chunk - 1) / chunk;
   return (int)(b < kDtMaxBlocks ? b : kDtMaxBlocks);
 }
@@ -2104,8 +2108,9 @@ template <class R>
 void launch_dt(int64_t nc, const R* QA, const double* Q64, const double* hdt, double gamma,
                double mu, int power, double T_ref, double mu_pow, double* partial, int nblocks,
                double* out, int* flag, cudaStream_t st) {
-  k_dt_partial<R><<<nblocks, kDtThreads, 0, st>>>(
-      nc, QA, Q64, hdt, DtParams{gamma, mu, T_ref, mu_pow, power}, partial, flag);
+  auto kern = nc >= kDtLargeCells ? k_dt_partial<R, 4> : k_dt_partial<R, 1>;
+  kern<<<nblocks, kDtThreads, 0, st>>>(nc, QA, Q64, hdt, DtParams{gamma, mu, T_ref, mu_pow, power},
+                                       partial, flag);
   k_dt_final<<<1, 256, 0, st>>>(partial, nblocks, out);
 }
 
