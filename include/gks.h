@@ -14,6 +14,9 @@
  *  - State arrays are float64, structure of arrays [5][n_cells] (rho, rho U, rho V, rho W, rho E),
  *    in the caller's cell order. Unless a call says otherwise they may be host or device
  *    pointers (unified addressing decides); device pointers must be on the solver's device.
+ *    gks_set_state, gks_get_state, gks_residual and gks_residual_vjp read and write device arrays
+ *    in place on the solver's stream (8-byte aligned ones; any other goes through a buffer of the
+ *    solver).
  *    The library never frees or keeps caller pointers beyond a call.
  *  - All device work is enqueued on the stream given to gks_init; calls that return values to
  *    the host (gks_max_dt, status checks) synchronise that stream.
@@ -214,8 +217,8 @@ gks_status gks_step(gks_solver* s, double dt, int nsteps);
 gks_status gks_check(gks_solver* s);
 
 /* Test hook for the bounded wait of the reconstruction (the paper has no counterpart): every
- * later reconstruction of this solver waits for its mbarrier (completed by the bulk copy of the
- * sub-stencil entries into shared memory, where a range stages them) at most wait_tries tries
+ * later reconstruction of this solver waits for its mbarrier (completed by the bulk copies of the
+ * tile's cell record and, where a range stages them, of its sub-stencil entries) at most wait_tries tries
  * per wait (0: the library default of 2^22), and with withhold_copies != 0 issues no copy and
  * expects 16 bytes more than the copies bring, so the barrier never completes, every block
  * gives up after its tries with nothing in flight, and the next status check (gks_check,
@@ -270,7 +273,7 @@ gks_status gks_residual(gks_solver* s, const double* Q, double dt, double* L, do
  * and nonlinear weights of Section 2, the derivative of |x| taken as sign(x) with +1 at 0), in
  * FP64 regardless of the solver's precision; deterministic (per-face and per-cell writes,
  * reverse-stencil gathers, no atomics). The first call allocates the adjoint buffers (and, for
- * a mixed-precision solver, an FP64 copy of the geometry). The flux adjoint keeps up to 1.7 KB
+ * a mixed-precision solver, an FP64 copy of the geometry). The flux adjoint keeps up to 0.9 KB
  * of stack per thread: when the context's per-thread stack limit (cudaLimitStackSize) is
  * smaller, the call raises it, which reserves local memory for every resident thread of the
  * context for as long as the context lives and may synchronise the device. Synchronises the

@@ -315,11 +315,17 @@ __global__ void __launch_bounds__(kVjpThreads, 4) k_vjp_recon(
 #pragma unroll
   for (int g = 0; g < 3; ++g) {
     if (3 * g > M) continue;
-    const double x = inv[3 * g], y = inv[3 * g + 1], z = inv[3 * g + 2], xy = x * y;
-    const double r = 1.0 / (xy * z), rz = r * z;
-    inv[3 * g] = rz * y;
-    inv[3 * g + 1] = rz * x;
-    inv[3 * g + 2] = r * xy;
+    const double x = inv[3 * g], y = inv[3 * g + 1], z = inv[3 * g + 2], xy = x * y, xyz = xy * z;
+    if (mid_range(xy) && mid_range(xyz)) {
+      const double r = 1.0 / xyz, rz = r * z;
+      inv[3 * g] = rz * y;
+      inv[3 * g + 1] = rz * x;
+      inv[3 * g + 2] = r * xy;
+    } else {
+      inv[3 * g] = 1.0 / x;
+      inv[3 * g + 1] = 1.0 / y;
+      inv[3 * g + 2] = 1.0 / z;
+    }
   }
   // w_j = gam_j (1 + r_j^p), r_j = tau inv_j; dw_j/dr_j = gam_j p r_j^(p-1)
   double w[kMaxSub + 1], S = 0.0;
@@ -529,8 +535,8 @@ void launch_vjp(const DevMesh& m, const Geo64& g64, const GeoR<double>& g, const
   // without a collision time the full form is the smooth one, as in the forward
   const Kern kern = fp.tau_model == 0 ? tab[0][1][m.bcs != 0 ? 1 : 0]
                                       : tab[fp.full ? 1 : 0][0][m.bcs != 0 ? 1 : 0];
-  // the flux adjoint keeps kilobytes of spilled state per thread in its stack frame (4-6 KB for
-  // the full flux): raise the context's per-thread stack limit to cover it before the launch
+  // the flux adjoint spills state to its stack frame (0.2-0.9 KB): raise the context's per-thread
+  // stack limit to cover it before the launch
   cudaFuncAttributes at;
   size_t cur = 0;
   if (cudaFuncGetAttributes(&at, kern) == cudaSuccess &&

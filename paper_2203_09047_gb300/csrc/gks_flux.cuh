@@ -314,7 +314,7 @@ GKS_HD void interface_flux(const FluxParams<R>& P, const Prim<R>& w, const R q0[
       E1[1 + j] = U[j] * E1[0] + Un * (c.H[j] + dp[j]) + w.hil * r + n[j] * pd;
     }
     E1[4] = (Ep + p) * (Un * c.divU + nH * w.ir) + Un * (c.G[4] + R(2) * c.Gp) +
-            w.hil * (Nn[4] + Np) + Ep * (Np - w.hil * Nn[0]) * w.ir;
+            w.hil * (Nn[4] + Np) + Ep * ((Np - w.hil * Nn[0]) * w.ir);
   } else {
 #pragma unroll
     for (int q = 0; q < 5; ++q) E1[q] = R(0);

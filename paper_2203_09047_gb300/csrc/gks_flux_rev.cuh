@@ -433,7 +433,7 @@ GKS_HD bool gp_flux_global_vjp(const FluxParams<double>& P, const double vl[5],
       E0[4] = Un * Ep;
       E1[0] = E10;
       E1[4] = (Ep + p) * (Un * c.divU + nH * w.ir) + Un * (c.G[4] + 2.0 * c.Gp) +
-              w.hil * (Nn[4] + Np) + Ep * (Np - w.hil * Nn[0]) * w.ir;
+              w.hil * (Nn[4] + Np) + Ep * ((Np - w.hil * Nn[0]) * w.ir);
       E2[0] = dmn;
       E2[4] = r2 * w.ir * Ep + Un * (t[4] + dpt);
 #pragma unroll

@@ -372,9 +372,8 @@ __device__ __forceinline__ float wdiv<float>(float a, float b) {
 
 // b[s] <- tau / b[s], s = 0..M (M <= 8; the entries beyond M are 1). FP32: one fast quotient
 // each. FP64: a division is a chain of a dozen FP64 instructions on a pipe that bounds the
-// kernel, so three reciprocals are taken from one division of 1 by the product of the three
-// (each product rounds once more; the indicators lie between the weights' epsilon and far below
-// 10^102, so no product leaves the range).
+// kernel, so three quotients are taken from one division by the product of the three (each product
+// rounds once more); a product near the ends of the FP64 range takes the three divisions.
 template <class R>
 __device__ __forceinline__ void quotients(R tau, int M, R b[kMaxSub + 1]) {
 #pragma unroll
@@ -386,11 +385,17 @@ __device__ __forceinline__ void quotients<double>(double tau, int M, double b[kM
 #pragma unroll
   for (int g = 0; g < 3; ++g) {
     if (3 * g > M) continue;
-    const double x = b[3 * g], y = b[3 * g + 1], z = b[3 * g + 2], xy = x * y;
-    const double r = tau / (xy * z), rz = r * z;
-    b[3 * g] = rz * y;
-    b[3 * g + 1] = rz * x;
-    b[3 * g + 2] = r * xy;
+    const double x = b[3 * g], y = b[3 * g + 1], z = b[3 * g + 2], xy = x * y, xyz = xy * z;
+    if (mid_range(xy) && mid_range(xyz)) {
+      const double r = tau / xyz, rz = r * z;
+      b[3 * g] = rz * y;
+      b[3 * g + 1] = rz * x;
+      b[3 * g + 2] = r * xy;
+    } else {
+      b[3 * g] = tau / x;
+      b[3 * g + 1] = tau / y;
+      b[3 * g + 2] = tau / z;
+    }
   }
 }
 
@@ -564,7 +569,8 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM<R>) k_recon(
   const bool sub_warp = warp >= kRowWarps;
   const int s_first = sub_warp ? warp - kRowWarps : (kStB ? kMaxSub : kRowShare + warp);
   const int s_end = !kStB && sub_warp && Mt > kRowShare ? kRowShare : Mt;
-  for (int s = s_first; s < s_end; s += sub_warp ? kReconWarps - kRowWarps : kMaxSub) {
+  // (a wait that ran out left no entries to index with)
+  for (int s = s_first; ok && s < s_end; s += sub_warp ? kReconWarps - kRowWarps : kMaxSub) {
     int slot = 0;
     for (int q = 0; q < s; ++q) slot += (int)((cnt >> (8 * q)) & 0xffu);
     const int cs = (int)((cnt >> (8 * s)) & 0xffu);
@@ -1356,7 +1362,8 @@ template <class R>
 __device__ __forceinline__ JPrim<R> prim_of(const R q[5], R gm1) {
   JPrim<R> w;
   w.ir = R(1) / q[0];
-  w.p = gm1 * (q[4] - R(0.5) * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) * w.ir);
+  w.p = gm1 * (q[4] - R(0.5) * (q[1] * (q[1] * w.ir) + q[2] * (q[2] * w.ir) +
+                                q[3] * (q[3] * w.ir)));
   const R c2 = (gm1 + R(1)) * w.p * w.ir;
   w.c = sqrt(c2 > R(0) ? c2 : R(0));
   w.pad = R(0);
@@ -1364,7 +1371,7 @@ __device__ __forceinline__ JPrim<R> prim_of(const R q[5], R gm1) {
 }
 template <class R>
 __device__ __forceinline__ R wave_speed(const R q[5], const JPrim<R>& w, const R n[3]) {
-  return fabs((q[1] * n[0] + q[2] * n[1] + q[3] * n[2]) * w.ir) + w.c;
+  return fabs(q[1] * w.ir * n[0] + q[2] * w.ir * n[1] + q[3] * w.ir * n[2]) + w.c;
 }
 template <class R>
 __device__ __forceinline__ void euler_flux_change(const R q[5], R ir, R p, const R d[5],

@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstdint>
+#include <cstring>
 
 #include "gks_internal.h"
 
@@ -23,12 +25,11 @@ GKS_HD double k_abs(double x) { return fabs(x); }
 GKS_HD float k_abs(float x) { return fabsf(x); }
 GKS_HD double k_pow(double x, double y) { return pow(x, y); }
 GKS_HD float k_pow(float x, float y) { return powf(x, y); }
-// Quotients of the per-state terms (reciprocals of rho and p, the half-line B, the frame
-// normalisation, the pressure jump): the IEEE division, except for FP32 on the device, which
-// takes the fast division intrinsic (within 2 ulp for divisors below 2^126). FP32 flux per
-// launch, against IEEE divisions: smooth form 0.438 -> 0.421 ms on the 64^3-cube mesh, full
-// form 6.52 -> 6.12 ms on the 128^3-cube explosion, 6.06 with the collision time and the
-// time-fit quotients as well.
+// Quotients of the per-state terms (reciprocals of rho and p, the half-line B, the pressure
+// jump): the IEEE division, except for FP32 on the device, which takes the fast division intrinsic
+// (within 2 ulp for divisors below 2^126). Against IEEE divisions, in the face-frame form of the
+// flux that preceded this one: smooth 0.438 -> 0.421 ms per launch on the 64^3-cube mesh, full
+// 6.52 -> 6.06 ms on the 128^3-cube explosion.
 template <class R>
 GKS_HD R k_div(R a, R b) {
   return a / b;
@@ -61,19 +62,33 @@ GKS_HD bool to_prim(const R q[5], R gamma, Prim<R>& w) {
   w.hil = w.p * w.ir;
   return (w.rho > R(0)) && (w.p > R(0));  // false also for NaN
 }
+// Whether a positive x lies well inside the FP64 range (2^-940 to 2^940), by its exponent bits.
+GKS_HD bool mid_range(double x) {
+#ifdef __CUDA_ARCH__
+  const uint32_t hi = (uint32_t)__double2hiint(x);
+#else
+  uint64_t u;
+  memcpy(&u, &x, sizeof(u));
+  const uint32_t hi = (uint32_t)(u >> 32);
+#endif
+  return hi - 0x05300000u < 0x75800000u;  // false for negative, zero, infinite and NaN as well
+}
 // FP64: both reciprocals from one division, 1 / (rho rho p) (a division is a chain of about ten
-// instructions on the FP64 pipe, which bounds the FP64 kernels).
+// instructions on the FP64 pipe, which bounds the FP64 kernels), where that product is positive
+// and far from the ends of the range.
 GKS_HD bool to_prim(const double q[5], double gamma, Prim<double>& w) {
   w.rho = q[0];
   const double rp = (gamma - 1.0) *
                     (q[0] * q[4] - 0.5 * (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]));  // rho p
-  const double r = 1.0 / (q[0] * rp);
+  const double rrp = q[0] * rp;
+  if (!mid_range(rrp) || !mid_range(rp)) return to_prim<double>(q, gamma, w);
+  const double r = 1.0 / rrp;
   w.ir = rp * r;
   w.U = q[1] * w.ir;
   w.V = q[2] * w.ir;
   w.W = q[3] * w.ir;
   w.p = rp * w.ir;
-  w.ip = q[0] * q[0] * r;
+  w.ip = q[0] * (q[0] * r);
   w.lam = 0.5 * w.rho * w.ip;
   w.hil = w.p * w.ir;
   return (w.rho > 0.0) && (w.p > 0.0);

@@ -50,3 +50,22 @@ def test_forms_against_oracle(layers, n, shape, min_stencil, wpow):
     lhs = (S.residual_vjp(Q, dt, gL, gLt).cpu().numpy() * dQ).sum()
     rhs = (gL * dL).sum() + (gLt * dLt).sum()
     assert abs(lhs - rhs) <= 1e-10 * abs(rhs), (lhs, rhs)
+
+
+@pytest.mark.parametrize("weps", [1e-150, 1e-110, 1e120, 1e200])
+def test_extreme_weight_epsilon(weps):
+    """Epsilons whose threefold product leaves the FP64 range, with variables whose indicators are
+    zero (gas at rest): the weights take the general divisions."""
+    m = I.layered_box_mesh(8, "hybrid8", shape=(5, 6))
+    om = oracle.Mesh(m, min_stencil=18)
+    Q = np.zeros((5, om.n_cells))
+    Q[0] = 1.0 + 0.1 * I.uniform01(53, np.arange(om.n_cells, dtype=np.uint64))
+    Q[4] = 2.5
+    p = dict(weno_eps=weps)
+    Lo, _ = om.residual(oracle.params_vec(**p), Q, 0.01)
+    S = gks.Solver(m, min_stencil=18, **p)
+    L, Lt = S.residual(Q, 0.01)
+    assert rel(L.cpu(), Lo) < 1e-12 and np.isfinite(Lt.cpu().numpy()).all()
+    gL, gLt, dQ = I.normal_directions(Q.shape, 3, 54)
+    g = S.residual_vjp(Q, 0.01, gL, gLt).cpu().numpy()
+    assert np.isfinite(g).all()
