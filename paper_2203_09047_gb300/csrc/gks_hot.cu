@@ -532,10 +532,9 @@ __global__ void __launch_bounds__(kReconThreads, kReconBlocksPerSM<R>) k_recon(
     if (!ok) ok = mbar_wait(bar, 0, tries);  // let copies still in flight land before leaving
   };
 
-  // phase 2: rows n = warp, warp + 5 of a = A+ dq (both in one member loop: each stencil
-  // difference is read once for the two rows), and the sub-stencil fits b_m with their
-  // indicators beta_m = |b_m|^2 (scaled coordinates); sub-stencils go to the warps in reverse
-  // order (m = 4 - warp, 9 - warp) so that the warp with one row takes two of them
+  // phase 2: rows n = 3 warp .. 3 warp + 2 of a = A+ dq on the row warps (in one member loop:
+  // each stencil difference is read once for the three rows), and the sub-stencil fits b_m with
+  // their indicators beta_m = |b_m|^2 (scaled coordinates) on the others meanwhile
   if (warp < kRowWarps) {
     R acc[3][5];
 #pragma unroll
