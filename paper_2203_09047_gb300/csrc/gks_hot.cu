@@ -1683,6 +1683,7 @@ __global__ void k_permute_out(int64_t nc, const int32_t* __restrict__ perm,
 struct DtParams {
   double gamma, mu, T_ref, mu_pow;
   int power;
+  float gm1;  // gamma - 1 of the FP64 gamma, for the FP32 estimate
 };
 __device__ __forceinline__ double dt_bound(const double q[5], double h, const DtParams& P) {
   const double u2 = (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) / (q[0] * q[0]);
@@ -1701,8 +1702,8 @@ __device__ __forceinline__ float dt_bound_f32(const float q[5], float h, const D
   ok = q[0] > 1e-15f && q[0] < 1e15f && h > 1e-15f && h < 1e15f && q[4] < 1e15f &&
        e - 0.5f * m2 > 1e-5f * e;
   if (!ok) return 0.f;
-  const float ir = 1.f / q[0], gm1 = (float)P.gamma - 1.f;
-  const float p = gm1 * (e - 0.5f * m2) * ir;
+  const float ir = 1.f / q[0];
+  const float p = P.gm1 * (e - 0.5f * m2) * ir;
   const float mue = P.power ? (float)P.mu * powf(p * ir / (float)P.T_ref, (float)P.mu_pow)
                             : (float)P.mu;
   const float b = h / (sqrtf(m2) * ir + sqrtf((float)P.gamma * p * ir) + 2.f * mue * ir / h);
@@ -2115,8 +2116,8 @@ void launch_dt(int64_t nc, const R* QA, const double* Q64, const double* hdt, do
                double mu, int power, double T_ref, double mu_pow, double* partial, int nblocks,
                double* out, int* flag, cudaStream_t st) {
   auto kern = nc >= kDtLargeCells ? k_dt_partial<R, 4> : k_dt_partial<R, 1>;
-  kern<<<nblocks, kDtThreads, 0, st>>>(nc, QA, Q64, hdt, DtParams{gamma, mu, T_ref, mu_pow, power},
-                                       partial, flag);
+  const DtParams P{gamma, mu, T_ref, mu_pow, power, (float)(gamma - 1.0)};
+  kern<<<nblocks, kDtThreads, 0, st>>>(nc, QA, Q64, hdt, P, partial, flag);
   k_dt_final<<<1, 256, 0, st>>>(partial, nblocks, out);
 }
 

@@ -1,0 +1,56 @@
+"""The time-step bound where the FP32 estimate that chooses the cells to evaluate in FP64 is weakest,
+against the oracle on the same states. The cells are of two kinds whose true bounds lie a few
+percent apart, so that an estimate that is off by more than its margin of 2^-9 picks the wrong
+kind and returns a step above the bound.
+
+Tolerance: a few roundings of 2^-53 (FP64) or of the float-float state, 2^-47, raised by the
+cancellation of the pressure, rho E over the internal energy."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+import oracle  # noqa: E402
+import paper_2203_09047_gb300 as gks  # noqa: E402
+from paper_2203_09047_gb300 import build, inputs as I  # noqa: E402
+
+PRECISIONS = [gks.GKS_PREC_FP64, gks.GKS_PREC_MIXED, gks.GKS_PREC_MIXED_FP64UPD]
+
+
+@pytest.fixture(scope="module")
+def cubes():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    build.build()
+    gks.load_library()
+    m = I.layered_box_mesh(8, "hex", jitter=0.0)  # every cell has the same size
+    return m, oracle.Mesh(m)
+
+
+def check(cubes, rho, U, e, prec, **prm):
+    """rho [n], U [n, 3], internal energy per mass e [n]."""
+    m, om = cubes
+    q = np.ascontiguousarray(np.stack([rho, *(rho[:, None] * U).T,
+                                       rho * (e + 0.5 * (U * U).sum(1))]))
+    S = gks.Solver(m, precision=prec, **prm)
+    S.set_state(q)
+    ref = om.max_dt(oracle.params_vec(**prm), q, 0.5)
+    cond = float((1.0 + 0.5 * (U * U).sum(1) / e).max())
+    tol = 8 * cond * 2.0 ** (-53 if prec == gks.GKS_PREC_FP64 else -46) + 1e-11
+    assert abs(S.max_dt(0.5) - ref) <= tol * ref
+
+
+def two_kinds(n):
+    return np.arange(n) % 2 == 0
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("gm1", [1e-3, 3e-7, 1e-7])
+def test_gamma_near_one(cubes, prec, gm1):
+    """Sound speed 1 at rest against a stream at 1.03: gamma - 1 has to be that of the FP64 gamma
+    (rounded to FP32 first, gamma - 1 = 3e-7 becomes 3.6e-7)."""
+    n, a, g = 512, two_kinds(512), 1.0 + gm1
+    U = np.zeros((n, 3))
+    U[~a, 0] = 1.03
+    check(cubes, np.ones(n), U, np.where(a, 1.0 / (g * (g - 1.0)), 1.0), prec, gamma=g)
