@@ -1693,20 +1693,26 @@ __device__ __forceinline__ double dt_bound(const double q[5], double h, const Dt
   const double mue = P.power ? P.mu * pow(p / (q[0] * P.T_ref), P.mu_pow) : P.mu;
   return h / (sqrt(u2) + c + 2.0 * mue / (q[0] * h));
 }
-// The same in FP32, to about 1e-5 for states and sizes well inside the FP32 range; 0 for any
-// other, which every caller takes as "evaluate in FP64". ok: rho > 0 and p > 0 beyond doubt.
+// The same in FP32, to about 1e-4 for states and sizes whose products stay inside the FP32 range;
+// 0 for any other, which every caller takes as "evaluate in FP64". ok: rho > 0 and p > 0 beyond
+// doubt. With w = rho p the three speeds have 1 / rho in common (c = sqrt(gamma w) / rho), so that
+// the lower limits of w, E and h keep every quantity that matters normal: what may still be
+// subnormal beside them (a kinetic energy, a viscous term) is below 1e-7 of the sum.
 __device__ __forceinline__ float dt_bound_f32(const float q[5], float h, const DtParams& P,
                                               bool& ok) {
   const float m2 = q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
-  const float e = q[0] * q[4];
-  ok = q[0] > 1e-15f && q[0] < 1e15f && h > 1e-15f && h < 1e15f && q[4] < 1e15f &&
-       e - 0.5f * m2 > 1e-5f * e;
+  const float e = q[0] * q[4], d = e - 0.5f * m2, w = P.gm1 * d;
+  ok = q[0] > 1e-15f && q[0] < 1e15f && h > 1e-15f && h < 1e15f && q[4] > 1e-25f &&
+       q[4] < 1e15f && d > 1e-5f * e && w > 1e-30f;
   if (!ok) return 0.f;
   const float ir = 1.f / q[0];
-  const float p = P.gm1 * (e - 0.5f * m2) * ir;
-  const float mue = P.power ? (float)P.mu * powf(p * ir / (float)P.T_ref, (float)P.mu_pow)
-                            : (float)P.mu;
-  const float b = h / (sqrtf(m2) * ir + sqrtf((float)P.gamma * p * ir) + 2.f * mue * ir / h);
+  float mue = (float)P.mu;
+  if (P.power) {
+    const float T = w * ir * ir, t = T / (float)P.T_ref;
+    if (!(T > 1e-30f && t > 1e-10f && t < 1e10f)) return 0.f;
+    mue *= powf(t, (float)P.mu_pow);
+  }
+  const float b = h / ((sqrtf(m2) + sqrtf((float)P.gamma * w) + 2.f * mue / h) * ir);
   return b > 1e-30f && b < 1e30f ? b : 0.f;
 }
 

@@ -54,3 +54,14 @@ def test_gamma_near_one(cubes, prec, gm1):
     U = np.zeros((n, 3))
     U[~a, 0] = 1.03
     check(cubes, np.ones(n), U, np.where(a, 1.0 / (g * (g - 1.0)), 1.0), prec, gamma=g)
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("rho,c", [(1e-10, 1.9545e-12), (1e-10, 2.6e-12)])
+def test_states_whose_products_are_subnormal_in_fp32(cubes, prec, rho, c):
+    """rho E of a few units of the smallest FP32 number: such cells are evaluated in FP64."""
+    n, a = 512, two_kinds(512)
+    U = np.zeros((n, 3))
+    U[~a, 1] = 0.8 * c
+    e = c * c / (1.4 * 0.4)
+    check(cubes, np.full(n, rho), U, np.where(a, e, 0.02 * e), prec)
