@@ -1684,7 +1684,14 @@ struct DtParams {
   double gamma, mu, T_ref, mu_pow;
   int power;
   float gm1;  // gamma - 1 of the FP64 gamma, for the FP32 estimate
+  float cut;  // smallest share of the internal energy in rho E that the estimate takes
 };
+// FP32 rounds rho E and |m|^2 / 2 to about 5e-7 of rho E. In the sum of the speeds that is at most
+// 1e-4 down to an internal share of 1e-5, as the speed of sound is small beside |U| there; the
+// viscosity of the power law has it in full, times the exponent over the share.
+inline float dt_cut(int power, double mu_pow) {
+  return power ? std::max(1e-5f, 4e-3f * (float)fabs(mu_pow)) : 1e-5f;
+}
 __device__ __forceinline__ double dt_bound(const double q[5], double h, const DtParams& P) {
   const double u2 = (q[1] * q[1] + q[2] * q[2] + q[3] * q[3]) / (q[0] * q[0]);
   const double p = (P.gamma - 1.0) * (q[4] - 0.5 * q[0] * u2);
@@ -1693,7 +1700,8 @@ __device__ __forceinline__ double dt_bound(const double q[5], double h, const Dt
   const double mue = P.power ? P.mu * pow(p / (q[0] * P.T_ref), P.mu_pow) : P.mu;
   return h / (sqrt(u2) + c + 2.0 * mue / (q[0] * h));
 }
-// The same in FP32, to about 1e-4 for states and sizes whose products stay inside the FP32 range;
+// The same in FP32, to better than 6e-4 (1e-4 without the power law; the margin of k_dt_partial is
+// 2^-9 = 2e-3 for two such errors) for states and sizes whose products stay inside the FP32 range;
 // 0 for any other, which every caller takes as "evaluate in FP64". ok: rho > 0 and p > 0 beyond
 // doubt. With w = rho p the three speeds have 1 / rho in common (c = sqrt(gamma w) / rho), so that
 // the lower limits of w, E and h keep every quantity that matters normal: what may still be
@@ -1703,7 +1711,7 @@ __device__ __forceinline__ float dt_bound_f32(const float q[5], float h, const D
   const float m2 = q[1] * q[1] + q[2] * q[2] + q[3] * q[3];
   const float e = q[0] * q[4], d = e - 0.5f * m2, w = P.gm1 * d;
   ok = q[0] > 1e-15f && q[0] < 1e15f && h > 1e-15f && h < 1e15f && q[4] > 1e-25f &&
-       q[4] < 1e15f && d > 1e-5f * e && w > 1e-30f;
+       q[4] < 1e15f && d > P.cut * e && w > 1e-30f;
   if (!ok) return 0.f;
   const float ir = 1.f / q[0];
   float mue = (float)P.mu;
@@ -1718,8 +1726,8 @@ __device__ __forceinline__ float dt_bound_f32(const float q[5], float h, const D
 
 // The smallest bound of all cells, bit for bit the FP64 one: a block takes kCells cells per
 // thread at a time, bounds them in FP32, and evaluates in FP64 only those within 2^-9 of the
-// block's smallest (or outside the FP32 range), which contain its FP64 minimum as the FP32 error
-// is far below that. The FP64 evaluation of every cell (two divisions, two square roots and a
+// block's smallest (or outside the estimate's range), which contain its FP64 minimum as two errors
+// of the estimate are below that. The FP64 evaluation of every cell (two divisions, two square roots and a
 // third division on a pipe of 1/64 of the FP32 rate, 44 us for 442,368 cells) and the passes that
 // unpacked and checked the state before it (25 us) are gone: 69 -> 16 us together. Each block
 // evaluates at least one warp in FP64, so large meshes take four cells per thread (a call on
@@ -2122,7 +2130,7 @@ void launch_dt(int64_t nc, const R* QA, const double* Q64, const double* hdt, do
                double mu, int power, double T_ref, double mu_pow, double* partial, int nblocks,
                double* out, int* flag, cudaStream_t st) {
   auto kern = nc >= kDtLargeCells ? k_dt_partial<R, 4> : k_dt_partial<R, 1>;
-  const DtParams P{gamma, mu, T_ref, mu_pow, power, (float)(gamma - 1.0)};
+  const DtParams P{gamma, mu, T_ref, mu_pow, power, (float)(gamma - 1.0), dt_cut(power, mu_pow)};
   kern<<<nblocks, kDtThreads, 0, st>>>(nc, QA, Q64, hdt, P, partial, flag);
   k_dt_final<<<1, 256, 0, st>>>(partial, nblocks, out);
 }

@@ -65,3 +65,39 @@ def test_states_whose_products_are_subnormal_in_fp32(cubes, prec, rho, c):
     U[~a, 1] = 0.8 * c
     e = c * c / (1.4 * 0.4)
     check(cubes, np.full(n, rho), U, np.where(a, e, 0.02 * e), prec)
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+@pytest.mark.parametrize("mach,warm,mu_pow", [(540.0, 0.998, 0.7), (540.0, 0.9995, 0.7),
+                                              (30.0, 0.9995, 0.7), (60.0, 0.999, 40.0), (2.0, 1.01, -300.0)])
+def test_power_law_viscosity_of_fast_gas(cubes, prec, mach, warm, mu_pow):
+    """A bound set by mu(T): the temperature of a fast gas loses rho E over the internal energy in
+    FP32, the exponent multiplies that."""
+    n, a = 512, two_kinds(512)
+    rng = np.random.default_rng(3)
+    d = rng.normal(size=(n, 3))
+    d /= np.linalg.norm(d, axis=1, keepdims=True)
+    U = np.where(a, 0.0, mach * np.sqrt(1.4) * (0.95 + 0.05 * rng.random(n)))[:, None] * d
+    check(cubes, np.ones(n), U, np.where(a, 1.0, warm) / 0.4, prec, mu=1e6, tau_model=3, T_ref=1.0,
+          mu_pow=mu_pow)
+
+
+@pytest.mark.parametrize("prec", PRECISIONS)
+def test_large_ragged_mesh(prec):
+    """Four cells per thread (from 155,648 cells on), the last block partly filled; the smallest
+    bound in the first, the last and an inner cell."""
+    m = I.layered_box_mesh(32, "hex", shape=(71, 69))
+    om = oracle.Mesh(m, lazy=True)
+    n = om.n_cells
+    assert n >= 155648 and n % 1024
+    rng = np.random.default_rng(64)
+    rho, u = 1 + 0.3 * rng.random(n), 0.5 * rng.normal(size=(n, 3))
+    q = I.primitive_to_conserved(rho, u, 1 + 0.3 * rng.random(n))
+    S = gks.Solver(m, precision=prec, mu=1e-4, tau_model=2)
+    for cell in (None, 0, n // 3, n - 1):
+        x = q.copy()
+        if cell is not None:
+            x[4, cell] *= 300.0
+        S.set_state(np.ascontiguousarray(x))
+        ref = om.max_dt(oracle.params_vec(mu=1e-4, tau_model=2), np.ascontiguousarray(x), 0.5)
+        assert abs(S.max_dt(0.5) - ref) <= (1e-13 if prec == gks.GKS_PREC_FP64 else 1e-11) * ref
