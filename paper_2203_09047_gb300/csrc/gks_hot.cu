@@ -373,7 +373,8 @@ __device__ __forceinline__ float wdiv<float>(float a, float b) {
 // b[s] <- tau / b[s], s = 0..M (M <= 8; the entries beyond M are 1). FP32: one fast quotient
 // each. FP64: a division is a chain of a dozen FP64 instructions on a pipe that bounds the
 // kernel, so three quotients are taken from one division by the product of the three (each product
-// rounds once more); a product near the ends of the FP64 range takes the three divisions.
+// rounds once more) where tau and the three lie in 2^-240..2^240 (tau may be zero: uniform data),
+// so that nothing on the way leaves the FP64 range; else the three divisions.
 template <class R>
 __device__ __forceinline__ void quotients(R tau, int M, R b[kMaxSub + 1]) {
 #pragma unroll
@@ -382,12 +383,17 @@ __device__ __forceinline__ void quotients(R tau, int M, R b[kMaxSub + 1]) {
 }
 template <>
 __device__ __forceinline__ void quotients<double>(double tau, int M, double b[kMaxSub + 1]) {
+  // positive and within 2^-240..2^240, by the exponent bits
+  auto inner = [](double x) {
+    return (uint32_t)__double2hiint(x) - 0x30f00000u < 0x1e000000u;
+  };
+  const bool tau_ok = inner(tau) || tau == 0.0;
 #pragma unroll
   for (int g = 0; g < 3; ++g) {
     if (3 * g > M) continue;
-    const double x = b[3 * g], y = b[3 * g + 1], z = b[3 * g + 2], xy = x * y, xyz = xy * z;
-    if (mid_range(xy) && mid_range(xyz)) {
-      const double r = tau / xyz, rz = r * z;
+    const double x = b[3 * g], y = b[3 * g + 1], z = b[3 * g + 2];
+    if (tau_ok && inner(x) && inner(y) && inner(z)) {
+      const double xy = x * y, r = tau / (xy * z), rz = r * z;
       b[3 * g] = rz * y;
       b[3 * g + 1] = rz * x;
       b[3 * g + 2] = r * xy;
