@@ -1074,9 +1074,11 @@ __device__ __forceinline__ void face_sums(int k0, int k1, const int32_t* __restr
 }
 // FP64 sums of FP32 face fluxes without FP64 arithmetic in the loop (GB300 runs FP64 at 1/64 of
 // the FP32 rate): each component is an unevaluated sum h + l + r of floats, TwoSum (Knuth)
-// carrying the rounding errors of h into l and those of l into r, so nothing above 2^-72 of the
-// sum is lost and the value handed on is the exact sum rounded to FP64 (a double accumulation
-// rounds at every face). r is zero unless the fluxes of a cell differ by more than 2^20.
+// carrying the rounding errors of h into l and those of l into r. As long as r is zero (the
+// partial sums fit 48 bits), h + l is the exact sum and the value handed on is rounded once, where
+// a double accumulation rounds at every face; otherwise the roundings of r lose about 2^-72 of the
+// largest partial sum and the value is rounded twice. A partial sum beyond the FP32 range, or a
+// flux that is not finite, leaves NaN in r: such a cell is summed in FP64.
 template <int kQ0, int kB>
 __device__ __forceinline__ void face_sums(int k0, int k1, const int32_t* __restrict__ cf_idx,
                                           const float* __restrict__ fface, double s[10]) {
@@ -1089,11 +1091,18 @@ __device__ __forceinline__ void face_sums(int k0, int k1, const int32_t* __restr
     l[q] = u.h;
     r[q] = __fadd_rn(r[q], u.l);
   });
-  bool rest = false;
+  bool rest = false, range = true;
 #pragma unroll
   for (int q = kQ0; q < 10; ++q) {
     rest = rest || r[q] != 0.f;
+    range = range && fabsf(r[q]) <= FLT_MAX;
     s[q] = widen(l[q]);
+  }
+  if (!range) {
+#pragma unroll
+    for (int q = kQ0; q < 10; ++q) s[q] = 0.0;
+    face_loop<kQ0, 1>(k0, k1, cf_idx, fface, [&](int q, float x) { s[q] += widen(x); });
+    return;
   }
   if (rest) {
 #pragma unroll 1
