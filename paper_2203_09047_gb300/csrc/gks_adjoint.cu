@@ -550,8 +550,11 @@ void launch_vjp(const DevMesh& m, const Geo64& g64, const GeoR<double>& g, const
   int kmax = 0;  // largest stencil of a tile: a column of each thread's differences
   for (int r = 0; r < m.rr.n; ++r) kmax = m.rr.K[r] > kmax ? m.rr.K[r] : kmax;
   const size_t smem = sizeof(double) * kVjpThreads * kmax;
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(k_vjp_recon, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  // the limit of the largest stencil, whatever this mesh's (solvers in several threads share it)
+  if (smem > 48 * 1024 &&
+      cudaFuncSetAttribute(k_vjp_recon, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(sizeof(double) * kVjpThreads * kMaxStencil)) != cudaSuccess)
+    return;
   k_vjp_recon<<<(unsigned)m.n_tiles, kVjpThreads, smem, st>>>(
       m.nc, QA, m.t_K, m.t_cnt, m.t_st, m.t_sb, m.t_idx, m.st_ptr, g.Ap, g.Bp, g.cell,
       p.weno_gamma, p.weno_eps, p.weno_pow, gpc, gdq, gq0);

@@ -1853,8 +1853,13 @@ void launch_recon_ranges(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p
     set.r[r - r0] = ReconUni{m.rr.uni[r], m.rr.K[r],  m.rr.S[r], m.rr.cnt[r],
                              m.rr.st0[r], m.rr.sb0[r], m.rr.t0[r]};
   auto run = [&](auto kern, const auto& arg) {
-    if (smem > 48 * 1024)
-      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // the limit belongs to the kernel, not to this mesh: always the same value, so that solvers of
+    // other sizes in other threads cannot lower it before the launch (a failure is left to the
+    // caller's check)
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kMaxBlockSmem) != cudaSuccess)
+      return;
     kern<<<(unsigned)(m.rr.t1[r1 - 1] - m.rr.t0[r0]), kReconThreads, smem, st>>>(
         m.nc, m.rr.t0[r0], K, S, M, arg, QA, m.t_K, m.t_cnt, m.t_st, m.t_sb, m.t_idx, g.Ap, g.Bp,
         g.cell, p.weno_gamma, p.weno_eps, p.weno_pow, poly, flag, p.wait_tries, p.withhold);
