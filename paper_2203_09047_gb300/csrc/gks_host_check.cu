@@ -202,46 +202,48 @@ gks::FluxParams<float> params_f32(const double* p) {
 }
 // point i: in[45 i ..] = vl[5], gl[5][3], vr[5], gr[5][3], n1[3], w, dt;
 // out[21 i ..] = scalar acc[10], packed acc[10], (scalar ok) + 2 (packed ok). The packed form is
-// the kernels': the smooth form pairs point i with the next one (first half: point i), the full
-// form the two sides of point i.
-__global__ void k_face_f32_pair(gks::FluxParams<float> P, int n, const float* __restrict__ in,
-                                float* __restrict__ out) {
+// the kernels': the smooth form pairs points 2 j and 2 j + 1 (the last of an odd count with point
+// 0) and each takes its own half, the full form (and with sides != 0 the smooth form of small
+// meshes) the two sides of point i.
+__global__ void k_face_f32_pair(gks::FluxParams<float> P, int n, int sides,
+                                const float* __restrict__ in, float* __restrict__ out) {
   using gks::P2;
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const float* x = in + 45 * (int64_t)i;
-  const float* y = in + 45 * (int64_t)((i + 1) % n);
   float vl[5], gl[5][3], vr[5], gr[5][3], n1[3];
-  P2 v[5], g[5][3], nn[3], acc2[10];
   for (int k = 0; k < 5; ++k) {
     vl[k] = x[k];
     vr[k] = x[20 + k];
-    v[k] = P2(x[k], y[k]);
     for (int a = 0; a < 3; ++a) {
       gl[k][a] = x[5 + 3 * k + a];
       gr[k][a] = x[25 + 3 * k + a];
-      g[k][a] = P2(x[5 + 3 * k + a], y[5 + 3 * k + a]);
     }
   }
-  for (int a = 0; a < 3; ++a) {
-    n1[a] = x[40 + a];
-    nn[a] = P2(x[40 + a], y[40 + a]);
-  }
+  for (int a = 0; a < 3; ++a) n1[a] = x[40 + a];
   const float w = x[43], dt = x[44];
   float acc_s[10], acc_p[10];
   const bool ok_s = gks::gp_flux_global(P, vl, gl, vr, gr, n1, w, dt, acc_s);
-  auto right = [&](P2* vv, P2 (*gg)[3]) {
-    for (int k = 0; k < 5; ++k) {
-      vv[k] = P2(x[20 + k], y[20 + k]);
-      for (int a = 0; a < 3; ++a) gg[k][a] = P2(x[25 + 3 * k + a], y[25 + 3 * k + a]);
-    }
-  };
   bool ok_p;
-  if (gks::full_terms(P)) {
+  if (sides || gks::full_terms(P)) {
     ok_p = gks::gp_flux_sides(P, vl, gl, vr, gr, n1, w, dt, acc_p);
   } else {
-    ok_p = gks::gp_flux_pair(P, v, g, right, nn, P2(w), dt, acc2) & 1u;
-    for (int q = 0; q < 10; ++q) acc_p[q] = acc2[q].lo();
+    const int odd = i & 1, j = i - odd;
+    const float* a0 = in + 45 * (int64_t)j;
+    const float* a1 = in + 45 * (int64_t)(j + 1 < n ? j + 1 : 0);
+    auto at = [&](int k) { return P2(a0[k], a1[k]); };
+    auto side = [&](int k0, P2* v, P2 (*g)[3]) {
+      for (int k = 0; k < 5; ++k) {
+        v[k] = at(k0 + k);
+        for (int a = 0; a < 3; ++a) g[k][a] = at(k0 + 5 + 3 * k + a);
+      }
+    };
+    P2 v[5], g[5][3], acc2[10];
+    side(0, v, g);
+    const P2 nn[3] = {at(40), at(41), at(42)};
+    auto right = [&](P2* vv, P2 (*gg)[3]) { side(20, vv, gg); };
+    ok_p = gks::gp_flux_pair(P, v, g, right, nn, at(43), dt, acc2) >> odd & 1u;
+    for (int q = 0; q < 10; ++q) acc_p[q] = odd ? acc2[q].hi() : acc2[q].lo();
   }
   float* o = out + 21 * (int64_t)i;
   for (int q = 0; q < 10; ++q) {
@@ -254,11 +256,17 @@ __global__ void k_face_f32_pair(gks::FluxParams<float> P, int n, const float* __
 
 // The FP32 Gauss-point contribution on the GPU in the scalar and the packed f32x2
 // instantiation of the flux templates, for n points: in [n][45], out [n][21] (device
-// pointers, layout above), p the parameter vector of gks_gp_face_host. Synchronises the
-// device; 0 on success, 1 on a CUDA error.
-extern "C" int gks_gp_face_f32_pair(const double* p, int n, const float* in, float* out) {
+// pointers, layout above), p the parameter vector of gks_gp_face_host; the packed form of large
+// meshes, or with gks_gp_face_f32_sides the two sides of each point in either form. Synchronises
+// the device; 0 on success, 1 on a CUDA error.
+static int face_f32(const double* p, int n, int sides, const float* in, float* out) {
   if (n <= 0) return 0;
-  k_face_f32_pair<<<(n + 127) / 128, 128>>>(params_f32(p), n, in, out);
+  k_face_f32_pair<<<(n + 127) / 128, 128>>>(params_f32(p), n, sides, in, out);
   return cudaDeviceSynchronize() == cudaSuccess ? 0 : 1;
 }
-
+extern "C" int gks_gp_face_f32_pair(const double* p, int n, const float* in, float* out) {
+  return face_f32(p, n, 0, in, out);
+}
+extern "C" int gks_gp_face_f32_sides(const double* p, int n, const float* in, float* out) {
+  return face_f32(p, n, 1, in, out);
+}
