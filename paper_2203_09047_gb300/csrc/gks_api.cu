@@ -139,7 +139,6 @@ template <class R>
 KParams<R> kparams(const gks_params& p) {
   KParams<R> k;
   k.gamma = (R)p.gamma;
-  k.K = (R)((5.0 - 3.0 * p.gamma) / (p.gamma - 1.0));
   k.mu = (R)p.mu;
   k.tau_eps = (R)p.tau_eps;
   k.tau_C = (R)p.tau_C;
@@ -260,13 +259,11 @@ cudaError_t input_of(gks_solver* s, const double* p, double* stage, const double
   return cudaMemcpyAsync(stage, p, sizeof(double) * 5 * s->m.nc, cudaMemcpyDefault, s->st);
 }
 
-// Refresh the FP64 form of the state from its gather copy after steps.
+// Refresh the FP64 master state of the FP64-update mode from its gather copy (after implicit
+// steps, which leave the newer state there).
 void sync_q(gks_solver* s) {
   if (!s->q_stale) return;
-  if (s->mixed)
-    launch_unpack<float>(s->m.nc, (const float*)s->QA, s->Q, s->st);
-  else
-    launch_unpack<double>(s->m.nc, (const double*)s->QA, s->Q, s->st);
+  launch_unpack(s->m.nc, (const float*)s->QA, s->Q, s->st);
   s->q_stale = false;
 }
 

@@ -144,7 +144,7 @@ struct GeoR {
 // Parameters of the hot kernels.
 template <class R>
 struct KParams {
-  R gamma, K, mu, tau_eps, tau_C, pr_fix;
+  R gamma, mu, tau_eps, tau_C, pr_fix;
   int flux_mode, tau_model;
   R weno_gamma, weno_eps;
   int weno_pow;
@@ -186,7 +186,7 @@ template <class R>
 void launch_recon(const DevMesh& m, const GeoR<R>& g, const KParams<R>& p, const R* QA,
                   R* poly, int* flag, cudaStream_t st, const ForkJoin* fj = nullptr);
 // The table of half_erfc (gks_kinetic.cuh): a constant of 41 KB, computed on the host in extended
-// precision at the first use (1.3 ms).
+// precision at the first use (1.3 ms); every solver uploads it.
 const std::vector<double>& erfc_table();
 // Kernel launches of one launch_recon.
 int recon_launches(const DevMesh& m);
@@ -239,10 +239,9 @@ template <class R>
 void launch_jacobi_sweep(const DevMesh& m, const JacobiBuf<R>& b, const R* QA, int it, int last,
                          R* QAout, const KParams<R>& kp, int* flag, cudaStream_t st);
 
-// The state [5][nc] in FP64 (internal order) from its gather copy.
-template <class R>
-void launch_unpack(int64_t nc, const R* QA, double* Q, cudaStream_t st);
-// The same in caller order.
+// The state [5][nc] in FP64 (internal order) from its gather copy of float pairs.
+void launch_unpack(int64_t nc, const float* QA, double* Q, cudaStream_t st);
+// The same in caller order, from either gather copy.
 template <class R>
 void launch_unpack_out(int64_t nc, const int32_t* perm, const R* QA, double* dst, cudaStream_t st);
 // Caller order -> internal order (dst) and gather copy (gq), either may be null; flag != null

@@ -46,6 +46,5 @@ __host__ __device__ __forceinline__ ff ff_from(double x) {
   const float h = (float)x;
   return {h, (float)(x - (double)h)};
 }
-__device__ __forceinline__ double ff_to_double(ff x) { return (double)x.h + (double)x.l; }
 
 }  // namespace gks

@@ -24,7 +24,6 @@ __device__ __forceinline__ P2 relaxation(const P2& dt, const P2& tau) {
 __device__ __forceinline__ FluxParams<P2> pair_params(const FluxParams<float>& P) {
   FluxParams<P2> o;
   o.gamma = P2(P.gamma);
-  o.K = P2(P.K);
   o.mu = P2(P.mu);
   o.tau_eps = P2(P.tau_eps);
   o.tau_C = P2(P.tau_C);

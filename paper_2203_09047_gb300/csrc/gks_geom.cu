@@ -1,13 +1,45 @@
 // FP64 geometry precompute on the device: cell quadrature (27-point Gauss on the trilinear map,
 // Section 2), face Gauss data (2x2 Gauss on the bilinear map, Eq. flux-qud), and the
-// least-squares pseudo-inverses of the big stencils and sub-stencils (Section 2).
+// least-squares pseudo-inverses of the big stencils and sub-stencils (Section 2); and on the host
+// the table of erfc and exp of the FP64 flux.
 #include <cuda_runtime.h>
 
 #include <cmath>
 
 #include "gks_device.cuh"
+#include "gks_kinetic.cuh"
 
 namespace gks {
+namespace {
+
+// Taylor coefficients of erfc(z)/2 about z = i/64: c_0 = erfc(z)/2 and
+// c_(k+1) = -(-1)^k H_k(z) exp(-z^2) / (sqrt(pi) (k+1)!), H_k the Hermite polynomials.
+std::vector<double> make_erfc_table() {
+  typedef long double L;
+  std::vector<double> tab((size_t)kErfcTerms * kErfcRecords);
+  for (int i = 0; i < kErfcRecords; ++i) {
+    const L z = (L)(i - kErfcSteps * kErfcMax) / kErfcSteps;
+    double* c = tab.data() + (size_t)kErfcTerms * i;
+    c[0] = (double)(0.5L * erfcl(z));
+    const L d1 = -expl(-z * z) / sqrtl(acosl(-1.0L));
+    L hm = 0, h = 1, fact = 1;
+    for (int k = 0; k + 1 < kErfcTerms; ++k) {
+      fact *= k + 1;
+      c[k + 1] = (double)(d1 * ((k & 1) ? -h : h) / fact);
+      const L hn = 2 * z * h - 2 * k * hm;
+      hm = h;
+      h = hn;
+    }
+  }
+  return tab;
+}
+}  // namespace
+
+const std::vector<double>& erfc_table() {
+  static const std::vector<double> tab = make_erfc_table();
+  return tab;
+}
+
 namespace {
 
 constexpr int kThreads = 128;

@@ -2,7 +2,7 @@
 // the same templated arithmetic as the flux kernels. They let the kinetic formulas and their
 // hand-written adjoint be checked on a CPU (against the oracle and finite differences). One
 // device entry runs the FP32 Gauss-point flux in its scalar and its packed f32x2 instantiation
-// side by side, a direct test of the pair arithmetic.
+// side by side, a direct test of the pair arithmetic (the smooth form in both packings).
 #include <cmath>
 #include <cstdint>
 #include <vector>
@@ -13,40 +13,12 @@
 #include "gks_flux_f32x2.cuh"
 #include "gks_kinetic_adj.cuh"
 
-// Taylor coefficients of erfc(z)/2 about z = i/64: c_0 = erfc(z)/2 and
-// c_(k+1) = -(-1)^k H_k(z) exp(-z^2) / (sqrt(pi) (k+1)!), H_k the Hermite polynomials.
-static std::vector<double> make_erfc_table() {
-  using namespace gks;
-  typedef long double L;
-  std::vector<double> tab((size_t)kErfcTerms * kErfcRecords);
-  for (int i = 0; i < kErfcRecords; ++i) {
-    const L z = (L)(i - kErfcSteps * kErfcMax) / kErfcSteps;
-    double* c = tab.data() + (size_t)kErfcTerms * i;
-    c[0] = (double)(0.5L * erfcl(z));
-    const L d1 = -expl(-z * z) / sqrtl(acosl(-1.0L));
-    L hm = 0, h = 1, fact = 1;
-    for (int k = 0; k + 1 < kErfcTerms; ++k) {
-      fact *= k + 1;
-      c[k + 1] = (double)(d1 * ((k & 1) ? -h : h) / fact);
-      const L hn = 2 * z * h - 2 * k * hm;
-      hm = h;
-      h = hn;
-    }
-  }
-  return tab;
-}
-const std::vector<double>& gks::erfc_table() {
-  static const std::vector<double> tab = make_erfc_table();
-  return tab;
-}
-
 namespace {
 gks::FluxParams<double> params_from(const double* p) {
   // p = {gamma, mu, tau_eps, tau_C, flux_mode, tau_model, Pr, T_ref, mu_pow,
   //      wall_u[6][3], wall_T[6], farfield[6][5]}
   gks::FluxParams<double> P;
   P.gamma = p[0];
-  P.K = (5.0 - 3.0 * p[0]) / (p[0] - 1.0);
   P.mu = p[1];
   P.tau_eps = p[2];
   P.tau_C = p[3];
@@ -189,7 +161,6 @@ gks::FluxParams<float> params_f32(const double* p) {
   const gks::FluxParams<double> d = params_from(p);
   gks::FluxParams<float> P;
   P.gamma = (float)d.gamma;
-  P.K = (float)d.K;
   P.mu = (float)d.mu;
   P.tau_eps = (float)d.tau_eps;
   P.tau_C = (float)d.tau_C;

@@ -97,20 +97,6 @@ __device__ __forceinline__ double unpack_value(const Gq<float>& g, int v) {
 }
 __device__ __forceinline__ double unpack_value(const Gq<double>& g, int v) { return g.q[v]; }
 
-// dq[v] = Q_member - Q_0 for one stencil entry (cell | mirrored-axis bits).
-template <class R>
-__device__ __forceinline__ void stencil_delta(const R* __restrict__ QA, int32_t e, const Gq<R>& c0,
-                                              R dq[5]) {
-  Gq<R> g;
-  g.load(QA, e & kCellMask);
-  const int fl = e >> kFlipShift;
-  if (fl & 1) g.flip(1);
-  if (fl & 2) g.flip(2);
-  if (fl & 4) g.flip(3);
-#pragma unroll
-  for (int v = 0; v < 5; ++v) dq[v] = g.minus(c0, v);
-}
-
 // ------------------------------------------------------------------------------------------
 // Asynchronous bulk copies global -> shared completed on an mbarrier (transaction bytes), and a
 // bounded wait on it.
@@ -1644,11 +1630,10 @@ __global__ void __launch_bounds__(256) k_jacobi_sweep(
   }
 }
 
-template <class R>
-__global__ void k_unpack(int64_t nc, const R* __restrict__ QA, double* __restrict__ Q) {
+__global__ void k_unpack(int64_t nc, const float* __restrict__ QA, double* __restrict__ Q) {
   const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
   if (i >= nc) return;
-  Gq<R> g;
+  Gq<float> g;
   g.load(QA, i);
 #pragma unroll
   for (int v = 0; v < 5; ++v) Q[v * nc + i] = unpack_value(g, v);
@@ -2121,9 +2106,8 @@ void launch_jacobi_sweep(const DevMesh& m, const JacobiBuf<R>& b, const R* QA, i
                                               b.hrs, b.dQ[(it - 1) & 1], b.dQ[it & 1], QAout,
                                               flux_params(kp), wall_table<R>(m), flag);
 }
-template <class R>
-void launch_unpack(int64_t nc, const R* QA, double* Q, cudaStream_t st) {
-  k_unpack<R><<<blocks_for(nc, 256), 256, 0, st>>>(nc, QA, Q);
+void launch_unpack(int64_t nc, const float* QA, double* Q, cudaStream_t st) {
+  k_unpack<<<blocks_for(nc, 256), 256, 0, st>>>(nc, QA, Q);
 }
 template <class R>
 void launch_unpack_out(int64_t nc, const int32_t* perm, const R* QA, double* dst,
@@ -2187,7 +2171,6 @@ template void launch_stage<double>(const DevMesh&, const GeoR<double>&, const do
 template void launch_stage<float>(const DevMesh&, const GeoR<float>&, const float*, int, double,
                                   void*, void*, float*, float*, int*, cudaStream_t, double*,
                                   const double*);
-template void launch_unpack<double>(int64_t, const double*, double*, cudaStream_t);
 template void launch_jacobi_plan<double>(const DevMesh&, const double*, int32_t*, double*,
                                          cudaStream_t);
 template void launch_jacobi_plan<float>(const DevMesh&, const float*, int32_t*, float*,
@@ -2204,6 +2187,5 @@ template void launch_jacobi_sweep<double>(const DevMesh&, const JacobiBuf<double
 template void launch_jacobi_sweep<float>(const DevMesh&, const JacobiBuf<float>&, const float*,
                                          int, int, float*, const KParams<float>&, int*,
                                          cudaStream_t);
-template void launch_unpack<float>(int64_t, const float*, double*, cudaStream_t);
 
 }  // namespace gks

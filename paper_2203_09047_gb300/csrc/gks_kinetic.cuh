@@ -128,7 +128,7 @@ GKS_HD bool half_erfc(const double* tab, double z, double& f, double& d) {
 
 template <class R>
 struct FluxParams {
-  R gamma, K, mu, tau_eps, tau_C;
+  R gamma, mu, tau_eps, tau_C;
   int full, tau_model;
   R pr_fix = R(0);  // 1/Pr - 1 (heat-flux correction of the smooth flux; 0 for the BGK value)
   R T_ref = R(1), mu_pow = R(0.7);  // power law mu (T / T_ref)^mu_pow (collision time 3)
@@ -164,7 +164,6 @@ template <class R, template <class> class KP>
 inline FluxParams<R> flux_params(const KP<R>& p) {
   FluxParams<R> fp;
   fp.gamma = p.gamma;
-  fp.K = p.K;
   fp.mu = p.mu;
   fp.tau_eps = p.tau_eps;
   fp.tau_C = p.tau_C;

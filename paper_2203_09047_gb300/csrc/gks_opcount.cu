@@ -54,7 +54,6 @@ extern "C" int gks_flux_opcount(int flux_mode, int tau_model, double* flops, dou
   using opc::Op;
   FluxParams<Op> P;
   P.gamma = 1.4;
-  P.K = 2.0;
   P.mu = 1e-3;
   P.tau_eps = 0.01;
   P.tau_C = 1.0;
