@@ -992,7 +992,8 @@ __device__ __forceinline__ bool physical(const double q[5]) {
 // they take all faces of a cell at once (kFaceBatch; ten stage-pairs of the 8^3-cube mesh 582 ->
 // 465 us together with the merged reconstruction launch, 495 with two or five at a time); on
 // large ones occupancy is worth more (64^3 cubes, FP32: 66.5 us per stage one at a time, 70.0
-// with three), so kB = 1.
+// with three; FP64 update of 419,328 cells 46.2 us against 57.4 with six, of 1,048,576 cells 95.5
+// against 123, of 55,296 cells 15.2 either way), so kB = 1.
 constexpr int kFaceBatch = 6;
 template <int kQ0, int kB, class F>
 __device__ __forceinline__ void face_loop(int k0, int k1, const int32_t* __restrict__ cf_idx,
@@ -2053,7 +2054,8 @@ void launch_stage(const DevMesh& m, const GeoR<R>& g, const R* fface, int stage,
   constexpr int kB = kFaceBatch;
   if constexpr (std::is_same<R, float>::value) {
     if (Q64) {  // FP64 update of the FP64 master state
-      auto kern = stage == 1 ? k_stage_fd<false, kB> : k_stage_fd<true, kB>;
+      auto kern = stage == 1 ? (small ? k_stage_fd<false, kB> : k_stage_fd<false, 1>)
+                             : (small ? k_stage_fd<true, kB> : k_stage_fd<true, 1>);
       kern<<<nb, nt, 0, st>>>(m.nc, m.cf_ptr, m.cf_idx, fface, ivol64, c1, c2,
                               static_cast<double*>(L), static_cast<double*>(Lt), Q64, QA, QsA,
                               flag);
