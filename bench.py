@@ -490,8 +490,7 @@ def run_gpu(args):
 
     # DRAM bytes (read + write) per pass of the FP32 reconstruction and per launch of the FP32
     # smooth flux from the ncu captures on the 48^3-cube mesh with the enlarged stencils
-    # (profiles/k_recon_float_advection48_ncu.md, profiles/k_flux_float_smooth_advection48_ncu.md),
-    # scaled by cells and by faces (same layer pattern and stencils)
+    # (profiles/ncu_kernels.md), scaled by cells and by faces (same layer pattern and stencils)
     dram_per_unit = {"recon": (1506.2, nc), "flux": (292.6, nf)}
 
     def roof_of(table, dom, is_mixed):

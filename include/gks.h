@@ -252,8 +252,10 @@ gks_status gks_s2o4_stage_vjp(int64_t n, int stage, double dt, const double* g, 
  * solved by kmax >= 1 Jacobi iterations from dQ^(0) = |Omega_i| Res_i / D_i, and
  * Q^{n+1} = Q^n + dQ^(kmax). T_n is the Euler flux through the face (n out of cell i, S the
  * face area), r_f = max over both sides of |U . n| + c at Q^n; a wall face couples a cell to
- * its mirror image. The first call allocates the step's buffers (face normals, residual,
- * diagonal, two iterates). Errors: GKS_E_INVAL (dt <= 0, nsteps < 0, kmax < 1), GKS_E_NOMEM,
+ * its mirror image. The first call of a solver allocates the step's buffers (a plan of six face
+ * slots per cell of any kind, primitives, residual, diagonal, two iterates: 248 bytes per cell in
+ * the mixed precisions, 440 in FP64), lays out the plan, and cannot be captured in a graph; the
+ * buffers live until gks_destroy. Errors: GKS_E_INVAL (dt <= 0, nsteps < 0, kmax < 1), GKS_E_NOMEM,
  * GKS_E_CUDA; non-physical states are reported by gks_check. */
 gks_status gks_step_implicit(gks_solver* s, double dt, int nsteps, int kmax);
 

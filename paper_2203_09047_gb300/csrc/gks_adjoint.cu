@@ -217,9 +217,9 @@ __global__ void __launch_bounds__(256) k_vjp_poly(int64_t nc, const int32_t* __r
 // take over once the forward part is done; nothing is indexed in local memory. Bound by the FP64
 // pipe (about 770 FP64 instructions per thread and 18-member stencil). One thread per cell with
 // the differences, fits and cotangents in local arrays moved 4.1 GB per launch through them: 2.18
-// -> 1.44 ms at 131,072 cells, 478 -> 213 us at 16,384 cells (256 blocks of 64
-// threads left most of the GPU idle); at four blocks per SM (96 registers, some spills) a whole
-// VJP of 131,072 cells 11.09 -> 10.64 ms (two, three, five blocks 10.72, 10.68, 10.68).
+// -> 1.44 ms at 131,072 cells, 478 -> 213 us at 16,384 cells (256 blocks of 64 threads left most
+// of the GPU idle); then 1.33 ms at four blocks per SM (96 registers, some spills; a whole VJP of
+// 131,072 cells 11.09 -> 10.64 ms, with two, three and five blocks 10.72, 10.68, 10.68).
 constexpr int kVjpThreads = 5 * kTile;
 __global__ void __launch_bounds__(kVjpThreads, 4) k_vjp_recon(
     int64_t nc, const double* __restrict__ QA, const int32_t* __restrict__ t_K,

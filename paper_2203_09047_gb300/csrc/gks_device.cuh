@@ -49,7 +49,8 @@ enum : int {
 // Contiguous ranges of tiles whose first cell has the same kind (cells are ordered by kind
 // first, so there is one range per kind present). Each range records its largest stencil K, its
 // largest sum S of per-sub-stencil member counts and its largest number M of sub-stencil slots;
-// the reconstruction is launched once per range with shared memory sized for that range.
+// the reconstruction is launched once per range with shared memory sized for that range, on small
+// meshes once over all of them with the largest of each (launch_recon).
 constexpr int kMaxTileRanges = 8;
 struct TileRanges {
   int n = 0;

@@ -1485,10 +1485,11 @@ __global__ void __launch_bounds__(256) k_jacobi_prim(int64_t nc, const R* __rest
 
 // Both kernels below wait on the gathers of a cell's neighbours in FP32, and on the FP64 pipe in
 // FP64. The plan's coalesced entries, one record per cell for the iterate, and 1/rho, p and c per
-// cell in place of per face took an FP32 step's init and three sweeps from 69 to 58 us (131,072
-// cells), the FP64 one from 256 to 160 us (48,000 cells, where blocks of 256 threads, 188 of
-// them, left every second SM with twice the work of the others: 234 us). Requesting two, three or
-// six faces of a cell together was slower (66, 68, 89 us).
+// cell in place of per face took an FP32 step's init and three sweeps from 80 to 65 us (131,072
+// cells, median launches), the FP64 one with its primitives from 548 to 415 us (131,072 cells) and
+// from 258 to 163 us (48,000 cells, where blocks of 256 threads, 188 of them, left every second SM
+// with twice the work of the others: 234 us). Requesting two, three or six faces of a cell together
+// took 8, 10 and 31 us more (FP32).
 template <class R>
 __global__ void __launch_bounds__(256) k_jacobi_init(
     int64_t nc, const int32_t* __restrict__ cf_ptr, const int32_t* __restrict__ cf_idx,
